@@ -161,7 +161,8 @@ const char *nlse_last_error(void);
 
 /* Which stage kernel the context uses:
  *   0 = generic one-thread-per-site kernel,
- *   1 = tiled kernel (2D halo tiles / 3D z-marching; on 1D lines of up to
+ *   1 = tiled kernel (3D z-marching; 2D halo tiles, in the FP32 forms a tile's
+ *       four stages in one launch per step; on 1D lines of up to
  *       ~49,000 sites in FP64 or ~98,000 in FP32 (not NLSE_C64_ACC64) one
  *       thread-block cluster of up to 16 CTAs keeps the line in shared memory
  *       and runs every step of an nlse_step call in one launch; longer lines
@@ -197,7 +198,9 @@ const char *nlse_last_error(void);
  *       workspace inside each chunk (the chunk ends in Psi).  Other steps,
  *       dtypes and grids run as 1.  Same results as 1, bit for bit.
  * tile_cfg picks the tiled kernel's CTA tile (x-by-y threads): 0 = 32x8,
- * 1 = 64x4, 2 = 32x16, 3 = 64x8, -1 = default; it never changes results.
+ * 1 = 64x4, 2 = 32x16, 3 = 64x8, -1 = default (FP32 forms in 2D: 32 columns
+ * for 0 and 2, 64 for 1 and 3, strips of 2 rows per thread for 0 and 1, 4
+ * for 2 and 3, the rows from the grid's size); it never changes results.
  * Call between nlse_step calls, not during one. */
 int nlse_set_kernel(nlse_t ctx, int variant, int tile_cfg);
 
@@ -208,9 +211,9 @@ int nlse_kernel_in_use(nlse_t ctx);
 
 /*
  * Autotuner: time every tile shape of the context's tiled kernel on its own
- * buffers (stage 1 then repeated stage-2 launches; Psi is read, never
- * written) and keep the fastest for this context.  The choice is cached for
- * the process per (dims, shape, dtype, order, bc, variant, V present), and
+ * buffers (stage 1 then repeated stage-2 launches, or whole steps into the
+ * workspace where a step is one launch; Psi is read, never written) and keep
+ * the fastest for this context.  The choice is cached for the process per (dims, shape, dtype, order, bc, variant, V present), and
  * appended to the text file named by the environment variable
  * NLSE_TUNE_CACHE when it is set (later processes read it instead of
  * timing).  Synchronises the stream.  *best_tile_cfg receives the chosen

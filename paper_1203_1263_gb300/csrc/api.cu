@@ -345,6 +345,43 @@ cudaError_t launch_step_fused(const nlse_ctx* c, double dt, cudaStream_t st, voi
   return c->order == 4 ? launch_fused_step<4>(A, tm12, tm34, L, st) : launch_fused_step<2>(A, tm12, tm34, L, st);
 }
 
+// The FP32 forms' 2D grids on the whole-step kernel (the tiled variants).
+bool step2_path(const nlse_ctx* c) {
+  return c->d == 2 && c->dtype != NLSE_C128 && (c->variant == 1 || c->variant == 2 || c->variant == 4);
+}
+
+// Psi's ping-pong copy on that path: the stage arrays it does not use (K_tot; in the mixed form K_tot and
+// Psi_tmp, which lie one after the other, hold the FP64 master).
+void* step2_alt(const nlse_ctx* c) { return c->at(c->lay.ktot); }
+
+template <class T>
+cudaError_t launch_step2(const nlse_ctx* c, double dt, cudaStream_t st, const void* cur, void* nxt) {
+  const Field<T> f = make_field<T>(c, cur);
+  Step2Args<T> A;
+  memset(&A, 0, sizeof(A));
+  A.n[0] = f.n[0];
+  A.n[1] = f.n[1];
+  A.bc = f.bc;
+  A.s = f.s;
+  A.h2_over_a = f.h2_over_a;
+  A.cL = f.cL;
+  A.tiny = f.tiny;
+  const double dtc[4] = {dt / 2.0, dt / 2.0, dt, dt / 6.0};
+  for (int i = 0; i < 4; ++i) A.dtc[i] = typename T::R(dtc[i]);
+  A.V = f.V;
+  A.in = (const typename T::M*)cur;
+  A.out = (typename T::M*)nxt;
+  A.flag = c->flag();
+  return launch_step2d<T>(A, c->order, c->tile_cfg, st);
+}
+
+cudaError_t launch_step2_any(const nlse_ctx* c, double dt, cudaStream_t st, const void* cur, void* nxt) {
+  switch (c->dtype) {
+    case NLSE_C64: return launch_step2<P32>(c, dt, st, cur, nxt);
+    default: return launch_step2<PMix>(c, dt, st, cur, nxt);
+  }
+}
+
 // The exact-sum stencil's scale for the next step: from the exponent stage 4
 // collected (psi == nullptr) or from a full pass over psi.
 cudaError_t update_fix(const nlse_ctx* c, const void* psi, cudaStream_t st) {
@@ -392,9 +429,13 @@ int ensure_graph(nlse_ctx* c, double dt) {
   cudaError_t e = cudaStreamBeginCapture(c->cap, cudaStreamCaptureModeThreadLocal);
   if (e != cudaSuccess) return cuda_fail(e, "cudaStreamBeginCapture");
   cudaError_t le = cudaSuccess;
-  const bool fused = fused_path(c);
+  const bool fused = fused_path(c), step2 = step2_path(c);
   for (int i = 0; i < kGraphSteps && le == cudaSuccess; ++i) {
-    if (fused) {   // ping-pong: even steps Psi -> copy, odd steps copy -> Psi (kGraphSteps is even)
+    if (step2) {   // ping-pong as below
+      void* a = c->psi;
+      void* b = step2_alt(c);
+      le = (i % 2 == 0) ? launch_step2_any(c, dt, c->cap, a, b) : launch_step2_any(c, dt, c->cap, b, a);
+    } else if (fused) {   // ping-pong: even steps Psi -> copy, odd steps copy -> Psi (kGraphSteps is even)
       void* a = c->psi;
       void* b = c->at(c->lay.alt);
       le = (i % 2 == 0) ? launch_step_fused(c, dt, c->cap, a, b) : launch_step_fused(c, dt, c->cap, b, a);
@@ -632,7 +673,7 @@ int nlse_step(nlse_t c, int64_t nsteps, double dt) {
   if (dt > bound) return fail(NLSE_EUNSTABLE, "dt = %g above the RK4 linear stability bound %g", dt, bound);
   if (nsteps == 0) return NLSE_OK;
   cudaError_t e = cudaSuccess;
-  if (c->dtype == NLSE_C64_ACC64)
+  if (c->dtype == NLSE_C64_ACC64 && !step2_path(c))
     e = launch_round_master((const double2*)c->psi, (float2*)c->at(c->lay.pn32), c->total, c->stream);
   if (e != cudaSuccess) return cuda_fail(e, "round master");
   // the exact-sum scale of the state as the caller left it (stage 4 keeps it current from here on)
@@ -652,6 +693,17 @@ int nlse_step(nlse_t c, int64_t nsteps, double dt) {
       e = cudaGraphLaunch(c->exec, c->stream);
       if (e != cudaSuccess) return cuda_fail(e, "cudaGraphLaunch");
     }
+  }
+  if (step2_path(c)) {   // pairs of steps end in Psi; an odd step goes through the copy and back
+    void* alt = step2_alt(c);
+    for (; left > 0 && e == cudaSuccess; left -= 2) {
+      e = launch_step2_any(c, dt, c->stream, c->psi, alt);
+      if (e != cudaSuccess) break;
+      if (left > 1) e = launch_step2_any(c, dt, c->stream, alt, c->psi);
+      else e = cudaMemcpyAsync(c->psi, alt, (c->dtype == NLSE_C64 ? 8 : 16) * (size_t)c->total,
+                               cudaMemcpyDeviceToDevice, c->stream);
+    }
+    return e == cudaSuccess ? NLSE_OK : cuda_fail(e, "step launch");
   }
   for (; left > 0; --left) {
     e = launch_step_any(c, dt, c->stream);
@@ -796,10 +848,13 @@ int nlse_autotune(nlse_t c, int* best_tile_cfg, float* best_ms) {
     if (e == cudaSuccess && c->exact()) e = update_fix(c, c->psi, c->stream);
     for (int t = 0; t < 4 && e == cudaSuccess; ++t) {
       c->tile_cfg = t;
-      e = launch_stage_any(c, 1, 1e-12, c->stream);
-      if (e == cudaSuccess) e = launch_stage_any(c, 2, 1e-12, c->stream);
+      const bool step2 = step2_path(c);   // one whole step, into Psi's ping-pong copy
+      if (step2) e = launch_step2_any(c, 1e-12, c->stream, c->psi, step2_alt(c));
+      else e = launch_stage_any(c, 1, 1e-12, c->stream);
+      if (e == cudaSuccess && !step2) e = launch_stage_any(c, 2, 1e-12, c->stream);
       if (e == cudaSuccess) e = cudaEventRecord(e0, c->stream);
-      for (int r = 0; r < 3 && e == cudaSuccess; ++r) e = launch_stage_any(c, 2, 1e-12, c->stream);
+      for (int r = 0; r < 3 && e == cudaSuccess; ++r)
+        e = step2 ? launch_step2_any(c, 1e-12, c->stream, c->psi, step2_alt(c)) : launch_stage_any(c, 2, 1e-12, c->stream);
       if (e == cudaSuccess) e = cudaEventRecord(e1, c->stream);
       if (e == cudaSuccess) e = cudaEventSynchronize(e1);
       float ms = 0.f;

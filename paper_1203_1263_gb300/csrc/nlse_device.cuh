@@ -47,6 +47,12 @@ struct PMix { using R = float; using C = float2;  using VR = float;  using M = d
 struct E32 { using R = double; using C = float2;  using VR = float;  using M = float2;  };
 struct EMix { using R = double; using C = double2; using VR = float; using M = double2; };
 
+// A potential held in shared memory (the read-only global path below cannot read it), and the traits of
+// stages whose fields all live there.
+template <class R> struct OnChip { R v; };
+struct L64 { using R = double; using C = double2; using VR = OnChip<double>; using M = double2; };
+struct L32 { using R = float;  using C = float2;  using VR = OnChip<float>;  using M = float2;  };
+
 template <class R, class C>
 __device__ __forceinline__ typename V2<R>::t ld2(const C* __restrict__ p, int64_t i) {
   const C v = __ldg(p + i);
@@ -55,6 +61,10 @@ __device__ __forceinline__ typename V2<R>::t ld2(const C* __restrict__ p, int64_
 template <class R, class VR>
 __device__ __forceinline__ R ldv(const VR* __restrict__ V, int64_t i) {
   return V ? R(__ldg(V + i)) : R(0);
+}
+template <class R>
+__device__ __forceinline__ R ldv(const OnChip<R>* V, int64_t i) {
+  return V ? V[i].v : R(0);
 }
 
 // |z|^2 with one fixed rounding order, so every kernel computes it alike.
@@ -589,15 +599,14 @@ __device__ __forceinline__ unsigned int rk_update(const StageArgs<T>& A, int64_t
 // (c + sum_k o_k e_k with o_k in {0} u {-1 if idx==1} u {+1 if idx==n-2}, not
 // all 0), with F_b = 0 (Dirichlet), F_b = i Im(F_c / Psi_c) Psi_b (MSD) or
 // F_b = i N_b Psi_b (L0; in units of cLF on the exact-sum stages, like F_c).
-// Out of line: only sites next to a wall call it.
-// S: the RK4 stage when the caller's kernel is built for one (-1: A.stage at run time).
-template <class T, int D, bool EXACT, class Acc, int S = -1>
-__device__ __forceinline__ unsigned int serve_walls(const StageArgs<T>& A, const Acc& acc, const int* idx, int64_t c,
-                                                 typename V2<typename T::R>::t pc, typename V2<typename T::R>::t F,
-                                                 typename T::R m2w) {
+// Only sites next to a wall call it.
+// Vs: V in units of cLF (exact-sum stages); upd(o, b, F_b) updates boundary site b = c + sum_k o_k e_k.
+template <class T, int D, bool EXACT, class Acc, class Upd>
+__device__ __forceinline__ unsigned int serve_walls_with(const Field<T>& f, const typename T::VR* Vs, const Acc& acc,
+                                                         const int* idx, int64_t c, typename V2<typename T::R>::t pc,
+                                                         typename V2<typename T::R>::t F, typename T::R m2w, Upd&& upd) {
   using R = typename T::R;
   using C2 = typename V2<R>::t;
-  const Field<T>& f = A.f;
   R theta = R(0);
   unsigned int ex = 0;
   if (f.bc == BC_MSD) {
@@ -639,12 +648,50 @@ __device__ __forceinline__ unsigned int serve_walls(const StageArgs<T>& A, const
       Fb = {-theta * pb.y, theta * pb.x};
     } else if (f.bc == BC_L0) {
       const C2 pb = acc.atv(o);
-      const R Nb = fma(EXACT ? f.sG : f.s, norm2(pb), -ldv<R>(EXACT ? A.Vs : f.V, b));
+      const R Nb = fma(EXACT ? f.sG : f.s, norm2(pb), -ldv<R>(EXACT ? Vs : f.V, b));
       Fb = {-Nb * pb.y, Nb * pb.x};
     }
-    ex = max(ex, rk_update<T, S>(A, b, Fb));
+    ex = max(ex, upd(o, b, Fb));
   }
   return ex;
+}
+
+// S: the RK4 stage when the caller's kernel is built for one (-1: A.stage at run time).
+template <class T, int D, bool EXACT, class Acc, int S = -1>
+__device__ __forceinline__ unsigned int serve_walls(const StageArgs<T>& A, const Acc& acc, const int* idx, int64_t c,
+                                                    typename V2<typename T::R>::t pc, typename V2<typename T::R>::t F,
+                                                    typename T::R m2w) {
+  return serve_walls_with<T, D, EXACT>(A.f, A.Vs, acc, idx, c, pc, F, m2w,
+                                       [&](const int*, int64_t b, typename V2<typename T::R>::t Fb) {
+                                         return rk_update<T, S>(A, b, Fb);
+                                       });
+}
+
+// F at interior site c; v is V there (in units of cLF on the exact-sum stages, and so is F).  Also Psi_c and,
+// on the exact-sum stages, |Psi_c|^2 of an MSD wall-adjacent site (0 below the guard), for its ghosts and theta.
+template <class T, int D, int ORDER, bool EXACT, class Acc>
+__device__ __forceinline__ typename V2<typename T::R>::t site_rhs(const Field<T>& f, const Acc& acc, const int* idx,
+                                                                  int64_t c, typename T::R v,
+                                                                  typename V2<typename T::R>::t* pc_out,
+                                                                  typename T::R* m2w_out) {
+  using R = typename T::R;
+  using C2 = typename V2<R>::t;
+  const C2 pc = acc.at0();
+  // exact-sum stages work in units of cLF: Nc / cLF (v holds V / cLF there)
+  const R Nc = fma(EXACT ? f.sG : f.s, norm2(pc), -v);
+  R m2w = R(0);
+  if constexpr (EXACT) {
+    if (f.bc == BC_MSD && near_wall2<D>(idx, f.n)) {
+      const R m2 = norm2(pc);
+      m2w = (m2 > f.tiny) ? m2 : R(0);
+    }
+  }
+  C2 aL;
+  if constexpr (EXACT) aL = a_lap_exact<T, D, ORDER>(f, acc, idx, c, pc, Nc, m2w);
+  else aL = a_lap<T, D, ORDER>(f, acc, idx, c, pc, Nc);
+  *pc_out = pc;
+  *m2w_out = m2w;
+  return {-fma(Nc, pc.y, aL.y), fma(Nc, pc.x, aL.x)};
 }
 
 // The full per-site work: F at interior site c, its update, and the update of
@@ -656,20 +703,9 @@ __device__ __forceinline__ unsigned int process_site_pv(const StageArgs<T>& A, c
   using R = typename T::R;
   using C2 = typename V2<R>::t;
   const Field<T>& f = A.f;
-  const C2 pc = acc.at0();
-  // exact-sum stages work in units of cLF: Nc / cLF (p.v holds V / cLF there)
-  const R Nc = fma(EXACT ? f.sG : f.s, norm2(pc), -p.v);
-  R m2w = R(0);
-  if constexpr (EXACT) {   // |Psi_c|^2 of an MSD wall-adjacent site (0 below the guard), for its ghosts and theta
-    if (f.bc == BC_MSD && near_wall2<D>(idx, f.n)) {
-      const R m2 = norm2(pc);
-      m2w = (m2 > f.tiny) ? m2 : R(0);
-    }
-  }
-  C2 aL;
-  if constexpr (EXACT) aL = a_lap_exact<T, D, ORDER>(f, acc, idx, c, pc, Nc, m2w);
-  else aL = a_lap<T, D, ORDER>(f, acc, idx, c, pc, Nc);
-  const C2 F = {-fma(Nc, pc.y, aL.y), fma(Nc, pc.x, aL.x)};
+  C2 pc;
+  R m2w;
+  const C2 F = site_rhs<T, D, ORDER, EXACT>(f, acc, idx, c, p.v, &pc, &m2w);
   unsigned int ex = rk_apply<T, S>(A, c, F, p);
 
   bool near = false;

@@ -4,10 +4,34 @@
 #include <stdint.h>
 
 #include "nlse_device.cuh"
+#include "stage_step2d.cuh"
 
 namespace nlse {
 
 constexpr int kMaxReduceBlocks = 1024;
+
+// A kernel that may start while the kernel before it in the stream still runs (programmatic dependent
+// launch): it calls grid_wait() before it touches anything an earlier kernel wrote or still reads, and
+// grid_launch_dependents() where the next kernel may start.  On a dependency that is not such a kernel
+// this is an ordinary launch.
+__device__ __forceinline__ void grid_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void grid_launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+
+template <class... P, class... Q>
+inline cudaError_t launch_early(void (*kern)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t stream,
+                                Q&&... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = block;
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = stream;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, kern, static_cast<P>(args)...);
+}
 
 // CTA tile (x-by-y threads) of the tiled 3D/2D kernels for tile_cfg 0..3.
 inline void tma_tile_shape(int tile_cfg, int* tx, int* ty) {
@@ -28,6 +52,10 @@ cudaError_t launch_fused_step(const StageArgs<P32>* A, const void* tm12, const v
 bool fused_grid_ok(int d, const int* n);
 // the fused kernel's TMA box: 64 + 8 complex values by 8 + 8 rows
 constexpr int kFusedBoxX = 2 * (64 + 8), kFusedBoxY = 8 + 8;
+
+// One RK4 step of a 2D grid in one launch, Psi^n in A.in to Psi^{n+1} in A.out (stage_step2d.cuh).
+template <class T>
+cudaError_t launch_step2d(const Step2Args<T>& A, int order, int tile_cfg, cudaStream_t stream);
 
 // 1D lines on one thread-block cluster (stage_line1d.cuh): nsteps RK4 steps of
 // an n-site line in one launch; A[0..3] are stages 1..4 with Psi updated in
