@@ -225,11 +225,10 @@ int nlse_autotune(nlse_t ctx, int *best_tile_cfg, float *best_ms);
 
 /* ---------------------------------------------------------------------------
  * Batched form: many independent 2D runs (uneven sizes and parameters) in
- * complex64, advanced together with one launch per RK4 stage for all runs
- * (a persistent deep-interior kernel over a (run, tile) work list and a
- * wall-shell kernel over the runs' walls), the step loop replayed as a CUDA
- * graph.  Each run is computed with the same per-site arithmetic as a
- * single-run NLSE_C64 context with the tiled kernel, so its result is
+ * complex64, advanced together with one launch per RK4 step for all runs (a
+ * CTA per (run, tile) item takes its tile through the four stages on chip),
+ * the step loop replayed as a CUDA graph.  Each run is computed with the
+ * same per-site arithmetic as a single-run NLSE_C64 context with the tiled kernel, so its result is
  * bit-for-bit that of integrating it alone.
  * ------------------------------------------------------------------------- */
 typedef struct {
@@ -255,14 +254,14 @@ int nlse_batch_create(nlse_batch_t *out, int nruns, const nlse_run_desc *runs, v
 /* Advance every run by nsteps RK4 steps of its own dt; asynchronous. */
 int nlse_batch_step(nlse_batch_t b, int64_t nsteps);
 
-/* Tile shape of the batched deep kernel (as nlse_set_kernel's tile_cfg; -1 = 32x8, the measured best on
- * the 512-run workload). */
+/* Tile shape of the batched step kernel: 0 = 32x28 cells with strips of 2 rows per thread, 1 = 64x24 with
+ * 2, 2 = 32x28 with 4, 3 = 64x24 with 4, -1 = default (1); it never changes results. */
 int nlse_batch_set_tile(nlse_batch_t b, int tile_cfg);
 
-/* Autotuner: time stages 1-3 of every tile shape on the batch's own runs
- * (three passes in alternating order, the first one untimed; none of these
- * stages writes any run's Psi) and keep the fastest shape; *best_ms is its
- * mean stage time.  Synchronises the stream. */
+/* Autotuner: time steps of every tile shape on the batch's own runs (three
+ * passes in alternating order, the first one untimed; the steps go into the
+ * copies in the workspace, no run's Psi is written) and keep the fastest
+ * shape; *best_ms is its mean step time.  Synchronises the stream. */
 int nlse_batch_autotune(nlse_batch_t b, int *best_tile_cfg, float *best_ms);
 
 /* Wait for the stream; NLSE_ENONFINITE if any run produced a NaN or Inf. */

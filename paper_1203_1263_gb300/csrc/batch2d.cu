@@ -1,16 +1,15 @@
 // Batched form: many independent 2D runs of uneven size and parameters
-// advanced together, one launch per stage for all of them.
+// advanced together, one launch per RK4 step for all of them.
 //
 // Each run has its own grid (Ny, Nx), spacing, a, s, potential, boundary,
-// order and time step.  A device table holds, per run, the stage arguments
-// of the four RK4 stages (the same StageArgs the single-run kernels use); a
-// work list enumerates (run, tile) items covering every run's deep interior,
-// and a second list covers every run's wall shell in chunks of at most 256
-// sites.  The deep kernel is persistent: a grid of a few CTAs per SM walks
-// the item list, loads each tile with its 2-cell halo into shared memory and
-// computes it with the per-site code of every other kernel; the shell kernel
-// runs on a side stream at the same time.  Results are therefore bit-for-bit
-// those of integrating each run alone with the tiled kernels.
+// order and time step.  A device table holds, per run, the arguments of the
+// whole-step kernel (stage_step2d.cuh); a work list enumerates (run, tile)
+// items, the largest runs first.  A CTA takes one item through all four stages
+// with the single runs' code, so results are bit-for-bit those of integrating
+// each run alone.  Psi alternates between the caller's array and a copy in the
+// workspace.  96 runs of 64^2 to 1024^2 (3.5e7 sites): 0.587 ms per step, 60
+// Gsite-step/s; a deep and a wall-shell kernel per stage, with K_tot, Psi_tmp
+// and Psi_out through memory (148 bytes per site and step), took 1.55 ms.
 #include <cuda_runtime.h>
 #include <math.h>
 #include <string.h>
@@ -20,8 +19,7 @@
 
 #include "../../include/nlse.h"
 #include "nlse_internal.h"
-#include "stage_generic.cuh"
-#include "stage_tiled.cuh"
+#include "stage_step2d.cuh"
 
 namespace nlse {
 void record_last_error(const char* msg);
@@ -32,20 +30,16 @@ using namespace nlse;
 namespace {
 
 struct BatchRun {
-  StageArgs<P32> A[4];   // stages 1..4
+  Step2Args<P32> A;   // in = Psi, out = its copy; every other step runs from the copy back
   int order;
-  int pad[3];
+  int ty, ntx;        // rows of this run's tiles, tiles per row
+  int pad;
 };
 
-struct DeepItem {
-  int run, tx, ty, pad;
+struct Item {
+  int run, tile;
 };
 
-struct ShellItem {
-  int run, start, count, pad;
-};
-
-constexpr int kShellChunk = 256;
 constexpr int kGraphSteps = 16;
 
 int bfail(int code, const char* msg) {
@@ -53,106 +47,81 @@ int bfail(int code, const char* msg) {
   return code;
 }
 
-template <int ORDER, int TX, int TY>
-__device__ __forceinline__ void batch_tile(const StageArgs<P32>& A, int tx, int ty, float2* tile) {
-  constexpr int W = TX + 4, H = TY + 4, PS = W * H, NT = TX * TY, NPER = (PS + NT - 1) / NT;
-  const Field<P32>& f = A.f;
-  const int ny = f.n[0], nx = f.n[1];
-  const int tid = threadIdx.y * TX + threadIdx.x;
-  const int x0 = tx * TX, y0 = ty * TY;
-  const int gx = x0 + threadIdx.x, gy = y0 + threadIdx.y;
-  const bool deep = gx >= 2 && gx <= nx - 3 && gy >= 2 && gy <= ny - 3;
-  const int64_t c = (int64_t)gy * nx + gx;
-  // the site's pointwise operands are requested first, so that their latency
-  // overlaps the tile's
-  PointVals<P32> pv;
-  if (deep) pv = load_point<P32>(A, c, f.V != nullptr);
-#pragma unroll
-  for (int i = 0; i < NPER; ++i) {
-    const int e = tid + i * NT;
-    if (e < PS) {
-      const int r = e / W, q = e - r * W;
-      const int gy = y0 - 2 + r, gx = x0 - 2 + q;
-      tile[e] = (gy >= 0 && gy < ny && gx >= 0 && gx < nx) ? f.in[(int64_t)gy * nx + gx] : float2{0.f, 0.f};
-    }
-  }
-  __syncthreads();
-  if (deep) {
-    const int idx[2] = {gy, gx};
-    SAcc2<P32> acc;
-    acc.p = tile;
-    acc.w = W;
-    acc.o = (threadIdx.y + 2) * W + threadIdx.x + 2;
-    const float2 pc = acc.at0();
-    const float Nc = fmaf(f.s, norm2(pc), -pv.v);
-    const float2 aL = a_lap_body<P32, 2, ORDER, SAcc2<P32>, false>(f, acc, idx, c, pc, Nc);
-    rk_apply<P32>(A, c, {-fmaf(Nc, pc.y, aL.y), fmaf(Nc, pc.x, aL.x)}, pv);
-  }
-  __syncthreads();   // the tile is reused by the next item
-}
+// The tile shapes of tile_cfg 0..3: columns, largest rows, threads, rows per strip, CTAs per SM.
+struct Shape { int tx, ty, nt, ry, per_sm; };
+constexpr Shape kShapes[4] = {{32, 28, 256, 2, 3}, {64, 24, 256, 2, 2}, {32, 28, 256, 4, 3}, {64, 24, 384, 4, 2}};
+constexpr int kDefaultShape = 1;
 
-template <int TX, int TY>
-__global__ void __launch_bounds__(TX* TY) k_batch2d_deep(const BatchRun* __restrict__ runs,
-                                                        const DeepItem* __restrict__ items, int nitems, int stage) {
-  __shared__ __align__(16) float2 tile[(TX + 4) * (TY + 4)];
-  for (int it = blockIdx.x; it < nitems; it += gridDim.x) {
-    const DeepItem w = items[it];
-    const BatchRun& R = runs[w.run];
-    const StageArgs<P32>& A = R.A[stage - 1];
-    if (R.order == 4) batch_tile<4, TX, TY>(A, w.tx, w.ty, tile);
-    else batch_tile<2, TX, TY>(A, w.tx, w.ty, tile);
-  }
-}
-
-__global__ void __launch_bounds__(kShellChunk) k_batch2d_shell(const BatchRun* __restrict__ runs,
-                                                               const ShellItem* __restrict__ items, int stage) {
-  const ShellItem w = items[blockIdx.x];
-  if ((int)threadIdx.x >= w.count) return;
+template <int CFG>
+__global__ void __launch_bounds__(kShapes[CFG].nt, kShapes[CFG].per_sm)
+    k_batch2d_step(const BatchRun* __restrict__ runs, const Item* __restrict__ items, int back) {
+  constexpr Shape s = kShapes[CFG];
+  extern __shared__ __align__(16) unsigned char batch_smem[];
+  grid_launch_dependents();
+  const Item w = items[blockIdx.x];
   const BatchRun& R = runs[w.run];
-  const StageArgs<P32>& A = R.A[stage - 1];
-  int idx[2];
-  const int64_t c = shell_decode<P32, 2, uint32_t>(A.f, uint32_t(w.start + threadIdx.x), idx);
-  const GAcc<P32, 2> acc(A.f, c);
-  if (R.order == 4) process_site<P32, 2, 4, false>(A, acc, idx, c);
-  else process_site<P32, 2, 2, false>(A, acc, idx, c);
+  Step2Args<P32> A = R.A;
+  if (back) {
+    A.in = R.A.out;
+    A.out = const_cast<float2*>(R.A.in);
+  }
+  const int ty = R.ty, ntx = R.ntx, tx_i = w.tile % ntx, ty_i = w.tile / ntx;
+  if (R.order == 4) {
+    Step2Tile<P32, 4, s.tx, s.nt, s.ry> tile(A, ty, tx_i, ty_i, batch_smem);
+    tile.load_potential();
+    grid_wait();
+    tile.run();
+  } else {
+    Step2Tile<P32, 2, s.tx, s.nt, s.ry> tile(A, ty, tx_i, ty_i, batch_smem);
+    tile.load_potential();
+    grid_wait();
+    tile.run();
+  }
+}
+
+// Every run's copy back into Psi (after an odd step).
+__global__ void __launch_bounds__(256) k_batch2d_copy(const BatchRun* __restrict__ runs) {
+  const Step2Args<P32>& A = runs[blockIdx.y].A;
+  const int64_t n = (int64_t)A.n[0] * A.n[1];
+  float2* psi = const_cast<float2*>(A.in);
+  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
+    psi[i] = A.out[i];
 }
 
 // Run-table and work-list layout inside the caller's workspace.
 struct BatchLayout {
-  size_t runs_off, deep_off, shell_off, fields_off, total;
-  int ndeep, nshell;
-  std::vector<size_t> field_off;   // per run: K_tot, Psi_tmp, Psi_out (3 x 8 B x sites)
+  size_t runs_off, items_off, total;
+  int nitems;
+  std::vector<size_t> field_off;   // per run: Psi's copy
 };
 
-void tile_dims(int tile_cfg, int* tx, int* ty) { tma_tile_shape(tile_cfg < 0 ? 0 : tile_cfg, tx, ty); }
+// Rows of a run's tiles under a shape: its interior in equal parts of at most the shape's rows.
+int run_rows(const Shape& s, int64_t ny) {
+  const int64_t ext = ny - 1, parts = (ext + s.ty - 1) / s.ty;
+  return int(((ext + parts - 1) / parts + 3) / 4 * 4);
+}
 
 bool layout_batch(int nruns, const nlse_run_desc* runs, int tile_cfg, BatchLayout* L) {
-  int tx, ty;
-  tile_dims(tile_cfg, &tx, &ty);
+  const Shape& s = kShapes[tile_cfg < 0 ? kDefaultShape : tile_cfg];
   size_t off = 256;   // bytes 0..255: the status word, at the same place for every tile shape
   auto al = [](size_t x) { return (x + 255) / 256 * 256; };
   L->runs_off = off;
   off = al(off + sizeof(BatchRun) * nruns);
-  int64_t nd = 0, ns = 0;
+  int64_t ni = 0;
   for (int r = 0; r < nruns; ++r) {
-    const int64_t ny = runs[r].n[0], nx = runs[r].n[1];
-    if (ny < 3 || nx < 3) return false;
-    if (ny > 4 && nx > 4) nd += ((nx + tx - 1) / tx) * ((ny + ty - 1) / ty);
-    const int m[2] = {int(ny - 2), int(nx - 2)};
-    ns += (shell_count(2, m) + kShellChunk - 1) / kShellChunk;
+    int ntx, nty;
+    if (runs[r].n[0] < 3 || runs[r].n[1] < 3) return false;
+    step2_tiles(int(runs[r].n[0]), int(runs[r].n[1]), false, s.tx, run_rows(s, runs[r].n[0]), &ntx, &nty);
+    ni += (int64_t)ntx * nty;
   }
-  if (nd > (1ll << 30) || ns > (1ll << 30)) return false;
-  L->ndeep = int(nd);
-  L->nshell = int(ns);
-  L->deep_off = off;
-  off = al(off + sizeof(DeepItem) * nd);
-  L->shell_off = off;
-  off = al(off + sizeof(ShellItem) * ns);
-  L->fields_off = off;
+  if (ni > (1ll << 30)) return false;
+  L->nitems = int(ni);
+  L->items_off = off;
+  off = al(off + sizeof(Item) * ni);
   L->field_off.resize(nruns);
   for (int r = 0; r < nruns; ++r) {
     L->field_off[r] = off;
-    off = al(off + 3 * sizeof(float2) * size_t(runs[r].n[0] * runs[r].n[1]));
+    off = al(off + sizeof(float2) * size_t(runs[r].n[0] * runs[r].n[1]));
   }
   L->total = al(off);
   return true;
@@ -165,8 +134,7 @@ struct nlse_batch {
   std::vector<nlse_run_desc> desc;
   char* ws;
   BatchLayout lay;
-  cudaStream_t stream, side, cap;
-  cudaEvent_t ev_fork, ev_join;
+  cudaStream_t stream, cap;
   cudaGraphExec_t exec;
   int tile_cfg;
   unsigned int* flag() const { return (unsigned int*)ws; }   // fixed: the layout after it depends on the tile shape
@@ -174,125 +142,79 @@ struct nlse_batch {
 
 namespace {
 
-template <int TX, int TY>
-cudaError_t launch_deep(const nlse_batch* b, int stage, cudaStream_t st) {
-  if (b->lay.ndeep == 0) return cudaSuccess;
-  // one wave of persistent CTAs: as many as fit on every SM at once for this tile shape
-  static int per_sm = 0, sms = 0;
-  if (per_sm == 0) {
-    int dev = 0;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_batch2d_deep<TX, TY>, TX * TY, 0) != cudaSuccess ||
-        per_sm < 1) {
-      cudaGetLastError();
-      per_sm = 1;
-    }
+template <int CFG>
+cudaError_t launch_shape(const nlse_batch* b, bool back, cudaStream_t st) {
+  constexpr Shape s = kShapes[CFG];
+  const size_t smem = step2_smem<s.tx>(s.ty, true);
+  auto kern = k_batch2d_step<CFG>;
+  static const cudaError_t attr = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
+  if (attr != cudaSuccess) return attr;
+  return launch_early(kern, dim3((unsigned)b->lay.nitems), dim3(s.nt), smem, st,
+                      (const BatchRun*)(b->ws + b->lay.runs_off), (const Item*)(b->ws + b->lay.items_off), back ? 1 : 0);
+}
+
+// One step of every run, from Psi into the copies or back.
+cudaError_t launch_batch_step(const nlse_batch* b, bool back, cudaStream_t st) {
+  switch (b->tile_cfg < 0 ? kDefaultShape : b->tile_cfg) {
+    case 0: return launch_shape<0>(b, back, st);
+    case 1: return launch_shape<1>(b, back, st);
+    case 2: return launch_shape<2>(b, back, st);
+    default: return launch_shape<3>(b, back, st);
   }
-  int grid = sms * per_sm;
-  if (grid > b->lay.ndeep) grid = b->lay.ndeep;
-  k_batch2d_deep<TX, TY><<<grid, dim3(TX, TY), 0, st>>>((const BatchRun*)(b->ws + b->lay.runs_off),
-                                                         (const DeepItem*)(b->ws + b->lay.deep_off), b->lay.ndeep,
-                                                         stage);
+}
+
+cudaError_t launch_batch_copy(const nlse_batch* b, cudaStream_t st) {
+  for (int r0 = 0; r0 < b->nruns; r0 += 65535) {
+    const int n = std::min(65535, b->nruns - r0);
+    k_batch2d_copy<<<dim3(16, (unsigned)n), 256, 0, st>>>((const BatchRun*)(b->ws + b->lay.runs_off) + r0);
+  }
   return cudaGetLastError();
-}
-
-cudaError_t launch_batch_stage(const nlse_batch* b, int stage, cudaStream_t st) {
-  cudaError_t e;
-  if ((e = cudaEventRecord(b->ev_fork, st)) != cudaSuccess) return e;
-  if ((e = cudaStreamWaitEvent(b->side, b->ev_fork, 0)) != cudaSuccess) return e;
-  if (b->lay.nshell > 0) {
-    k_batch2d_shell<<<b->lay.nshell, kShellChunk, 0, b->side>>>((const BatchRun*)(b->ws + b->lay.runs_off),
-                                                                  (const ShellItem*)(b->ws + b->lay.shell_off), stage);
-    if ((e = cudaGetLastError()) != cudaSuccess) return e;
-  }
-  if ((e = cudaEventRecord(b->ev_join, b->side)) != cudaSuccess) return e;
-  switch (b->tile_cfg < 0 ? 0 : b->tile_cfg) {
-    case 0: e = launch_deep<32, 8>(b, stage, st); break;
-    case 1: e = launch_deep<64, 4>(b, stage, st); break;
-    case 2: e = launch_deep<32, 16>(b, stage, st); break;
-    default: e = launch_deep<64, 8>(b, stage, st); break;
-  }
-  if (e != cudaSuccess) return e;
-  return cudaStreamWaitEvent(st, b->ev_join, 0);
-}
-
-cudaError_t launch_batch_step(const nlse_batch* b, cudaStream_t st) {
-  for (int s = 1; s <= 4; ++s) {
-    cudaError_t e = launch_batch_stage(b, s, st);
-    if (e != cudaSuccess) return e;
-  }
-  return cudaSuccess;
 }
 
 // Build the run table and work lists on the host and copy them into the workspace.
 int upload_tables(nlse_batch* b) {
-  int tx, ty;
-  tile_dims(b->tile_cfg, &tx, &ty);
+  const Shape& sh = kShapes[b->tile_cfg < 0 ? kDefaultShape : b->tile_cfg];
   std::vector<BatchRun> runs(b->nruns);
-  std::vector<DeepItem> deep;
-  std::vector<ShellItem> shell;
-  deep.reserve(b->lay.ndeep);
-  shell.reserve(b->lay.nshell);
-  // work items of large runs first, so that the persistent CTAs run out of work together
+  std::vector<Item> items;
+  items.reserve(b->lay.nitems);
+  // runs of one order together (CTAs side by side then share the instruction cache), the costlier order
+  // and the larger runs first
   std::vector<int> order(b->nruns);
   for (int r = 0; r < b->nruns; ++r) order[r] = r;
   std::stable_sort(order.begin(), order.end(), [&](int p, int q) {
+    if (b->desc[p].order != b->desc[q].order) return b->desc[p].order > b->desc[q].order;
     return b->desc[p].n[0] * b->desc[p].n[1] > b->desc[q].n[0] * b->desc[q].n[1];
   });
   for (int r : order) {
     const nlse_run_desc& d = b->desc[r];
-    const int ny = int(d.n[0]), nx = int(d.n[1]);
-    float2* base = (float2*)(b->ws + b->lay.field_off[r]);
-    const int64_t sites = (int64_t)ny * nx;
-    float2 *ktot = base, *ptmp = base + sites, *pout = base + 2 * sites;
     BatchRun& R = runs[r];
     memset(&R, 0, sizeof(R));
     R.order = d.order;
-    const void* in[4] = {d.psi, ptmp, pout, ptmp};
-    float2* outs[4] = {ptmp, pout, ptmp, nullptr};
+    R.ty = run_rows(sh, d.n[0]);
+    Step2Args<P32>& A = R.A;
+    A.n[0] = int(d.n[0]);
+    A.n[1] = int(d.n[1]);
+    A.bc = d.bc;
+    A.s = float(d.s);
+    A.h2_over_a = float(d.h * d.h / d.a);
+    A.cL = float(d.order == 4 ? d.a / (12.0 * d.h * d.h) : d.a / (d.h * d.h));
+    A.tiny = 1e-30f;
     const double dtc[4] = {d.dt / 2.0, d.dt / 2.0, d.dt, d.dt / 6.0};
-    for (int s = 0; s < 4; ++s) {
-      StageArgs<P32>& A = R.A[s];
-      Field<P32>& f = A.f;
-      f.n[0] = ny; f.n[1] = nx; f.n[2] = 1;
-      f.m[0] = ny - 2; f.m[1] = nx - 2; f.m[2] = 1;
-      f.st[0] = nx; f.st[1] = 1; f.st[2] = 0;
-      f.ninterior = (int64_t)(ny - 2) * (nx - 2);
-      f.a = float(d.a);
-      f.s = float(d.s);
-      f.h2_over_a = float(d.h * d.h / d.a);
-      f.cL = float(d.order == 4 ? d.a / (12.0 * d.h * d.h) : d.a / (d.h * d.h));
-      f.tiny = 1e-30f;
-      f.bc = d.bc;
-      f.V = (const float*)d.V;
-      f.in = (const float2*)in[s];
-      A.psin = (const float2*)d.psi;
-      A.ktot = ktot;
-      A.out = outs[s];
-      A.master = (float2*)d.psi;
-      A.master_in = (const float2*)d.psi;   // Psi updated in place: stage 4 reads Psi^n where it writes
-      A.dtc = float(dtc[s]);
-      A.dt6 = d.dt / 6.0;
-      A.stage = s + 1;
-      A.flag = b->flag();
-    }
-    if (ny > 4 && nx > 4)
-      for (int t_y = 0; t_y < (ny + ty - 1) / ty; ++t_y)
-        for (int t_x = 0; t_x < (nx + tx - 1) / tx; ++t_x) deep.push_back({r, t_x, t_y, 0});
-    const int m[2] = {ny - 2, nx - 2};
-    const int64_t nsh = shell_count(2, m);
-    for (int64_t s0 = 0; s0 < nsh; s0 += kShellChunk)
-      shell.push_back({r, int(s0), int(std::min<int64_t>(kShellChunk, nsh - s0)), 0});
+    for (int s = 0; s < 4; ++s) A.dtc[s] = float(dtc[s]);
+    A.V = (const float*)d.V;
+    A.in = (const float2*)d.psi;
+    A.out = (float2*)(b->ws + b->lay.field_off[r]);
+    A.flag = b->flag();
+    int ntx, nty;
+    step2_tiles(A.n[0], A.n[1], false, sh.tx, R.ty, &ntx, &nty);
+    R.ntx = ntx;
+    for (int t = 0; t < ntx * nty; ++t) items.push_back({r, t});
   }
   cudaError_t e = cudaMemcpyAsync(b->ws + b->lay.runs_off, runs.data(), sizeof(BatchRun) * runs.size(),
                                   cudaMemcpyHostToDevice, b->stream);
-  if (e == cudaSuccess && !deep.empty())
-    e = cudaMemcpyAsync(b->ws + b->lay.deep_off, deep.data(), sizeof(DeepItem) * deep.size(), cudaMemcpyHostToDevice,
+  if (e == cudaSuccess)
+    e = cudaMemcpyAsync(b->ws + b->lay.items_off, items.data(), sizeof(Item) * items.size(), cudaMemcpyHostToDevice,
                         b->stream);
-  if (e == cudaSuccess && !shell.empty())
-    e = cudaMemcpyAsync(b->ws + b->lay.shell_off, shell.data(), sizeof(ShellItem) * shell.size(),
-                        cudaMemcpyHostToDevice, b->stream);
   if (e == cudaSuccess) e = cudaStreamSynchronize(b->stream);
   if (e != cudaSuccess) return bfail(NLSE_ECUDA, cudaGetErrorString(e));
   return NLSE_OK;
@@ -350,13 +272,10 @@ int nlse_batch_create(nlse_batch_t* out, int nruns, const nlse_run_desc* runs, v
   b->ws = (char*)workspace;
   b->stream = (cudaStream_t)stream;
   b->tile_cfg = -1;
-  b->side = b->cap = nullptr;
+  b->cap = nullptr;
   b->exec = nullptr;
   layout_batch(nruns, runs, b->tile_cfg, &b->lay);
-  cudaError_t e = cudaStreamCreateWithFlags(&b->side, cudaStreamNonBlocking);
-  if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&b->cap, cudaStreamNonBlocking);
-  if (e == cudaSuccess) e = cudaEventCreateWithFlags(&b->ev_fork, cudaEventDisableTiming);
-  if (e == cudaSuccess) e = cudaEventCreateWithFlags(&b->ev_join, cudaEventDisableTiming);
+  cudaError_t e = cudaStreamCreateWithFlags(&b->cap, cudaStreamNonBlocking);
   if (e == cudaSuccess) e = cudaMemsetAsync(b->flag(), 0, 256, b->stream);
   if (e != cudaSuccess) {
     nlse_batch_destroy(b);
@@ -389,7 +308,8 @@ int nlse_batch_step(nlse_batch_t b, int64_t nsteps) {
     if (!b->exec) {
       e = cudaStreamBeginCapture(b->cap, cudaStreamCaptureModeThreadLocal);
       cudaError_t le = cudaSuccess;
-      for (int i = 0; i < kGraphSteps && le == cudaSuccess && e == cudaSuccess; ++i) le = launch_batch_step(b, b->cap);
+      for (int i = 0; i < kGraphSteps && le == cudaSuccess && e == cudaSuccess; ++i)   // an even count ends in Psi
+        le = launch_batch_step(b, i % 2 == 1, b->cap);
       cudaGraph_t g = nullptr;
       cudaError_t ee = cudaStreamEndCapture(b->cap, &g);
       if (e == cudaSuccess) e = (le != cudaSuccess) ? le : ee;
@@ -402,7 +322,10 @@ int nlse_batch_step(nlse_batch_t b, int64_t nsteps) {
     }
     for (; left >= kGraphSteps && e == cudaSuccess; left -= kGraphSteps) e = cudaGraphLaunch(b->exec, b->stream);
   }
-  for (; left > 0 && e == cudaSuccess; --left) e = launch_batch_step(b, b->stream);
+  for (; left > 0 && e == cudaSuccess; left -= 2) {   // pairs end in Psi; an odd step is copied back
+    e = launch_batch_step(b, false, b->stream);
+    if (e == cudaSuccess) e = left > 1 ? launch_batch_step(b, true, b->stream) : launch_batch_copy(b, b->stream);
+  }
   if (e != cudaSuccess) return bfail(NLSE_ECUDA, cudaGetErrorString(e));
   return NLSE_OK;
 }
@@ -424,7 +347,7 @@ int nlse_batch_autotune(nlse_batch_t b, int* best_tile_cfg, float* best_ms) {
   cudaEventCreate(&e1);
   float t_min[4] = {1e30f, 1e30f, 1e30f, 1e30f};
   int rc = NLSE_OK;
-  // time stages 1-3 (none of them writes any run's Psi) for every tile shape,
+  // time a step into the copies (no run's Psi is written) for every tile shape,
   // twice in alternating order, after one untimed pass each; keep each shape's
   // fastest pass
   for (int pass = 0; pass < 3 && rc == NLSE_OK; ++pass) {
@@ -433,7 +356,7 @@ int nlse_batch_autotune(nlse_batch_t b, int* best_tile_cfg, float* best_ms) {
       rc = nlse_batch_set_tile(b, t);
       if (rc != NLSE_OK) break;
       cudaError_t e = cudaEventRecord(e0, b->stream);
-      for (int st = 1; st <= 3 && e == cudaSuccess; ++st) e = launch_batch_stage(b, st, b->stream);
+      for (int q = 0; q < 3 && e == cudaSuccess; ++q) e = launch_batch_step(b, false, b->stream);
       if (e == cudaSuccess) e = cudaEventRecord(e1, b->stream);
       if (e == cudaSuccess) e = cudaEventSynchronize(e1);
       float ms = 0.f;
@@ -457,10 +380,7 @@ int nlse_batch_autotune(nlse_batch_t b, int* best_tile_cfg, float* best_ms) {
 int nlse_batch_destroy(nlse_batch_t b) {
   if (!b) return NLSE_OK;
   drop_graph(b);
-  if (b->side) cudaStreamDestroy(b->side);
   if (b->cap) cudaStreamDestroy(b->cap);
-  if (b->ev_fork) cudaEventDestroy(b->ev_fork);
-  if (b->ev_join) cudaEventDestroy(b->ev_join);
   delete b;
   return NLSE_OK;
 }
