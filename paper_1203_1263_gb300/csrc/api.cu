@@ -128,6 +128,7 @@ struct nlse_ctx {
   int* fdev() const { return (int*)(ws + lay.status + 16); }                    // current fraction bits
   unsigned int* emax() const { return (unsigned int*)(ws + lay.status + 20); }  // stage-4 largest exponent
   bool exact() const { return dtype == NLSE_C128 && variant >= 2 && variant <= 3; }
+  unsigned int* done() const { return (unsigned int*)(ws + lay.status + 32); }  // blocks of a reduction that are through
   double* result() const { return (double*)(ws + lay.status + 64); }
   double* partials() const { return (double*)(ws + lay.partials); }
 };
@@ -462,11 +463,15 @@ __global__ void k_round_master(const double2* __restrict__ m, float2* __restrict
   }
 }
 
-int read_status(nlse_ctx* c) {
-  unsigned int flag = 0;
-  cudaError_t e = cudaMemcpyAsync(&flag, c->flag(), sizeof(flag), cudaMemcpyDeviceToHost, c->stream);
+// Wait for the stream, with *value (if given) the reduction's result: it lies beside the status word, one copy.
+int read_status(nlse_ctx* c, double* value = nullptr) {
+  unsigned char words[72];
+  cudaError_t e = cudaMemcpyAsync(words, c->flag(), value ? 72 : 4, cudaMemcpyDeviceToHost, c->stream);
   if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
   if (e != cudaSuccess) return cuda_fail(e, "status read");
+  unsigned int flag = 0;
+  memcpy(&flag, words, sizeof(flag));
+  if (value) memcpy(value, words + 64, sizeof(double));
   if (flag & kFlagTimeoutBit) {
     // Report once and clear every status bit: nothing a timed-out step wrote
     // is valid (a non-finite value it produced included); the caller restores
@@ -739,11 +744,10 @@ int nlse_rhs(nlse_t c, const void* psi_in, void* F_out) {
 int nlse_mass(nlse_t c, double* out_host) {
   if (!c || !out_host) return fail(NLSE_EINVAL, "NULL argument");
   cudaError_t e = launch_mass(c->psi, c->dtype != NLSE_C64, c->total, pow(c->h, c->d), c->partials(), c->result(),
-                              c->flag(), c->stream);
+                              c->flag(), c->done(), c->stream);
   double v = 0.0;
-  if (e == cudaSuccess) e = cudaMemcpyAsync(&v, c->result(), sizeof(double), cudaMemcpyDeviceToHost, c->stream);
   if (e != cudaSuccess) return cuda_fail(e, "mass");
-  int rc = read_status(c);
+  int rc = read_status(c, &v);
   if (rc != NLSE_OK) return rc;
   *out_host = v;
   return NLSE_OK;
@@ -757,21 +761,20 @@ int nlse_energy(nlse_t c, double* out_host) {
     using T = decltype(tag);
     Field<T> f = make_field<T>(c, c->psi);
     switch (c->d * 10 + c->order) {
-      case 12: return launch_energy<T, 1, 2>(f, scale, c->partials(), c->result(), c->flag(), c->stream);
-      case 14: return launch_energy<T, 1, 4>(f, scale, c->partials(), c->result(), c->flag(), c->stream);
-      case 22: return launch_energy<T, 2, 2>(f, scale, c->partials(), c->result(), c->flag(), c->stream);
-      case 24: return launch_energy<T, 2, 4>(f, scale, c->partials(), c->result(), c->flag(), c->stream);
-      case 32: return launch_energy<T, 3, 2>(f, scale, c->partials(), c->result(), c->flag(), c->stream);
-      default: return launch_energy<T, 3, 4>(f, scale, c->partials(), c->result(), c->flag(), c->stream);
+      case 12: return launch_energy<T, 1, 2>(f, scale, c->partials(), c->result(), c->flag(), c->done(), c->stream);
+      case 14: return launch_energy<T, 1, 4>(f, scale, c->partials(), c->result(), c->flag(), c->done(), c->stream);
+      case 22: return launch_energy<T, 2, 2>(f, scale, c->partials(), c->result(), c->flag(), c->done(), c->stream);
+      case 24: return launch_energy<T, 2, 4>(f, scale, c->partials(), c->result(), c->flag(), c->done(), c->stream);
+      case 32: return launch_energy<T, 3, 2>(f, scale, c->partials(), c->result(), c->flag(), c->done(), c->stream);
+      default: return launch_energy<T, 3, 4>(f, scale, c->partials(), c->result(), c->flag(), c->done(), c->stream);
     }
   };
   if (c->dtype == NLSE_C128) e = run(P64{});
   else if (c->dtype == NLSE_C64) e = run(E32{});
   else e = run(EMix{});
   double v = 0.0;
-  if (e == cudaSuccess) e = cudaMemcpyAsync(&v, c->result(), sizeof(double), cudaMemcpyDeviceToHost, c->stream);
   if (e != cudaSuccess) return cuda_fail(e, "energy");
-  int rc = read_status(c);
+  int rc = read_status(c, &v);
   if (rc != NLSE_OK) return rc;
   *out_host = v;
   return NLSE_OK;

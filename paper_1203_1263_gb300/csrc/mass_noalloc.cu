@@ -12,9 +12,9 @@
 // every GPU that loads the library keeps until the process exits.
 //
 // The kernels are a variant of the context's mass reduction: each block sums a
-// fixed run of sites with Neumaier's compensated summation, writes one
-// (sum, compensation) pair into the scratch array, and a one-block second pass
-// adds the pairs in a fixed order.
+// fixed run of sites exactly (wide_sum.cuh), writes one (sum, compensation)
+// pair into the scratch array, and a one-block second pass adds the pairs in a
+// fixed order.
 #include <cuda_runtime.h>
 #include <math.h>
 #include <stdarg.h>
@@ -24,6 +24,7 @@
 #include <mutex>
 
 #include "../../include/nlse.h"
+#include "wide_sum.cuh"
 
 namespace nlse {
 void record_last_error(const char* msg);   // api.cu
@@ -55,69 +56,66 @@ int fail(int code, const char* fmt, ...) {
   return code;
 }
 
-struct Pair {
-  double s, c;
-};
-
-__device__ __forceinline__ void nadd(Pair& a, double x) {
-  const double t = a.s + x;
-  if (fabs(a.s) >= fabs(x)) a.c += (a.s - t) + x;
-  else a.c += (x - t) + a.s;
-  a.s = t;
+__device__ __forceinline__ bool add_norm2(nlse::WideSum& w, double2 v) {
+  const double x = fma(v.x, v.x, v.y * v.y);
+  const bool ok = isfinite(x);
+  if (ok) w.add(x);
+  return ok;
+}
+__device__ __forceinline__ bool add_norm2(nlse::WideSum& w, float2 v) {
+  const bool ok = isfinite(v.x) && isfinite(v.y);
+  if (ok) {
+    w.add_square(v.x);
+    w.add_square(v.y);
+  }
+  return ok;
 }
 
-__device__ __forceinline__ Pair block_sum(Pair v) {
-  __shared__ double ss[kThreads / 32], sc[kThreads / 32];
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    const double s = __shfl_down_sync(0xffffffffu, v.s, o), c = __shfl_down_sync(0xffffffffu, v.c, o);
-    nadd(v, s);
-    v.c += c;
-  }
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  if (lane == 0) { ss[warp] = v.s; sc[warp] = v.c; }
-  __syncthreads();
-  if (warp == 0) {
-    v = (lane < kThreads / 32) ? Pair{ss[lane], sc[lane]} : Pair{0.0, 0.0};
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-      const double s = __shfl_down_sync(0xffffffffu, v.s, o), c = __shfl_down_sync(0xffffffffu, v.c, o);
-      nadd(v, s);
-      v.c += c;
-    }
-  }
-  return v;
-}
-
+// A thread's 16 sites are loaded together and added exactly on the integer pipe.
 template <class C>
 __global__ void __launch_bounds__(kThreads) k_mass_noalloc_blocks(const C* __restrict__ psi, int64_t total,
                                                                   double* scratch) {
-  Pair acc = {0.0, 0.0};
-  const int64_t base = (int64_t)blockIdx.x * kSitesPerBlock;
-  for (int i = threadIdx.x; i < kSitesPerBlock; i += kThreads) {
-    const int64_t p = base + i;
-    if (p < total) {
-      const C v = psi[p];
-      const double x = double(v.x), y = double(v.y);
-      nadd(acc, fma(x, x, y * y));
+  constexpr int U = 8;
+  nlse::WideSum w;
+  bool ok = true;
+  const int64_t base = (int64_t)blockIdx.x * kSitesPerBlock + threadIdx.x;
+#pragma unroll
+  for (int i0 = 0; i0 < kSitesPerBlock / kThreads; i0 += U) {
+    C v[U];
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      const int64_t p = base + (int64_t)(i0 + u) * kThreads;
+      v[u] = p < total ? psi[p] : C{0, 0};
     }
+#pragma unroll
+    for (int u = 0; u < U; ++u) ok &= add_norm2(w, v[u]);
   }
-  acc = block_sum(acc);
+  ok = __syncthreads_and(ok);
+  w = nlse::block_wide_sum<kThreads>(w);
   if (threadIdx.x == 0) {
-    scratch[2 * blockIdx.x] = acc.s;
-    scratch[2 * blockIdx.x + 1] = acc.c;
+    double s, c;
+    w.pair(&s, &c);
+    scratch[2 * blockIdx.x] = ok ? s : __longlong_as_double(0x7FF8000000000000ll);   // a NaN or Inf in psi shows
+    scratch[2 * blockIdx.x + 1] = c;
   }
 }
 
 __global__ void __launch_bounds__(kThreads) k_mass_noalloc_finish(const double* scratch, int nb, double scale,
                                                                   double* out) {
-  Pair acc = {0.0, 0.0};
-  for (int i = threadIdx.x; i < nb; i += kThreads) {
-    nadd(acc, scratch[2 * i]);
-    acc.c += scratch[2 * i + 1];
+  nlse::WideSum w;
+  bool ok = true;
+  for (int i = threadIdx.x; i < 2 * nb; i += kThreads) {
+    const double x = scratch[i];
+    if (isfinite(x)) w.add(x);
+    else ok = false;
   }
-  acc = block_sum(acc);
-  if (threadIdx.x == 0) out[0] = scale * (acc.s + acc.c);
+  ok = __syncthreads_and(ok);
+  w = nlse::block_wide_sum<kThreads>(w);
+  if (threadIdx.x == 0) {
+    double s, c;
+    w.pair(&s, &c);
+    out[0] = ok ? scale * (s + c) : __longlong_as_double(0x7FF8000000000000ll);
+  }
 }
 
 // Device address of the scratch array on the current device (set up once per

@@ -53,14 +53,35 @@ template <class R> struct OnChip { R v; };
 struct L64 { using R = double; using C = double2; using VR = OnChip<double>; using M = double2; };
 struct L32 { using R = float;  using C = float2;  using VR = OnChip<float>;  using M = float2;  };
 
+// float <-> double on the integer pipe (GB300 issues FP64-pipe instructions,
+// conversions included, at 1/75 of the FP32 rate).  Both follow IEEE-754:
+// widening is exact, narrowing rounds to nearest even; zeros, subnormals,
+// infinities and NaN take the hardware conversion.
+__device__ __forceinline__ double f2d_exact(float v) {
+  const unsigned int u = __float_as_uint(v);
+  const unsigned int e = (u >> 23) & 0xFFu;
+  if (e == 0u || e == 0xFFu) return double(v);
+  const unsigned long long bits = ((unsigned long long)(u & 0x80000000u) << 32) |
+                                  ((unsigned long long)(e - 127u + 1023u) << 52) |
+                                  ((unsigned long long)(u & 0x7FFFFFu) << 29);
+  return __longlong_as_double((long long)bits);
+}
+
+// A stored value in arithmetic type R.
+template <class R, class S>
+__device__ __forceinline__ R widen(S v) {
+  if constexpr (std::is_same<R, double>::value && std::is_same<S, float>::value) return f2d_exact(v);
+  else return R(v);
+}
+
 template <class R, class C>
 __device__ __forceinline__ typename V2<R>::t ld2(const C* __restrict__ p, int64_t i) {
   const C v = __ldg(p + i);
-  return {R(v.x), R(v.y)};
+  return {widen<R>(v.x), widen<R>(v.y)};
 }
 template <class R, class VR>
 __device__ __forceinline__ R ldv(const VR* __restrict__ V, int64_t i) {
-  return V ? R(__ldg(V + i)) : R(0);
+  return V ? widen<R>(__ldg(V + i)) : R(0);
 }
 template <class R>
 __device__ __forceinline__ R ldv(const OnChip<R>* V, int64_t i) {
@@ -491,20 +512,6 @@ struct StageArgs {
   int xwall;                   // 3D tiled path: the shell also owns x in [2, 1 + xwall] and its mirror
                                // (deep-interior kernels start at x = 2 + xwall); 0 by default
 };
-
-// float <-> double on the integer pipe (GB300 issues FP64-pipe instructions,
-// conversions included, at 1/75 of the FP32 rate).  Both follow IEEE-754:
-// widening is exact, narrowing rounds to nearest even; zeros, subnormals,
-// infinities and NaN take the hardware conversion.
-__device__ __forceinline__ double f2d_exact(float v) {
-  const unsigned int u = __float_as_uint(v);
-  const unsigned int e = (u >> 23) & 0xFFu;
-  if (e == 0u || e == 0xFFu) return double(v);
-  const unsigned long long bits = ((unsigned long long)(u & 0x80000000u) << 32) |
-                                  ((unsigned long long)(e - 127u + 1023u) << 52) |
-                                  ((unsigned long long)(u & 0x7FFFFFu) << 29);
-  return __longlong_as_double((long long)bits);
-}
 
 __device__ __forceinline__ float d2f_rn(double v) {
   const unsigned long long u = (unsigned long long)__double_as_longlong(v);

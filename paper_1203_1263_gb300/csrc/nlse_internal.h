@@ -67,10 +67,10 @@ cudaError_t launch_line_steps(const StageArgs<T>* A, int64_t nsteps, int n, int 
                               int fix_offset, cudaStream_t stream);
 
 cudaError_t launch_mass(const void* psi, bool psi_double, int64_t total, double scale, double* partials,
-                        double* result, unsigned int* flag, cudaStream_t stream);
+                        double* result, unsigned int* flag, unsigned int* done, cudaStream_t stream);
 template <class T, int D, int ORDER>
 cudaError_t launch_energy(const Field<T>& f, double scale, double* partials, double* result, unsigned int* flag,
-                          cudaStream_t stream);
+                          unsigned int* done, cudaStream_t stream);
 cudaError_t launch_vmax(const void* V, bool v_double, int64_t total, unsigned long long* out, cudaStream_t stream);
 // Exact-sum scale: with psi (complex128, n = 2 x sites components) first the
 // largest exponent of psi into *emax, then *fdev = the fraction bits for it
