@@ -162,23 +162,25 @@ const char *nlse_last_error(void);
 /* Which stage kernel the context uses:
  *   0 = generic one-thread-per-site kernel,
  *   1 = tiled kernel (3D z-marching; 2D halo tiles, in the FP32 forms a tile's
- *       four stages in one launch per step; on 1D lines of up to
- *       ~49,000 sites in FP64 or ~98,000 in FP32 (not NLSE_C64_ACC64) one
- *       thread-block cluster of up to 16 CTAs keeps the line in shared memory
- *       and runs every step of an nlse_step call in one launch; longer lines
- *       and the mixed form use the generic kernel),
+ *       four stages in one launch per step; 1D: several steps per launch, FP64
+ *       lines of up to ~49,000 sites, FP32 stages at any length; longer FP64
+ *       lines use the generic kernel),
  *   2 = tiled kernel with the exact-sum stencil (NLSE_C128 only; other
  *       dtypes treat it as 1): the Laplacian's stencil sums are formed exactly
- *       in 64-bit fixed point on the integer pipe and converted to FP64 once,
+ *       in 64-bit fixed point on the integer pipe and converted to FP64 once;
+ *       on 1D lines of up to ~49,000 sites one thread-block cluster of up to 16
+ *       CTAs keeps the line in shared memory and runs every step of an
+ *       nlse_step call in one launch,
  *   3 = generic kernel with the exact-sum stencil (NLSE_C128; else as 0).
  * Variants 0 and 1 give bit-for-bit the same result, and so do 2 and 3.
  * Default: 2 for NLSE_C128 and 1 otherwise, except on grids small enough
  * that a step is bound by latency rather than by throughput: 3D grids of at
  * most 2^15 sites (NLSE_C128) or 2^17 sites (the FP32 forms) take 0,
  * NLSE_C128 2D grids of at most 80,000 sites take 1, and NLSE_C128 1D lines
- * take 1 (the cluster path) up to 2500 sites, 0 up to 2^15 sites and 3
- * beyond (the plain FP64 stencil's instruction chain is shorter than the
- * exact-sum stencil's conversions; a cluster's 16 SMs bound longer lines).
+ * take 1 up to 2500 sites, 0 up to 2^15 sites and 3 beyond (the plain FP64
+ * stencil's instruction chain is shorter than the exact-sum stencil's
+ * conversions).  Where 0 is such a line's default rather than the caller's
+ * choice, its steps run several per launch as with 1 (the same arithmetic).
  * The exact-sum stencil's fixed-point scale follows the state: before every
  * step it is taken from the largest component of Psi (every component
  * below 2^53 in fixed point, 4x below the accepted range, so the largest

@@ -105,6 +105,7 @@ struct nlse_ctx {
   int fixF;          // reference fraction bits F0 of the exact-sum stencil (FP64 path): cLF = cL 2^-F0
   int fix_offset;    // test hook added to the derived fraction bits (nlse_debug_set)
   int variant, tile_cfg;
+  bool chosen;       // the caller chose the variant (nlse_set_kernel)
   cudaStream_t cap;
   cudaGraphExec_t exec;
   double graph_dt;
@@ -318,22 +319,72 @@ LaunchCfg launch_cfg(const nlse_ctx* c) {
   return L;
 }
 
-// 1D lines that take the cluster path: FP64 or FP32 (not the mixed form), variant 1, 2 or 4.
+// 1D lines that take the cluster path: FP64 with the exact-sum stencil (variant 2).
 bool line_path(const nlse_ctx* c) {
-  if (c->d != 1 || c->line_failed || c->dtype == NLSE_C64_ACC64) return false;
-  if (c->variant != 1 && c->variant != 2 && c->variant != 4) return false;
-  return line_ok(int(c->n[0]), c->dtype == NLSE_C128);
+  return c->d == 1 && !c->line_failed && c->dtype == NLSE_C128 && c->variant == 2 && line_ok(int(c->n[0]), true);
+}
+
+// 1D lines that run several steps per launch: variant 1 (and what runs as it) with the FP64 stencil up to the
+// length the cluster path has, with FP32 stages at any length; and FP64 lines whose default is one thread per site
+// with the FP64 stencil (variant 0: the same arithmetic).
+bool lines_path(const nlse_ctx* c) {
+  if (c->d != 1) return false;
+  if (c->dtype == NLSE_C128) {
+    if (c->variant == 0) return !c->chosen;
+    return (c->variant == 1 || c->variant == 4) && line_ok(int(c->n[0]), true);
+  }
+  return c->variant == 1 || c->variant == 2 || c->variant == 4;
 }
 
 cudaError_t launch_line(const nlse_ctx* c, int64_t nsteps, double dt) {
-  if (c->dtype == NLSE_C128) {
-    StageArgs<P64> A[4];
-    for (int s = 1; s <= 4; ++s) A[s - 1] = stage_args<P64>(c, s, dt, c->psi, c->psi);
-    return launch_line_steps<P64>(A, nsteps, int(c->n[0]), c->order, c->exact(), c->fixF, c->fix_offset, c->stream);
+  StageArgs<P64> A[4];
+  for (int s = 1; s <= 4; ++s) A[s - 1] = stage_args<P64>(c, s, dt, c->psi, c->psi);
+  return launch_line_steps(A, nsteps, int(c->n[0]), c->order, c->fixF, c->fix_offset, c->stream);
+}
+
+// Psi's ping-pong copy on the whole-step paths: the stage arrays they do not use (K_tot; in the mixed form K_tot
+// and Psi_tmp, which lie one after the other, hold the FP64 master).
+void* step_alt(const nlse_ctx* c) { return c->at(c->lay.ktot); }
+
+// The arguments that the 1D and 2D whole-step kernels share.
+template <class T, class A>
+A step_args(const nlse_ctx* c, double dt, const void* cur, void* nxt) {
+  const Field<T> f = make_field<T>(c, cur);
+  A a;
+  memset(&a, 0, sizeof(a));
+  a.bc = f.bc;
+  a.s = f.s;
+  a.h2_over_a = f.h2_over_a;
+  a.cL = f.cL;
+  a.tiny = f.tiny;
+  const double dtc[4] = {dt / 2.0, dt / 2.0, dt, dt / 6.0};
+  for (int i = 0; i < 4; ++i) a.dtc[i] = typename T::R(dtc[i]);
+  a.V = f.V;
+  a.in = (const typename T::M*)cur;
+  a.out = (typename T::M*)nxt;
+  a.flag = c->flag();
+  return a;
+}
+
+int steps_per_launch(const nlse_ctx* c) {
+  const int n = int(c->n[0]);
+  return c->dtype == NLSE_C128 ? steps1d_per_launch<P64>(n)
+                               : (c->dtype == NLSE_C64 ? steps1d_per_launch<P32>(n) : steps1d_per_launch<PMix>(n));
+}
+
+template <class T>
+cudaError_t launch_steps1(const nlse_ctx* c, double dt, int steps, cudaStream_t st, const void* cur, void* nxt) {
+  Step1Args<T> A = step_args<T, Step1Args<T>>(c, dt, cur, nxt);
+  A.n = int(c->n[0]);
+  return launch_steps1d<T>(A, c->order, steps, st);
+}
+
+cudaError_t launch_steps1_any(const nlse_ctx* c, double dt, int steps, cudaStream_t st, const void* cur, void* nxt) {
+  switch (c->dtype) {
+    case NLSE_C128: return launch_steps1<P64>(c, dt, steps, st, cur, nxt);
+    case NLSE_C64: return launch_steps1<P32>(c, dt, steps, st, cur, nxt);
+    default: return launch_steps1<PMix>(c, dt, steps, st, cur, nxt);
   }
-  StageArgs<P32> A[4];
-  for (int s = 1; s <= 4; ++s) A[s - 1] = stage_args<P32>(c, s, dt, c->psi, c->psi);
-  return launch_line_steps<P32>(A, nsteps, int(c->n[0]), c->order, false, c->fixF, c->fix_offset, c->stream);
 }
 
 // One step of the fused path from buffer cur to buffer nxt (Psi or its ping-pong copy).
@@ -351,28 +402,11 @@ bool step2_path(const nlse_ctx* c) {
   return c->d == 2 && c->dtype != NLSE_C128 && (c->variant == 1 || c->variant == 2 || c->variant == 4);
 }
 
-// Psi's ping-pong copy on that path: the stage arrays it does not use (K_tot; in the mixed form K_tot and
-// Psi_tmp, which lie one after the other, hold the FP64 master).
-void* step2_alt(const nlse_ctx* c) { return c->at(c->lay.ktot); }
-
 template <class T>
 cudaError_t launch_step2(const nlse_ctx* c, double dt, cudaStream_t st, const void* cur, void* nxt) {
-  const Field<T> f = make_field<T>(c, cur);
-  Step2Args<T> A;
-  memset(&A, 0, sizeof(A));
-  A.n[0] = f.n[0];
-  A.n[1] = f.n[1];
-  A.bc = f.bc;
-  A.s = f.s;
-  A.h2_over_a = f.h2_over_a;
-  A.cL = f.cL;
-  A.tiny = f.tiny;
-  const double dtc[4] = {dt / 2.0, dt / 2.0, dt, dt / 6.0};
-  for (int i = 0; i < 4; ++i) A.dtc[i] = typename T::R(dtc[i]);
-  A.V = f.V;
-  A.in = (const typename T::M*)cur;
-  A.out = (typename T::M*)nxt;
-  A.flag = c->flag();
+  Step2Args<T> A = step_args<T, Step2Args<T>>(c, dt, cur, nxt);
+  A.n[0] = int(c->n[0]);
+  A.n[1] = int(c->n[1]);
   return launch_step2d<T>(A, c->order, c->tile_cfg, st);
 }
 
@@ -430,11 +464,16 @@ int ensure_graph(nlse_ctx* c, double dt) {
   cudaError_t e = cudaStreamBeginCapture(c->cap, cudaStreamCaptureModeThreadLocal);
   if (e != cudaSuccess) return cuda_fail(e, "cudaStreamBeginCapture");
   cudaError_t le = cudaSuccess;
-  const bool fused = fused_path(c), step2 = step2_path(c);
-  for (int i = 0; i < kGraphSteps && le == cudaSuccess; ++i) {
-    if (step2) {   // ping-pong as below
+  const bool fused = fused_path(c), step2 = step2_path(c), lines = lines_path(c);
+  const int per = lines ? steps_per_launch(c) : 1;   // divides kGraphSteps an even number of times
+  for (int i = 0; i < kGraphSteps / per && le == cudaSuccess; ++i) {
+    if (lines) {   // ping-pong as below
       void* a = c->psi;
-      void* b = step2_alt(c);
+      void* b = step_alt(c);
+      le = (i % 2 == 0) ? launch_steps1_any(c, dt, per, c->cap, a, b) : launch_steps1_any(c, dt, per, c->cap, b, a);
+    } else if (step2) {
+      void* a = c->psi;
+      void* b = step_alt(c);
       le = (i % 2 == 0) ? launch_step2_any(c, dt, c->cap, a, b) : launch_step2_any(c, dt, c->cap, b, a);
     } else if (fused) {   // ping-pong: even steps Psi -> copy, odd steps copy -> Psi (kGraphSteps is even)
       void* a = c->psi;
@@ -569,10 +608,9 @@ int nlse_create(nlse_t* out, int dims, const int64_t* N, double h, double a, dou
   // instruction chain wins: 3D grids of at most 2^15 sites (one thread per site; 21^3: 62.6 against
   // 93.7 for the tiled exact-sum kernel, 32^3: 67.2 against 95.9; 36^3: 89.7 against 86.3), 2D grids of
   // at most 80,000 sites (tiled; 100^2: 32.9 against 51.7, 282^2: 49.7 against 56.6; 316^2: 61.1
-  // against 54.0) and 1D lines: up to 2500 sites on the cluster path (2001 sites: 14.3 against 19.7
-  // with the exact-sum stencil, 18.1 against 19.4 for one thread per site on the dark soliton), up to
-  // 2^15 sites one thread per site (beyond ~2500 sites the cluster's 16 SMs bound it: 10,000 sites 34.8
-  // against 19.0; 20,000: 21.5 against 23.8 with the exact-sum stencil; 100,000: 36.9 against 29.0).
+  // against 54.0) and 1D lines up to 2^15 sites, which run several steps per launch (2001 sites: 8.6 with MSD walls
+  // against 19.2 for a launch per stage and 23.8 with the exact-sum stencil on a cluster; 32,000: 18.6 against 24.4
+  // for the exact-sum stencil one thread per site; 49,000: 23.5 against 25.7).
   // The FP32 forms take the tiled kernel on 3D grids above 2^17 sites (64^3: 41.8 against 47.1 for one
   // thread per site, 128^3: 88.3 against 176.8; 46^3: 39.2 against 34.5).
   c->variant = (dtype == NLSE_C128) ? 2 : 1;
@@ -636,6 +674,7 @@ int nlse_set_kernel(nlse_t c, int variant, int tile_cfg) {
   if (tile_cfg < -1 || tile_cfg > 3) return fail(NLSE_EINVAL, "tile_cfg must be -1..3");
   c->variant = variant;
   c->tile_cfg = tile_cfg;
+  c->chosen = true;
   drop_graph(c);
   return NLSE_OK;
 }
@@ -643,7 +682,8 @@ int nlse_set_kernel(nlse_t c, int variant, int tile_cfg) {
 int nlse_kernel_in_use(nlse_t c) {
   if (!c) return fail(NLSE_EINVAL, "NULL context");
   if (fused_path(c)) return 4;
-  if (line_path(c)) return c->exact() ? 2 : 1;
+  if (line_path(c)) return 2;
+  if (lines_path(c)) return c->variant == 0 ? 0 : 1;
   if (c->variant == 4) return c->d == 1 ? 0 : 1;
   if (c->d == 1) return (c->dtype == NLSE_C128 && c->variant >= 2) ? 3 : 0;
   if (c->dtype != NLSE_C128 && c->variant >= 2) return c->variant - 2;
@@ -678,7 +718,7 @@ int nlse_step(nlse_t c, int64_t nsteps, double dt) {
   if (dt > bound) return fail(NLSE_EUNSTABLE, "dt = %g above the RK4 linear stability bound %g", dt, bound);
   if (nsteps == 0) return NLSE_OK;
   cudaError_t e = cudaSuccess;
-  if (c->dtype == NLSE_C64_ACC64 && !step2_path(c))
+  if (c->dtype == NLSE_C64_ACC64 && !step2_path(c) && !lines_path(c))
     e = launch_round_master((const double2*)c->psi, (float2*)c->at(c->lay.pn32), c->total, c->stream);
   if (e != cudaSuccess) return cuda_fail(e, "round master");
   // the exact-sum scale of the state as the caller left it (stage 4 keeps it current from here on)
@@ -699,8 +739,24 @@ int nlse_step(nlse_t c, int64_t nsteps, double dt) {
       if (e != cudaSuccess) return cuda_fail(e, "cudaGraphLaunch");
     }
   }
+  if (lines_path(c) && left > 0) {   // launches of up to `per` steps; an odd number of them ends in the copy
+    void *cur = c->psi, *nxt = step_alt(c);
+    const int per = steps_per_launch(c);
+    while (left > 0 && e == cudaSuccess) {
+      const int k = left < per ? int(left) : per;
+      e = launch_steps1_any(c, dt, k, c->stream, cur, nxt);
+      void* t = cur;
+      cur = nxt;
+      nxt = t;
+      left -= k;
+    }
+    if (e == cudaSuccess && cur != c->psi)
+      e = cudaMemcpyAsync(c->psi, cur, (c->dtype == NLSE_C64 ? 8 : 16) * (size_t)c->total, cudaMemcpyDeviceToDevice,
+                          c->stream);
+    return e == cudaSuccess ? NLSE_OK : cuda_fail(e, "step launch");
+  }
   if (step2_path(c)) {   // pairs of steps end in Psi; an odd step goes through the copy and back
-    void* alt = step2_alt(c);
+    void* alt = step_alt(c);
     for (; left > 0 && e == cudaSuccess; left -= 2) {
       e = launch_step2_any(c, dt, c->stream, c->psi, alt);
       if (e != cudaSuccess) break;
@@ -852,12 +908,12 @@ int nlse_autotune(nlse_t c, int* best_tile_cfg, float* best_ms) {
     for (int t = 0; t < 4 && e == cudaSuccess; ++t) {
       c->tile_cfg = t;
       const bool step2 = step2_path(c);   // one whole step, into Psi's ping-pong copy
-      if (step2) e = launch_step2_any(c, 1e-12, c->stream, c->psi, step2_alt(c));
+      if (step2) e = launch_step2_any(c, 1e-12, c->stream, c->psi, step_alt(c));
       else e = launch_stage_any(c, 1, 1e-12, c->stream);
       if (e == cudaSuccess && !step2) e = launch_stage_any(c, 2, 1e-12, c->stream);
       if (e == cudaSuccess) e = cudaEventRecord(e0, c->stream);
       for (int r = 0; r < 3 && e == cudaSuccess; ++r)
-        e = step2 ? launch_step2_any(c, 1e-12, c->stream, c->psi, step2_alt(c)) : launch_stage_any(c, 2, 1e-12, c->stream);
+        e = step2 ? launch_step2_any(c, 1e-12, c->stream, c->psi, step_alt(c)) : launch_stage_any(c, 2, 1e-12, c->stream);
       if (e == cudaSuccess) e = cudaEventRecord(e1, c->stream);
       if (e == cudaSuccess) e = cudaEventSynchronize(e1);
       float ms = 0.f;

@@ -4,6 +4,7 @@
 #include <stdint.h>
 
 #include "nlse_device.cuh"
+#include "stage_step1d.cuh"
 #include "stage_step2d.cuh"
 
 namespace nlse {
@@ -57,14 +58,19 @@ constexpr int kFusedBoxX = 2 * (64 + 8), kFusedBoxY = 8 + 8;
 template <class T>
 cudaError_t launch_step2d(const Step2Args<T>& A, int order, int tile_cfg, cudaStream_t stream);
 
+// Up to steps1d_per_launch(n) RK4 steps of an n-site line in one launch, from A.in to A.out (stage_step1d.cuh).
+template <class T>
+int steps1d_per_launch(int n);
+template <class T>
+cudaError_t launch_steps1d(const Step1Args<T>& A, int order, int steps, cudaStream_t stream);
+
 // 1D lines on one thread-block cluster (stage_line1d.cuh): nsteps RK4 steps of
 // an n-site line in one launch; A[0..3] are stages 1..4 with Psi updated in
 // place.  cudaErrorInvalidConfiguration when the line does not fit or the
 // cluster cannot be co-scheduled (the caller then takes the per-site kernel).
 bool line_ok(int n, bool fp64);
-template <class T>
-cudaError_t launch_line_steps(const StageArgs<T>* A, int64_t nsteps, int n, int order, bool exact, int F0,
-                              int fix_offset, cudaStream_t stream);
+cudaError_t launch_line_steps(const StageArgs<P64>* A, int64_t nsteps, int n, int order, int F0, int fix_offset,
+                              cudaStream_t stream);
 
 cudaError_t launch_mass(const void* psi, bool psi_double, int64_t total, double scale, double* partials,
                         double* result, unsigned int* flag, unsigned int* done, cudaStream_t stream);

@@ -28,13 +28,12 @@ bool line_ok(int n, bool fp64) {
   return line_plan(n, fp64 ? 16 : 8, &cl, &seg, &smem);
 }
 
-template <class T>
-cudaError_t launch_line_steps(const StageArgs<T>* A, int64_t nsteps, int n, int order, bool exact, int F0,
-                              int fix_offset, cudaStream_t stream) {
+cudaError_t launch_line_steps(const StageArgs<P64>* A, int64_t nsteps, int n, int order, int F0, int fix_offset,
+                              cudaStream_t stream) {
   int cl, seg;
   size_t smem;
-  if (!line_plan(n, sizeof(typename T::C), &cl, &seg, &smem)) return cudaErrorInvalidConfiguration;
-  LineArgs<T> L;
+  if (!line_plan(n, sizeof(double2), &cl, &seg, &smem)) return cudaErrorInvalidConfiguration;
+  LineArgs<P64> L;
   memset(&L, 0, sizeof(L));
   for (int s = 0; s < 4; ++s) L.A[s] = A[s];
   L.nsteps = nsteps;
@@ -42,14 +41,7 @@ cudaError_t launch_line_steps(const StageArgs<T>* A, int64_t nsteps, int n, int 
   L.seg = seg;
   L.F0 = F0;
   L.fix_offset = fix_offset;
-  if constexpr (std::is_same<T, P64>::value) {
-    if (exact)
-      return order == 4 ? launch_line1d<T, 4, true>(L, cl, smem, stream) : launch_line1d<T, 2, true>(L, cl, smem, stream);
-  }
-  return order == 4 ? launch_line1d<T, 4, false>(L, cl, smem, stream) : launch_line1d<T, 2, false>(L, cl, smem, stream);
+  return order == 4 ? launch_line1d<P64, 4, true>(L, cl, smem, stream) : launch_line1d<P64, 2, true>(L, cl, smem, stream);
 }
-
-template cudaError_t launch_line_steps<P64>(const StageArgs<P64>*, int64_t, int, int, bool, int, int, cudaStream_t);
-template cudaError_t launch_line_steps<P32>(const StageArgs<P32>*, int64_t, int, int, bool, int, int, cudaStream_t);
 
 }  // namespace nlse
