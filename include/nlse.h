@@ -168,7 +168,8 @@ const char *nlse_last_error(void);
  *   2 = tiled kernel with the exact-sum stencil (NLSE_C128 only; other
  *       dtypes treat it as 1): the Laplacian's stencil sums are formed exactly
  *       in 64-bit fixed point on the integer pipe and converted to FP64 once;
- *       on 1D lines of up to ~49,000 sites one thread-block cluster of up to 16
+ *       2D grids of up to about 280 x 280 run a tile's four stages in one
+ *       launch per step; on 1D lines of up to ~49,000 sites one thread-block cluster of up to 16
  *       CTAs keeps the line in shared memory and runs every step of an
  *       nlse_step call in one launch,
  *   3 = generic kernel with the exact-sum stencil (NLSE_C128; else as 0).
@@ -176,19 +177,18 @@ const char *nlse_last_error(void);
  * Default: 2 for NLSE_C128 and 1 otherwise, except on grids small enough
  * that a step is bound by latency rather than by throughput: 3D grids of at
  * most 2^15 sites (NLSE_C128) or 2^17 sites (the FP32 forms) take 0,
- * NLSE_C128 2D grids of at most 80,000 sites take 1, and NLSE_C128 1D lines
- * take 1 up to 2500 sites, 0 up to 2^15 sites and 3 beyond (the plain FP64
+ * and NLSE_C128 1D lines take 1 up to 2500 sites, 0 up to 2^15 sites and 3 beyond (the plain FP64
  * stencil's instruction chain is shorter than the exact-sum stencil's
  * conversions).  Where 0 is such a line's default rather than the caller's
  * choice, its steps run several per launch as with 1 (the same arithmetic).
  * The exact-sum stencil's fixed-point scale follows the state: before every
- * step it is taken from the largest component of Psi (every component
- * below 2^53 in fixed point, 4x below the accepted range, so the largest
- * components keep all 53 bits), at the start of each nlse_step from a pass
+ * step it is taken from the largest component of Psi (below 1.6 2^54 in fixed
+ * point, 1.25x or more below the accepted range, so the largest components
+ * keep all 53 bits), at the start of each nlse_step from a pass
  * over Psi (the caller may have written it) and after each step from the
  * values the step wrote; a site whose operand is still out of range (a
- * stage state more than 4x the step's largest component) takes the FP64
- * stencil.  The resolution is thus 2^-52 or finer relative to max|Psi| for
+ * stage state that far above the step's largest component) takes the FP64
+ * stencil.  The resolution is thus 2^-54 or finer relative to max|Psi| for
  * any state, and results never depend on how steps are split into calls.
  *   4 = NLSE_C64 on 3D grids: two RK4 stages per pass (stages 1+2 and 3+4,
  *       temporal blocking): the first stage's result for a tile plus a
@@ -219,7 +219,7 @@ int nlse_kernel_in_use(nlse_t ctx);
  * appended to the text file named by the environment variable
  * NLSE_TUNE_CACHE when it is set (later processes read it instead of
  * timing).  Synchronises the stream.  *best_tile_cfg receives the chosen
- * tile_cfg (-1 when nothing is tiled: 1D grids, variants 0 and 3) and
+ * tile_cfg (-1 when there is none to choose: 1D grids, small FP64 2D grids, variants 0 and 3) and
  * *best_ms the measured stage-2 time (0 when taken from a cache); either
  * pointer may be NULL.  Tiles never change results.
  */

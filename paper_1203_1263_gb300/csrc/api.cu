@@ -129,6 +129,7 @@ struct nlse_ctx {
   int* fdev() const { return (int*)(ws + lay.status + 16); }                    // current fraction bits
   unsigned int* emax() const { return (unsigned int*)(ws + lay.status + 20); }  // stage-4 largest exponent
   bool exact() const { return dtype == NLSE_C128 && variant >= 2 && variant <= 3; }
+  unsigned int* expo() const { return (unsigned int*)(ws + lay.status + 40); }  // the whole-step kernel's four words
   unsigned int* done() const { return (unsigned int*)(ws + lay.status + 32); }  // blocks of a reduction that are through
   double* result() const { return (double*)(ws + lay.status + 64); }
   double* partials() const { return (double*)(ws + lay.partials); }
@@ -171,6 +172,7 @@ Field<T> make_field(const nlse_ctx* c, const void* in) {
   f.bc = c->bc;
   f.F = c->fixF;
   f.Fdev = (c->dtype == NLSE_C128) ? c->fdev() : nullptr;
+  f.fine = c->d == 2 && step2x_fits(int(c->n[0]), int(c->n[1]), c->bc == NLSE_BC_PERIODIC);
   f.cLF = ldexp(c->order == 4 ? c->a / (12.0 * c->h * c->h) : c->a / (c->h * c->h), -c->fixF);
   f.invcLF = R(1.0 / f.cLF);
   f.sG = R(c->s / f.cLF);
@@ -397,6 +399,12 @@ cudaError_t launch_step_fused(const nlse_ctx* c, double dt, cudaStream_t st, voi
   return c->order == 4 ? launch_fused_step<4>(A, tm12, tm34, L, st) : launch_fused_step<2>(A, tm12, tm34, L, st);
 }
 
+// Small 2D grids of the exact-sum stencil on the whole-step kernel.
+bool step2x_path(const nlse_ctx* c) {
+  return c->d == 2 && c->dtype == NLSE_C128 && c->variant == 2 &&
+         step2x_fits(int(c->n[0]), int(c->n[1]), c->bc == NLSE_BC_PERIODIC);
+}
+
 // The FP32 forms' 2D grids on the whole-step kernel (the tiled variants).
 bool step2_path(const nlse_ctx* c) {
   return c->d == 2 && c->dtype != NLSE_C128 && (c->variant == 1 || c->variant == 2 || c->variant == 4);
@@ -410,8 +418,27 @@ cudaError_t launch_step2(const nlse_ctx* c, double dt, cudaStream_t st, const vo
   return launch_step2d<T>(A, c->order, c->tile_cfg, st);
 }
 
-cudaError_t launch_step2_any(const nlse_ctx* c, double dt, cudaStream_t st, const void* cur, void* nxt) {
+cudaError_t launch_step2x_any(const nlse_ctx* c, double dt, cudaStream_t st, const void* cur, void* nxt, int turn) {
+  const Field<P64> f = make_field<P64>(c, cur);
+  Step2xArgs A = step_args<P64, Step2xArgs>(c, dt, cur, nxt);
+  A.n[0] = int(c->n[0]);
+  A.n[1] = int(c->n[1]);
+  A.cLF = f.cLF;
+  A.invcLF = f.invcLF;
+  A.sG = f.sG;
+  for (int i = 0; i < 4; ++i) A.dtc[i] = A.dtc[i] * f.cLF;
+  A.Vs = c->V ? (const double*)c->at(c->lay.vs) : nullptr;
+  A.expo = c->expo();
+  A.turn = turn & 3;
+  A.F0 = c->fixF;
+  A.fix_offset = c->fix_offset;
+  return launch_step2x(A, c->order, st);
+}
+
+// Step i of a run of steps.
+cudaError_t launch_step2_any(const nlse_ctx* c, double dt, cudaStream_t st, const void* cur, void* nxt, int i = 0) {
   switch (c->dtype) {
+    case NLSE_C128: return launch_step2x_any(c, dt, st, cur, nxt, i);
     case NLSE_C64: return launch_step2<P32>(c, dt, st, cur, nxt);
     default: return launch_step2<PMix>(c, dt, st, cur, nxt);
   }
@@ -464,7 +491,7 @@ int ensure_graph(nlse_ctx* c, double dt) {
   cudaError_t e = cudaStreamBeginCapture(c->cap, cudaStreamCaptureModeThreadLocal);
   if (e != cudaSuccess) return cuda_fail(e, "cudaStreamBeginCapture");
   cudaError_t le = cudaSuccess;
-  const bool fused = fused_path(c), step2 = step2_path(c), lines = lines_path(c);
+  const bool fused = fused_path(c), step2 = step2_path(c) || step2x_path(c), lines = lines_path(c);
   const int per = lines ? steps_per_launch(c) : 1;   // divides kGraphSteps an even number of times
   for (int i = 0; i < kGraphSteps / per && le == cudaSuccess; ++i) {
     if (lines) {   // ping-pong as below
@@ -474,7 +501,7 @@ int ensure_graph(nlse_ctx* c, double dt) {
     } else if (step2) {
       void* a = c->psi;
       void* b = step_alt(c);
-      le = (i % 2 == 0) ? launch_step2_any(c, dt, c->cap, a, b) : launch_step2_any(c, dt, c->cap, b, a);
+      le = (i % 2 == 0) ? launch_step2_any(c, dt, c->cap, a, b, i) : launch_step2_any(c, dt, c->cap, b, a, i);
     } else if (fused) {   // ping-pong: even steps Psi -> copy, odd steps copy -> Psi (kGraphSteps is even)
       void* a = c->psi;
       void* b = c->at(c->lay.alt);
@@ -606,16 +633,13 @@ int nlse_create(nlse_t* out, int dims, const int64_t* N, double h, double a, dou
   // FP64 takes the exact-sum stencil on the tiled kernels, except where the grid is so small that a
   // step is bound by latency, not by the FP64 pipe's throughput, and the plain FP64 stencil's shorter
   // instruction chain wins: 3D grids of at most 2^15 sites (one thread per site; 21^3: 62.6 against
-  // 93.7 for the tiled exact-sum kernel, 32^3: 67.2 against 95.9; 36^3: 89.7 against 86.3), 2D grids of
-  // at most 80,000 sites (tiled; 100^2: 32.9 against 51.7, 282^2: 49.7 against 56.6; 316^2: 61.1
-  // against 54.0) and 1D lines up to 2^15 sites, which run several steps per launch (2001 sites: 8.6 with MSD walls
+  // 93.7 for the tiled exact-sum kernel, 32^3: 67.2 against 95.9; 36^3: 89.7 against 86.3) and 1D lines up to 2^15 sites, which run several steps per launch (2001 sites: 8.6 with MSD walls
   // against 19.2 for a launch per stage and 23.8 with the exact-sum stencil on a cluster; 32,000: 18.6 against 24.4
   // for the exact-sum stencil one thread per site; 49,000: 23.5 against 25.7).
   // The FP32 forms take the tiled kernel on 3D grids above 2^17 sites (64^3: 41.8 against 47.1 for one
   // thread per site, 128^3: 88.3 against 176.8; 46^3: 39.2 against 34.5).
   c->variant = (dtype == NLSE_C128) ? 2 : 1;
   if (dims == 3 && total <= (dtype == NLSE_C128 ? (int64_t(1) << 15) : (int64_t(1) << 17))) c->variant = 0;
-  if (dims == 2 && dtype == NLSE_C128 && total <= 80000) c->variant = 1;
   if (dims == 1 && dtype == NLSE_C128)
     c->variant = (total <= 2500 && line_ok(int(N[0]), true)) ? 1 : (total <= (int64_t(1) << 15) ? 0 : 3);
   c->tile_cfg = -1;
@@ -640,7 +664,7 @@ int nlse_create(nlse_t* out, int dims, const int64_t* N, double h, double a, dou
     }
   }
   // Exact-sum stencil reference scale F0: the largest component of Psi0 below
-  // 2^53 in fixed point (operands are accepted below 2^55).
+  // 2^53 in fixed point.
   c->fixF = 52;
   if (e == cudaSuccess && dtype == NLSE_C128) {
     e = launch_vmax(psi, true, 2 * total, c->vbits(), c->stream);
@@ -722,7 +746,11 @@ int nlse_step(nlse_t c, int64_t nsteps, double dt) {
     e = launch_round_master((const double2*)c->psi, (float2*)c->at(c->lay.pn32), c->total, c->stream);
   if (e != cudaSuccess) return cuda_fail(e, "round master");
   // the exact-sum scale of the state as the caller left it (stage 4 keeps it current from here on)
-  if (c->exact() && (e = update_fix(c, c->psi, c->stream)) != cudaSuccess) return cuda_fail(e, "scale");
+  if (step2x_path(c)) {
+    e = cudaMemsetAsync(c->expo(), 0, 16, c->stream);
+    if (e == cudaSuccess) e = launch_max_expo((const double*)c->psi, 2 * c->total, c->expo(), c->stream);
+    if (e != cudaSuccess) return cuda_fail(e, "scale");
+  } else if (c->exact() && (e = update_fix(c, c->psi, c->stream)) != cudaSuccess) return cuda_fail(e, "scale");
   if (line_path(c)) {   // 1D: the whole call on one thread-block cluster
     e = launch_line(c, nsteps, dt);
     if (e == cudaSuccess) return NLSE_OK;
@@ -755,12 +783,12 @@ int nlse_step(nlse_t c, int64_t nsteps, double dt) {
                           c->stream);
     return e == cudaSuccess ? NLSE_OK : cuda_fail(e, "step launch");
   }
-  if (step2_path(c)) {   // pairs of steps end in Psi; an odd step goes through the copy and back
+  if (step2_path(c) || step2x_path(c)) {   // pairs of steps end in Psi; an odd step goes through the copy and back
     void* alt = step_alt(c);
-    for (; left > 0 && e == cudaSuccess; left -= 2) {
-      e = launch_step2_any(c, dt, c->stream, c->psi, alt);
+    for (int i = 0; left > 0 && e == cudaSuccess; left -= 2, i += 2) {
+      e = launch_step2_any(c, dt, c->stream, c->psi, alt, i);
       if (e != cudaSuccess) break;
-      if (left > 1) e = launch_step2_any(c, dt, c->stream, alt, c->psi);
+      if (left > 1) e = launch_step2_any(c, dt, c->stream, alt, c->psi, i + 1);
       else e = cudaMemcpyAsync(c->psi, alt, (c->dtype == NLSE_C64 ? 8 : 16) * (size_t)c->total,
                                cudaMemcpyDeviceToDevice, c->stream);
     }
@@ -876,7 +904,7 @@ void tune_file_store(const std::string& key, int cfg) {
 
 int nlse_autotune(nlse_t c, int* best_tile_cfg, float* best_ms) {
   if (!c) return fail(NLSE_EINVAL, "NULL context");
-  if (c->d == 1 || c->variant == 0 || c->variant == 3) {   // nothing tiled to tune
+  if (c->d == 1 || c->variant == 0 || c->variant == 3 || step2x_path(c)) {   // no tile to choose
     if (best_tile_cfg) *best_tile_cfg = -1;
     if (best_ms) *best_ms = 0.f;
     return NLSE_OK;

@@ -108,6 +108,7 @@ struct Field {
   int F;             // exact-sum stencil: the reference fraction bits F0 that cLF and V / cLF are scaled by
   const int* Fdev;   // exact-sum stencil: device word holding the fraction bits of the current state
                      //   (derived from max |Psi| every step; nullptr: use F)
+  int fine;          // exact-sum stencil, 2D: the nearest neighbours' rounding is taken back too (fix_correction)
   double cLF;        // exact-sum stencil: cL * 2^-F
   R sG;              // exact-sum stencil: s / cLF
   R invcLF;          // exact-sum stencil: 1 / cLF
@@ -247,8 +248,8 @@ __device__ __forceinline__ typename V2<typename T::R>::t a_lap(const Field<T>& f
 // 16 s1 - s2 - 30 d Psi_c (or s1 - 2d Psi_c) are then exact integers, and one
 // conversion and one multiply by cL 2^-F give a*Lap in FP64.  An operand is
 // accepted while |v| 2^F < 2^55; F follows the state so that its largest
-// component stays below 2^53 (4x headroom for the stages' intermediate
-// states), which keeps all 53 bits of the largest components.  An operand
+// component stays below 1.6 2^54 (see range_bits), which keeps all 53 bits of
+// the largest components.  An operand
 // outside the range (or Inf/NaN) yields kFixBad and the site falls back to
 // the FP64 stencil, so the result is always defined.  Bounds of the sums
 // (L = 2^55): a deep site's 16 s1 - s2 - 30 d Psi_c stays below 64 d L
@@ -275,7 +276,7 @@ __device__ __forceinline__ longlong2 fix2(double2 v, int F) { return make_longlo
 
 // The fraction bits the exact-sum stencil uses for the current state: F is
 // re-derived on the device before every step from the largest component of
-// Psi^n (|v| 2^F < 2^53, 4x below the accepted range), so the fixed-point resolution
+// Psi^n (see range_bits), so the fixed-point resolution
 // 2^-F always follows the state's own scale.  The stencil sums are formed at
 // that scale and converted to units of cLF = cL 2^-F0 (F0: the reference
 // scale fixed at creation) by an exact power-of-two exponent shift.
@@ -286,13 +287,51 @@ __device__ __forceinline__ int cur_fix(const Field<T>& f) { return f.Fdev ? __ld
 __device__ __forceinline__ unsigned int expo_bits(double v) { return (unsigned int)(__double2hiint(v) >> 20) & 0x7FFu; }
 __device__ __forceinline__ unsigned int expo_bits(float v) { return 0u; }
 
-// Largest biased exponent over a full warp into *p (one atomic per warp, skipped when *p is already as
+// What the fixed-point scale follows: the biased exponent of |v|, one more from 1.6 times its power of two on, 2047
+// or more for Inf / NaN.  With F = 1077 - (the largest of the state) the largest component lies in
+// [0.8, 1.6) 2^54: 53 bits kept for every component down to a quarter of it, and a factor of 1.25 at least up to
+// the accepted range for the stages' intermediate states (beyond, a site takes the FP64 stencil).
+__device__ __forceinline__ unsigned int range_bits(double v) {
+  return (unsigned int)((__double2hiint(v) & 0x7FFFFFFF) + 0x66667) >> 20;
+}
+__device__ __forceinline__ unsigned int range_bits(float v) { return 0u; }
+
+// Largest range_bits over a full warp into *p (one atomic per warp, skipped when *p is already as
 // large).  Every lane of the warp must call it.
 __device__ __forceinline__ void emax_commit(unsigned int* p, unsigned int e) {
   e = __reduce_max_sync(0xffffffffu, e);
   if ((threadIdx.x & 31) == 0 && e > __ldcg(p)) atomicMax(p, e);
 }
 __device__ __forceinline__ bool fbad(longlong2 v) { return (v.x == kFixBad) | (v.y == kFixBad); }
+
+// What rounding component v to fixed point left out, in 1/256 of the resolution (-128 .. 127).
+__device__ __forceinline__ int fix_low(double v, int F) {
+  const unsigned long long u = (unsigned long long)__double_as_longlong(v);
+  const int e = int((u >> 52) & 0x7FF), k = 1075 - F - e;   // bits of the mantissa below the resolution
+  if (e == 0 || k <= 0 || k > 62) return 0;
+  const long long m = (long long)((u & 0x000FFFFFFFFFFFFFull) | 0x0010000000000000ull);
+  long long r = m;                                  // the remainder in units of 2^-k of the resolution
+  if (k <= 54) r -= ((m + (1ll << (k - 1))) >> k) << k;
+  const int lo = int(k > 8 ? r >> (k - 8) : r << (8 - k));
+  return min((u >> 63) ? -lo : lo, 127);
+}
+
+// The 2SHOC sum's correction for its operands' rounding on planes and lines: the centre's, which the sum weighs
+// 30 d times (in 2D 60 against 16 and 1: alone it halves the sum's error), and on small planes (Field::fine), where
+// the FP64 stencil's lower error is the measure, the nearest neighbours' too.
+template <class T, int D, class Acc>
+__device__ __forceinline__ longlong2 fix_correction(const Field<T>& f, const Acc& acc, double2 pc, int F) {
+  int x = -30 * D * fix_low(pc.x, F), y = -30 * D * fix_low(pc.y, F);
+  if (D == 2 && f.fine) {
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      const double2 v = acc.at1(q >> 1, (q & 1) ? 1 : -1);
+      x += 16 * fix_low(v.x, F);
+      y += 16 * fix_low(v.y, F);
+    }
+  }
+  return make_longlong2((x + 128) >> 8, (y + 128) >> 8);
+}
 
 // The FP64 stencil as an out-of-line call (out-of-range operands).
 template <class T, int D, int ORDER, class Acc>
@@ -405,7 +444,9 @@ __device__ __forceinline__ double2 a_lap_exact(const Field<T>& f, const Acc& acc
     s1x += u.x + w.x;
     s1y += u.y + w.y;
   }
-  const double Nc = Ng * f.cLF;   // physical N_c, for the walls' ghosts and the fallback
+  // physical N_c, for the walls' ghosts and the fallback (never contracted into what uses it, so that every
+  // kernel rounds it alike)
+  const double Nc = __dmul_rn(Ng, f.cLF);
   if constexpr (ORDER == 2) {
     if (bad) {
       const double2 aL = a_lap_slow<T, D, ORDER>(f, acc, idx, c, pc, Nc);
@@ -434,8 +475,13 @@ __device__ __forceinline__ double2 a_lap_exact(const Field<T>& f, const Acc& acc
     const double2 aL = a_lap_slow<T, D, ORDER>(f, acc, idx, c, pc, Nc);
     return {aL.x * f.invcLF, aL.y * f.invcLF};
   }
-  const long long Sx = 16 * s1x - s2x - 30 * D * cc.x;
-  const long long Sy = 16 * s1y - s2y - 30 * D * cc.y;
+  long long Sx = 16 * s1x - s2x - 30 * D * cc.x;
+  long long Sy = 16 * s1y - s2y - 30 * D * cc.y;
+  if constexpr (D < 3) {
+    const longlong2 r = fix_correction<T, D>(f, acc, pc, acc.fixF());
+    Sx += r.x;
+    Sy += r.y;
+  }
   return {i2d_rn(Sx, eadj), i2d_rn(Sy, eadj)};
 }
 
@@ -476,8 +522,13 @@ __device__ __forceinline__ double2 a_lap_exact_deep(const Field<T>& f, const Acc
     const double2 aL = a_lap_body<T, D, ORDER, Acc, false>(f, acc, idx, c, pc, Ng * f.cLF);
     return {aL.x * f.invcLF, aL.y * f.invcLF};
   }
-  const long long Sx = 16 * s1x - s2x - 30 * D * cc.x;
-  const long long Sy = 16 * s1y - s2y - 30 * D * cc.y;
+  long long Sx = 16 * s1x - s2x - 30 * D * cc.x;
+  long long Sy = 16 * s1y - s2y - 30 * D * cc.y;
+  if constexpr (D < 3) {
+    const longlong2 r = fix_correction<T, D>(f, acc, pc, acc.fixF());
+    Sx += r.x;
+    Sy += r.y;
+  }
   return {i2d_rn(Sx, eadj), i2d_rn(Sy, eadj)};
 }
 
@@ -591,7 +642,7 @@ __device__ __forceinline__ unsigned int rk_apply(const StageArgs<T>& A, int64_t 
       }
       A.master[i] = q;
       if (!(finite_bits(q.x) && finite_bits(q.y))) atomicOr(A.flag, 1u);
-      return max(expo_bits(q.x), expo_bits(q.y));
+      return max(range_bits(q.x), range_bits(q.y));
     }
   }
   return 0u;

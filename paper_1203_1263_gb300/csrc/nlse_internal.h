@@ -6,6 +6,7 @@
 #include "nlse_device.cuh"
 #include "stage_step1d.cuh"
 #include "stage_step2d.cuh"
+#include "stage_step2x.cuh"
 
 namespace nlse {
 
@@ -57,6 +58,12 @@ constexpr int kFusedBoxX = 2 * (64 + 8), kFusedBoxY = 8 + 8;
 // One RK4 step of a 2D grid in one launch, Psi^n in A.in to Psi^{n+1} in A.out (stage_step2d.cuh).
 template <class T>
 cudaError_t launch_step2d(const Step2Args<T>& A, int order, int tile_cfg, cudaStream_t stream);
+
+// The same for FP64 with the exact-sum stencil (stage_step2x.cuh); launch_max_expo puts the largest exponent of a
+// complex128 array (n components) into the word of the first step.
+bool step2x_fits(int ny, int nx, bool periodic);   // grids it is the faster one for
+cudaError_t launch_step2x(const Step2xArgs& A, int order, cudaStream_t stream);
+cudaError_t launch_max_expo(const double* psi, int64_t n, unsigned int* expo, cudaStream_t stream);
 
 // Up to steps1d_per_launch(n) RK4 steps of an n-site line in one launch, from A.in to A.out (stage_step1d.cuh).
 template <class T>

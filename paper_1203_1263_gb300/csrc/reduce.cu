@@ -188,36 +188,41 @@ __global__ void __launch_bounds__(256) k_vmax(const VR* __restrict__ V, int64_t 
   if ((threadIdx.x & 31) == 0) atomicMax(out, (unsigned long long)__double_as_longlong(m));
 }
 
-// Largest biased exponent over the components of a complex128 array into *out
+// Largest range_bits over the components of a complex128 array into *out
 // (exact-sum scale of the current state; *out must start at 0).
 __global__ void __launch_bounds__(256) k_max_expo(const double* __restrict__ v, int64_t n, unsigned int* out) {
   unsigned int e = 0;
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
-    e = max(e, expo_bits(__ldg(v + i)));
+    e = max(e, range_bits(__ldg(v + i)));
   emax_commit(out, e);
 }
 
-// Fraction bits of the exact-sum stencil for the state whose largest
-// component has biased exponent E (collected in *emax by k_max_expo or by
-// stage 4): |v| < 2^(E - 1022), so F = 1075 - E keeps every component below
-// 2^53 in fixed point, 4x below the accepted range 2^55.  A zero state keeps F0;
-// a non-finite one keeps the previous F (the non-finite flag reports it).
-// `offset` is a test hook (nlse_debug_set).  Resets *emax for the next step.
+// Fraction bits of the exact-sum stencil for the state whose largest range_bits
+// is E (collected in *emax by k_max_expo or by stage 4): F = 1077 - E.  A zero
+// state keeps F0; a non-finite one keeps the previous F (the non-finite flag
+// reports it).  `offset` is a test hook (nlse_debug_set).  Resets *emax for the
+// next step.
 __global__ void k_fix_update(unsigned int* emax, int* fdev, int F0, int offset) {
   if (threadIdx.x == 0 && blockIdx.x == 0) {
     const unsigned int E = *emax;
     if (E == 0u) *fdev = F0 + offset;
-    else if (E < 2047u) *fdev = 1075 - int(E) + offset;
+    else if (E < 2047u) *fdev = 1077 - int(E) + offset;
     *emax = 0u;
   }
+}
+
+cudaError_t launch_max_expo(const double* psi, int64_t n, unsigned int* expo, cudaStream_t stream) {
+  int64_t b = (n + 255) / 256;
+  if (b > 152 * 8) b = 152 * 8;
+  k_max_expo<<<(unsigned)b, 256, 0, stream>>>(psi, n, expo);
+  return cudaGetLastError();
 }
 
 cudaError_t launch_fix_update(const double* psi, int64_t n, unsigned int* emax, int* fdev, int F0, int offset,
                               cudaStream_t stream) {
   if (psi) {
-    int64_t b = (n + 255) / 256;
-    if (b > 152 * 8) b = 152 * 8;
-    k_max_expo<<<(unsigned)b, 256, 0, stream>>>(psi, n, emax);
+    const cudaError_t e = launch_max_expo(psi, n, emax, stream);
+    if (e != cudaSuccess) return e;
   }
   k_fix_update<<<1, 32, 0, stream>>>(emax, fdev, F0, offset);
   return cudaGetLastError();

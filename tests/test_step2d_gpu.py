@@ -46,3 +46,15 @@ def test_whole_step_equals_per_site_bitwise(shape, bc, order, dtype):
             ref = run(psi, V, bc, order, dtype, 0, -1, steps)
             for tile in (-1, 0, 1, 2, 3):
                 assert np.array_equal(run(psi, V, bc, order, dtype, 1, tile, steps), ref), (tile, steps, V is None)
+
+
+@pytest.mark.parametrize("shape", SHAPES)
+@pytest.mark.parametrize("bc", ["dirichlet", "msd", "l0", "periodic"])
+@pytest.mark.parametrize("order", [2, 4])
+def test_whole_fp64_step_equals_per_site_exact_sum_bitwise(shape, bc, order):
+    """The FP64 whole step (exact-sum stencil) against the one-thread-per-site exact-sum kernel."""
+    psi = field(shape, bc)
+    for V in (None, W.random_potential(shape, 5, 0.1)):
+        for steps in ((1,), (2, 19), (5,)):
+            ref = run(psi, V, bc, order, "c128", 3, -1, steps)
+            assert np.array_equal(run(psi, V, bc, order, "c128", 2, -1, steps), ref), (steps, V is None)
