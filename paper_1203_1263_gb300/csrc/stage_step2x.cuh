@@ -130,7 +130,7 @@ struct Step2xTile {
     __syncthreads();
     for (int e = threadIdx.x; e < PS; e += NT) {
       X0[e] = fix2(P[e], F);
-      if (ORDER == 4) L0[e] = low(P[e], F);
+      L0[e] = low(P[e], F);
     }
     __syncthreads();
   }
@@ -159,17 +159,18 @@ struct Step2xTile {
     const longlong2 cc = x[e], xm = x[e - 1], xp = x[e + 1], ym = x[e - W], yp = x[e + W];
     bool bad = fbad(cc) | fbad(xm) | fbad(xp) | fbad(ym) | fbad(yp);
     long long sx = (yp.x + ym.x) + (xp.x + xm.x), sy = (yp.y + ym.y) + (xp.y + xm.y);
+    const char2 lc = l[e], l0 = l[e - 1], l1 = l[e + 1], l2 = l[e - W], l3 = l[e + W];   // fix_correction
     if constexpr (ORDER == 4) {
       const longlong2 xm2 = x[e - 2], xp2 = x[e + 2], ym2 = x[e - 2 * W], yp2 = x[e + 2 * W];
       bad |= fbad(xm2) | fbad(xp2) | fbad(ym2) | fbad(yp2);
       sx = 16 * sx - ((ym2.x + yp2.x) + (xm2.x + xp2.x)) - 60 * cc.x;
       sy = 16 * sy - ((ym2.y + yp2.y) + (xm2.y + xp2.y)) - 60 * cc.y;
-      const char2 lc = l[e], l0 = l[e - 1], l1 = l[e + 1], l2 = l[e - W], l3 = l[e + W];   // fix_correction
-      sx += (16 * ((l0.x + l1.x) + (l2.x + l3.x)) - 60 * lc.x + 128) >> 8;
-      sy += (16 * ((l0.y + l1.y) + (l2.y + l3.y)) - 60 * lc.y + 128) >> 8;
+      const char2 m0 = l[e - 2], m1 = l[e + 2], m2 = l[e - 2 * W], m3 = l[e + 2 * W];
+      sx += (16 * ((l0.x + l1.x) + (l2.x + l3.x)) - ((m0.x + m1.x) + (m2.x + m3.x)) - 60 * lc.x + 128) >> 8;
+      sy += (16 * ((l0.y + l1.y) + (l2.y + l3.y)) - ((m0.y + m1.y) + (m2.y + m3.y)) - 60 * lc.y + 128) >> 8;
     } else {
-      sx -= 4 * cc.x;
-      sy -= 4 * cc.y;
+      sx += -4 * cc.x + (((l0.x + l1.x) + (l2.x + l3.x) - 4 * lc.x + 128) >> 8);
+      sy += -4 * cc.y + (((l0.y + l1.y) + (l2.y + l3.y) - 4 * lc.y + 128) >> 8);
     }
     const double N = fma(A.sG, norm2(pc), -(with_v ? Vs[e] : 0.0));
     double2 aL;
@@ -199,7 +200,7 @@ struct Step2xTile {
       const double2 y = {fma(A.dtc[S - 1], Fv.x, pn.x), fma(A.dtc[S - 1], Fv.y, pn.y)};
       d[e] = y;
       x[e] = fix2(y, F);
-      if (ORDER == 4) l[e] = low(y, F);
+      l[e] = low(y, F);
     } else if (own) {
       const double2 pn = P[e], kt = *k;
       const double2 q = {fma(A.dtc[3], kt.x + Fv.x, pn.x), fma(A.dtc[3], kt.y + Fv.y, pn.y)};
@@ -230,7 +231,7 @@ struct Step2xTile {
     return c;
   }
 
-  __device__ __forceinline__ void ghosts(const Clip& c, const double2* d, longlong2* x) {
+  __device__ __forceinline__ void ghosts(const Clip& c, const double2* d, longlong2* x, char2* l) {
     const Field<L64> f = field();
     const int rw = c.xhi - c.xlo, rh = c.yhi - c.ylo;
     const int n0 = c.top ? rw : 0, n1 = n0 + (c.bot ? rw : 0), n2 = n1 + (c.left ? rh : 0), n3 = n2 + (c.right ? rh : 0);
@@ -256,6 +257,7 @@ struct Step2xTile {
       if (row) g = ghost_fix<L64, 2>(f, acc, 0, dir, e, pc, dh, Nc, m2, F, &bad);
       else g = ghost_fix<L64, 2>(f, acc, 1, dir, e, pc, dh, Nc, m2, F, &bad);
       x[e + 2 * dir * (row ? W : 1)] = bad ? longlong2{kFixBad, kFixBad} : g;
+      l[e + 2 * dir * (row ? W : 1)] = make_char2(0, 0);
     }
   }
 
@@ -304,7 +306,7 @@ struct Step2xTile {
     for (int S = 1; S <= 4; ++S) {
       const Clip c = clip(S);
       if (ORDER == 4 && walls) {
-        ghosts(c, din, xin);
+        ghosts(c, din, xin, lin);
         __syncthreads();
       }
       const unsigned rw = (unsigned)(c.xhi - c.xlo), n = rw * (unsigned)(c.yhi - c.ylo);
