@@ -1,6 +1,7 @@
 // 2D stage launches: variant 0 = generic kernel, 1 = halo-tiled kernel,
 // 2 / 3 = tiled / generic with the exact-sum stencil (FP64 only).
 #include "stage_generic.cuh"
+#include "stage_split.cuh"
 #include "stage_tiled.cuh"
 
 namespace nlse {
@@ -16,8 +17,8 @@ cudaError_t launch_stage(const StageArgs<T>& A, const LaunchCfg& L, cudaStream_t
       if constexpr (fp64) if (exact) return launch_generic_periodic<T, D, ORDER, true>(A, stream);
       return launch_generic_periodic<T, D, ORDER>(A, stream);
     }
-    if constexpr (fp64) if (exact) return launch_generic<T, D, ORDER, true>(A, stream);
-    return launch_generic<T, D, ORDER>(A, stream);
+    if constexpr (fp64) if (exact) return launch_split<T, D, ORDER, true>(A, stream, true, true);
+    return launch_split<T, D, ORDER>(A, stream, true, true);
   }
   // tiled: deep interior + the wall shell (periodic grids: the two layers at each end of each axis)
   auto deep = [&](cudaStream_t st) -> cudaError_t {
@@ -29,8 +30,8 @@ cudaError_t launch_stage(const StageArgs<T>& A, const LaunchCfg& L, cudaStream_t
       if constexpr (fp64) if (exact) return launch_shell_periodic<T, D, ORDER, true>(A, st);
       return launch_shell_periodic<T, D, ORDER>(A, st);
     }
-    if constexpr (fp64) if (exact) return launch_shell<T, D, ORDER, true>(A, st);
-    return launch_shell<T, D, ORDER>(A, st);
+    if constexpr (fp64) if (exact) return launch_split<T, D, ORDER, true>(A, st, false, false);
+    return launch_split<T, D, ORDER>(A, st, false, false);
   };
   return launch_deep_and_shell(L, stream, has_deep(D, A.f.m), deep, shell);
 }

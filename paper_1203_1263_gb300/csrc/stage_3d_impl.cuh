@@ -6,6 +6,7 @@
 #pragma once
 #include "stage_generic.cuh"
 #include "stage_slab.cuh"
+#include "stage_split.cuh"
 #include "stage_tiled.cuh"
 #include "stage_tma.cuh"
 
@@ -22,8 +23,8 @@ cudaError_t launch_stage(const StageArgs<T>& A, const LaunchCfg& L, cudaStream_t
       if constexpr (fp64) if (exact) return launch_generic_periodic<T, D, ORDER, true>(A, stream);
       return launch_generic_periodic<T, D, ORDER>(A, stream);
     }
-    if constexpr (fp64) if (exact) return launch_generic<T, D, ORDER, true>(A, stream);
-    return launch_generic<T, D, ORDER>(A, stream);
+    if constexpr (fp64) if (exact) return launch_split<T, D, ORDER, true>(A, stream, true, true);
+    return launch_split<T, D, ORDER>(A, stream, true, true);
   }
   // tiled: deep interior (TMA-fed when the layout allows) + the wall shell, as
   // shared-memory slabs (FP32 stages: three x layers per x wall) or, for thin
@@ -47,8 +48,8 @@ cudaError_t launch_stage(const StageArgs<T>& A, const LaunchCfg& L, cudaStream_t
       if constexpr (fp64) if (exact) return launch_shell_slabs<T, ORDER, true, nsx>(B, st, L.side_yx);
       return launch_shell_slabs<T, ORDER, false, nsx>(B, st, L.side_yx);
     }
-    if constexpr (fp64) if (exact) return launch_shell<T, D, ORDER, true>(B, st);
-    return launch_shell<T, D, ORDER>(B, st);
+    if constexpr (fp64) if (exact) return launch_split<T, D, ORDER, true>(B, st, false, false);
+    return launch_split<T, D, ORDER>(B, st, false, false);
   };
   if (slabs) return launch_deep_and_shell(L, stream, has_deep(D, A.f.m), deep, shell);
   LaunchCfg L1 = L;   // one shell kernel: no use for the slabs' extra streams

@@ -1,0 +1,169 @@
+// The wall-aware per-site stage as three kinds of threads.
+//
+// A site next to a wall takes a longer chain of instructions than one in the
+// deep interior (ghosts with divisions, then the boundary sites it serves, each
+// with its own loads and stores), and in a kernel with one thread per interior
+// site every warp of a row holds both kinds, so each warp runs both chains one
+// after the other.  On small grids that chain is the stage's time.  Here the
+// deep sites, the sites next to a wall and the boundary sites are three ranges of
+// blocks: warps hold one kind, and a boundary site has a thread of its own, which
+// evaluates F at its interior neighbour once more (MSD; Eq. msd) instead of
+// waiting for that site's thread.  The arithmetic is site_rhs, serve_walls and
+// rk_apply as everywhere, so results are bit-for-bit those of one thread per
+// interior site (21^3 FP64 2SHOC MSD: 38.6 against 60.5 us per step).
+#pragma once
+#include "nlse_internal.h"
+#include "stage_generic.cuh"
+
+namespace nlse {
+
+// The t-th boundary site: the sites with some index 0 or N - 1, as shell_decode's faces.
+template <class T, int D, class I>
+__device__ __forceinline__ int64_t boundary_decode(const Field<T>& f, I t, int* idx) {
+  auto outer = [&](int k, int q) { return q == 0 ? 0 : f.n[k] - 1; };
+  if constexpr (D == 1) {
+    idx[0] = outer(0, int(t));
+  } else if constexpr (D == 2) {
+    const I F0 = I(2) * I(f.n[1]);
+    if (t < F0) {
+      idx[0] = outer(0, t < I(f.n[1]) ? 0 : 1);
+      idx[1] = int(t < I(f.n[1]) ? t : t - I(f.n[1]));
+    } else {
+      t -= F0;
+      idx[0] = 1 + int(t >> 1);
+      idx[1] = outer(1, int(t & 1));
+    }
+  } else {
+    const I plane = I(f.n[1]) * I(f.n[2]), F0 = I(2) * plane, F1 = I(f.m[0]) * I(2) * I(f.n[2]);
+    if (t < F0) {
+      idx[0] = outer(0, t < plane ? 0 : 1);
+      const I r = t < plane ? t : t - plane;
+      idx[1] = int(r / I(f.n[2]));
+      idx[2] = int(r % I(f.n[2]));
+    } else if (t < F0 + F1) {
+      t -= F0;
+      const I pa = I(2) * I(f.n[2]);
+      idx[0] = 1 + int(t / pa);
+      const I r = t % pa;
+      idx[1] = outer(1, r < I(f.n[2]) ? 0 : 1);
+      idx[2] = int(r < I(f.n[2]) ? r : r - I(f.n[2]));
+    } else {
+      t -= F0 + F1;
+      const I pa = I(2) * I(f.m[1]);
+      idx[0] = 1 + int(t / pa);
+      const I r = t % pa;
+      idx[1] = 1 + int(r >> 1);
+      idx[2] = outer(2, int(r & 1));
+    }
+  }
+  int64_t s = 0;
+#pragma unroll
+  for (int k = 0; k < D; ++k) s += idx[k] * f.st[k];
+  return s;
+}
+
+inline int64_t boundary_count(int D, const int* n, const int* m) {
+  int64_t all = 1, inner = 1;
+  for (int k = 0; k < D; ++k) {
+    all *= n[k];
+    inner *= m[k];
+  }
+  return all - inner;
+}
+
+// Blocks [0, b1): the n1 deep sites; [b1, b2): the n2 shell sites; the rest: the n3 boundary sites.
+template <class T, int D, int ORDER, bool EXACT, class I>
+__global__ void __launch_bounds__(256) k_stage_split(const StageArgs<T> A, unsigned b1, unsigned b2, int64_t n1, int64_t n2,
+                                                     int64_t n3) {
+  using R = typename T::R;
+  using C2 = typename V2<R>::t;
+  const Field<T>& f = A.f;
+  unsigned int ex = 0;
+  int idx[D];
+  grid_launch_dependents();
+  grid_wait();
+  if (blockIdx.x < b1) {
+    const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (t < n1) {
+      I rem = I(t);
+      int64_t c = 0;
+#pragma unroll
+      for (int k = D - 1; k >= 0; --k) {
+        const I mk = I(f.n[k] - 4), q = rem / mk;
+        idx[k] = int(rem - q * mk) + 2;
+        rem = q;
+        c += idx[k] * f.st[k];
+      }
+      const GAcc<T, D> acc(f, c);
+      const PointVals<T> p = load_point<T, -1, EXACT>(A, c, true);
+      const C2 pc = acc.at0();
+      const R N = fma(EXACT ? f.sG : f.s, norm2(pc), -p.v);
+      C2 aL;
+      if constexpr (EXACT) aL = a_lap_exact_deep<T, D, ORDER>(f, acc, idx, c, pc, N);
+      else aL = a_lap_body<T, D, ORDER, GAcc<T, D>, false>(f, acc, idx, c, pc, N);
+      ex = rk_apply<T>(A, c, {-fma(N, pc.y, aL.y), fma(N, pc.x, aL.x)}, p);
+    }
+  } else if (blockIdx.x < b2) {
+    const int64_t t = (int64_t)(blockIdx.x - b1) * blockDim.x + threadIdx.x;
+    if (t < n2) {
+      const int64_t c = shell_decode<T, D, I>(f, I(t), idx);
+      const GAcc<T, D> acc(f, c);
+      const PointVals<T> p = load_point<T, -1, EXACT>(A, c, true);
+      C2 pc;
+      R m2w;
+      ex = rk_apply<T>(A, c, site_rhs<T, D, ORDER, EXACT>(f, acc, idx, c, p.v, &pc, &m2w), p);
+    }
+  } else {
+    const int64_t t = (int64_t)(blockIdx.x - b2) * blockDim.x + threadIdx.x;
+    if (t < n3) {
+      const int64_t b = boundary_decode<T, D, I>(f, I(t), idx);
+      const PointVals<T> p = load_point<T, -1, EXACT>(A, b, true);
+      C2 Fb = {R(0), R(0)};
+      if (f.bc == BC_MSD) {   // see serve_walls
+        const C2 pb = ld2<R>(f.in, b);
+        int64_t c = 0;
+#pragma unroll
+        for (int k = 0; k < D; ++k) {
+          idx[k] = min(max(idx[k], 1), f.n[k] - 2);
+          c += idx[k] * f.st[k];
+        }
+        const GAcc<T, D> acc(f, c);
+        C2 pc;
+        R m2w;
+        const C2 F = site_rhs<T, D, ORDER, EXACT>(f, acc, idx, c, ldv<R>(EXACT ? A.Vs : f.V, c), &pc, &m2w);
+        const R m2 = EXACT ? m2w : norm2(pc);
+        R theta = R(0);
+        if (EXACT ? m2 > R(0) : m2 > f.tiny) theta = fma(F.y, pc.x, -(F.x * pc.y)) / m2;
+        Fb = {-theta * pb.y, theta * pb.x};
+      } else if (f.bc == BC_L0) {
+        const C2 pb = ld2<R>(f.in, b);
+        const R Nb = fma(EXACT ? f.sG : f.s, norm2(pb), -p.v);
+        Fb = {-Nb * pb.y, Nb * pb.x};
+      }
+      ex = rk_apply<T>(A, b, Fb, p);
+    }
+  }
+  if (A.emax) emax_commit(A.emax, ex);
+}
+
+// Every site (deep: the tiled kernels' part left out).  `early`: on the step's own stream, where the kernel before may
+// still run.
+template <class T, int D, int ORDER, bool EXACT = false>
+cudaError_t launch_split(const StageArgs<T>& A, cudaStream_t stream, bool deep, bool early) {
+  int64_t n1 = 1;
+  for (int k = 0; k < D; ++k) n1 *= A.f.n[k] > 4 ? A.f.n[k] - 4 : 0;
+  const int64_t n2 = A.f.ninterior - n1, n3 = boundary_count(D, A.f.n, A.f.m);
+  if (!deep) n1 = 0;
+  const int threads = site_kernel_threads(n1 + n2 + n3);
+  auto blocks = [&](int64_t n) { return (unsigned)((n + threads - 1) / threads); };
+  const unsigned b1 = blocks(n1), b2 = b1 + blocks(n2), b3 = b2 + blocks(n3);
+  auto run = [&](auto kern) -> cudaError_t {
+    if (early) return launch_early(kern, dim3(b3), dim3((unsigned)threads), 0, stream, A, b1, b2, n1, n2, n3);
+    kern<<<b3, threads, 0, stream>>>(A, b1, b2, n1, n2, n3);
+    return cudaGetLastError();
+  };
+  if (A.f.ninterior + n3 < (int64_t(1) << 31)) return run(k_stage_split<T, D, ORDER, EXACT, uint32_t>);
+  return run(k_stage_split<T, D, ORDER, EXACT, uint64_t>);
+}
+
+}  // namespace nlse
