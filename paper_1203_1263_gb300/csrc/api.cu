@@ -632,12 +632,12 @@ int nlse_create(nlse_t* out, int dims, const int64_t* N, double h, double a, dou
   // Default kernel per form and size, from timings of the paper's workloads (MSD, 2SHOC, us per step):
   // FP64 takes the exact-sum stencil on the tiled kernels, except where the grid is so small that a
   // step is bound by latency, not by the FP64 pipe's throughput, and the plain FP64 stencil's shorter
-  // instruction chain wins: 3D grids of at most 2^15 sites (one thread per site; 21^3: 62.6 against
-  // 93.7 for the tiled exact-sum kernel, 32^3: 67.2 against 95.9; 36^3: 89.7 against 86.3) and 1D lines up to 2^15 sites, which run several steps per launch (2001 sites: 8.6 with MSD walls
+  // instruction chain wins: 3D grids of at most 2^15 sites (one thread per site; 21^3: 38.6 against
+  // 94.1 for the tiled exact-sum kernel, 32^3: 62.1 against 93.6) and 1D lines up to 2^15 sites, which run several steps per launch (2001 sites: 8.6 with MSD walls
   // against 19.2 for a launch per stage and 23.8 with the exact-sum stencil on a cluster; 32,000: 18.6 against 24.4
   // for the exact-sum stencil one thread per site; 49,000: 23.5 against 25.7).
-  // The FP32 forms take the tiled kernel on 3D grids above 2^17 sites (64^3: 41.8 against 47.1 for one
-  // thread per site, 128^3: 88.3 against 176.8; 46^3: 39.2 against 34.5).
+  // The FP32 forms take the tiled kernel on 3D grids above 2^17 sites (64^3: 26.6 against 30.0 for one
+  // thread per site, 128^3: 67.5 against 105; 40^3: 17.1 against 15.3).
   c->variant = (dtype == NLSE_C128) ? 2 : 1;
   if (dims == 3 && total <= (dtype == NLSE_C128 ? (int64_t(1) << 15) : (int64_t(1) << 17))) c->variant = 0;
   if (dims == 1 && dtype == NLSE_C128)

@@ -1,10 +1,12 @@
-// 3D stage launches: variant 0 = generic kernel, 1 = z-marching tiled kernel
-// (TMA-fed when the layout allows, else cooperative loads),
+// 3D stage launches: variant 0 = one thread per site, 1 = z-marching tiled kernel
+// (TMA-fed when the layout allows, else cooperative loads; FP32 forms of a few
+// million sites or without TMA: columns through the L1 cache),
 // 2 / 3 = tiled / generic with the exact-sum stencil (FP64 only).
 // Included by one small translation unit per (precision, order), so that the
 // many kernel instantiations compile in parallel.
 #pragma once
 #include "stage_generic.cuh"
+#include "stage_march.cuh"
 #include "stage_slab.cuh"
 #include "stage_split.cuh"
 #include "stage_tiled.cuh"
@@ -25,6 +27,13 @@ cudaError_t launch_stage(const StageArgs<T>& A, const LaunchCfg& L, cudaStream_t
     }
     if constexpr (fp64) if (exact) return launch_split<T, D, ORDER, true>(A, stream, true, true);
     return launch_split<T, D, ORDER>(A, stream, true, true);
+  }
+  if constexpr (!fp64) {
+    // a few million sites, or rows TMA cannot take: one launch (see the figures in stage_march.cuh; the hook that
+    // drives the TMA kernels' bounded waits keeps those)
+    const bool small = (int64_t)A.f.n[0] * A.f.n[1] * A.f.n[2] <= 3000000;
+    if (A.stage >= 1 && (small || !L.tmap) && march_ok(A.f.n, A.f.bc) && !L.extra_tx)
+      return launch_march<T, ORDER>(A, stream);
   }
   // tiled: deep interior (TMA-fed when the layout allows) + the wall shell, as
   // shared-memory slabs (FP32 stages: three x layers per x wall) or, for thin

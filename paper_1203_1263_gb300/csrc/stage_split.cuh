@@ -71,6 +71,54 @@ inline int64_t boundary_count(int D, const int* n, const int* m) {
   return all - inner;
 }
 
+// The t-th of n sites next to the walls, without the boundary sites it serves.
+template <class T, int D, int ORDER, bool EXACT, class I>
+__device__ __forceinline__ unsigned int shell_site(const StageArgs<T>& A, int64_t t, int64_t n) {
+  if (t >= n) return 0u;
+  int idx[D];
+  const int64_t c = shell_decode<T, D, I>(A.f, I(t), idx);
+  const GAcc<T, D> acc(A.f, c);
+  const PointVals<T> p = load_point<T, -1, EXACT>(A, c, true);
+  typename V2<typename T::R>::t pc;
+  typename T::R m2w;
+  return rk_apply<T>(A, c, site_rhs<T, D, ORDER, EXACT>(A.f, acc, idx, c, p.v, &pc, &m2w), p);
+}
+
+// The t-th of n boundary sites.
+template <class T, int D, int ORDER, bool EXACT, class I>
+__device__ __forceinline__ unsigned int boundary_site(const StageArgs<T>& A, int64_t t, int64_t n) {
+  using R = typename T::R;
+  using C2 = typename V2<R>::t;
+  const Field<T>& f = A.f;
+  if (t >= n) return 0u;
+  int idx[D];
+  const int64_t b = boundary_decode<T, D, I>(f, I(t), idx);
+  const PointVals<T> p = load_point<T, -1, EXACT>(A, b, true);
+  C2 Fb = {R(0), R(0)};
+  if (f.bc == BC_MSD) {   // see serve_walls
+    const C2 pb = ld2<R>(f.in, b);
+    int64_t c = 0;
+#pragma unroll
+    for (int k = 0; k < D; ++k) {
+      idx[k] = min(max(idx[k], 1), f.n[k] - 2);
+      c += idx[k] * f.st[k];
+    }
+    const GAcc<T, D> acc(f, c);
+    C2 pc;
+    R m2w;
+    const C2 F = site_rhs<T, D, ORDER, EXACT>(f, acc, idx, c, ldv<R>(EXACT ? A.Vs : f.V, c), &pc, &m2w);
+    const R m2 = EXACT ? m2w : norm2(pc);
+    R theta = R(0);
+    if (EXACT ? m2 > R(0) : m2 > f.tiny) theta = fma(F.y, pc.x, -(F.x * pc.y)) / m2;
+    Fb = {-theta * pb.y, theta * pb.x};
+  } else if (f.bc == BC_L0) {
+    const C2 pb = ld2<R>(f.in, b);
+    const R Nb = fma(EXACT ? f.sG : f.s, norm2(pb), -p.v);
+    Fb = {-Nb * pb.y, Nb * pb.x};
+  }
+  return rk_apply<T>(A, b, Fb, p);
+}
+
 // Blocks [0, b1): the n1 deep sites; [b1, b2): the n2 shell sites; the rest: the n3 boundary sites.
 template <class T, int D, int ORDER, bool EXACT, class I>
 __global__ void __launch_bounds__(256) k_stage_split(const StageArgs<T> A, unsigned b1, unsigned b2, int64_t n1, int64_t n2,
@@ -79,12 +127,12 @@ __global__ void __launch_bounds__(256) k_stage_split(const StageArgs<T> A, unsig
   using C2 = typename V2<R>::t;
   const Field<T>& f = A.f;
   unsigned int ex = 0;
-  int idx[D];
   grid_launch_dependents();
   grid_wait();
   if (blockIdx.x < b1) {
     const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (t < n1) {
+      int idx[D];
       I rem = I(t);
       int64_t c = 0;
 #pragma unroll
@@ -104,44 +152,9 @@ __global__ void __launch_bounds__(256) k_stage_split(const StageArgs<T> A, unsig
       ex = rk_apply<T>(A, c, {-fma(N, pc.y, aL.y), fma(N, pc.x, aL.x)}, p);
     }
   } else if (blockIdx.x < b2) {
-    const int64_t t = (int64_t)(blockIdx.x - b1) * blockDim.x + threadIdx.x;
-    if (t < n2) {
-      const int64_t c = shell_decode<T, D, I>(f, I(t), idx);
-      const GAcc<T, D> acc(f, c);
-      const PointVals<T> p = load_point<T, -1, EXACT>(A, c, true);
-      C2 pc;
-      R m2w;
-      ex = rk_apply<T>(A, c, site_rhs<T, D, ORDER, EXACT>(f, acc, idx, c, p.v, &pc, &m2w), p);
-    }
+    ex = shell_site<T, D, ORDER, EXACT, I>(A, (int64_t)(blockIdx.x - b1) * blockDim.x + threadIdx.x, n2);
   } else {
-    const int64_t t = (int64_t)(blockIdx.x - b2) * blockDim.x + threadIdx.x;
-    if (t < n3) {
-      const int64_t b = boundary_decode<T, D, I>(f, I(t), idx);
-      const PointVals<T> p = load_point<T, -1, EXACT>(A, b, true);
-      C2 Fb = {R(0), R(0)};
-      if (f.bc == BC_MSD) {   // see serve_walls
-        const C2 pb = ld2<R>(f.in, b);
-        int64_t c = 0;
-#pragma unroll
-        for (int k = 0; k < D; ++k) {
-          idx[k] = min(max(idx[k], 1), f.n[k] - 2);
-          c += idx[k] * f.st[k];
-        }
-        const GAcc<T, D> acc(f, c);
-        C2 pc;
-        R m2w;
-        const C2 F = site_rhs<T, D, ORDER, EXACT>(f, acc, idx, c, ldv<R>(EXACT ? A.Vs : f.V, c), &pc, &m2w);
-        const R m2 = EXACT ? m2w : norm2(pc);
-        R theta = R(0);
-        if (EXACT ? m2 > R(0) : m2 > f.tiny) theta = fma(F.y, pc.x, -(F.x * pc.y)) / m2;
-        Fb = {-theta * pb.y, theta * pb.x};
-      } else if (f.bc == BC_L0) {
-        const C2 pb = ld2<R>(f.in, b);
-        const R Nb = fma(EXACT ? f.sG : f.s, norm2(pb), -p.v);
-        Fb = {-Nb * pb.y, Nb * pb.x};
-      }
-      ex = rk_apply<T>(A, b, Fb, p);
-    }
+    ex = boundary_site<T, D, ORDER, EXACT, I>(A, (int64_t)(blockIdx.x - b2) * blockDim.x + threadIdx.x, n3);
   }
   if (A.emax) emax_commit(A.emax, ex);
 }
