@@ -121,7 +121,8 @@ bool layout_batch(int nruns, const nlse_run_desc* runs, int tile_cfg, BatchLayou
   L->field_off.resize(nruns);
   for (int r = 0; r < nruns; ++r) {
     L->field_off[r] = off;
-    off = al(off + sizeof(float2) * size_t(runs[r].n[0] * runs[r].n[1]));
+    // a run's share is at least two arrays, as callers may rely on; the copy takes the first
+    off = al(off + 2 * sizeof(float2) * size_t(runs[r].n[0] * runs[r].n[1]));
   }
   L->total = al(off);
   return true;

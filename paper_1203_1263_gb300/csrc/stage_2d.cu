@@ -1,5 +1,5 @@
-// 2D stage launches: variant 0 = generic kernel, 1 = halo-tiled kernel,
-// 2 / 3 = tiled / generic with the exact-sum stencil (FP64 only).
+// 2D stage launches: variant 0 = one thread per site, 1 = halo-tiled kernel,
+// 2 / 3 = tiled / per site with the exact-sum stencil (FP64 only).
 #include "stage_generic.cuh"
 #include "stage_split.cuh"
 #include "stage_tiled.cuh"
@@ -12,7 +12,8 @@ cudaError_t launch_stage(const StageArgs<T>& A, const LaunchCfg& L, cudaStream_t
   const int variant = (!fp64 && L.variant >= 2) ? L.variant - 2 : L.variant;   // exact sums are FP64 only
   const bool exact = variant >= 2;
   const bool periodic = A.f.bc == BC_PERIODIC;
-  if (variant == 0 || variant == 3) {
+  // (the FP32 forms' tiled steps are step2d.cu's; here their one thread per site, and nlse_rhs)
+  if (!fp64 || variant == 0 || variant == 3) {
     if (periodic) {
       if constexpr (fp64) if (exact) return launch_generic_periodic<T, D, ORDER, true>(A, stream);
       return launch_generic_periodic<T, D, ORDER>(A, stream);
@@ -21,19 +22,22 @@ cudaError_t launch_stage(const StageArgs<T>& A, const LaunchCfg& L, cudaStream_t
     return launch_split<T, D, ORDER>(A, stream, true, true);
   }
   // tiled: deep interior + the wall shell (periodic grids: the two layers at each end of each axis)
-  auto deep = [&](cudaStream_t st) -> cudaError_t {
-    if constexpr (fp64) if (exact) return launch2d_tiled<T, ORDER, true>(A, L.tile_cfg, st);
-    return launch2d_tiled<T, ORDER>(A, L.tile_cfg, st);
-  };
-  auto shell = [&](cudaStream_t st) -> cudaError_t {
-    if (periodic) {
-      if constexpr (fp64) if (exact) return launch_shell_periodic<T, D, ORDER, true>(A, st);
-      return launch_shell_periodic<T, D, ORDER>(A, st);
-    }
-    if constexpr (fp64) if (exact) return launch_split<T, D, ORDER, true>(A, st, false, false);
-    return launch_split<T, D, ORDER>(A, st, false, false);
-  };
-  return launch_deep_and_shell(L, stream, has_deep(D, A.f.m), deep, shell);
+  if constexpr (fp64) {
+    auto deep = [&](cudaStream_t st) -> cudaError_t {
+      if (exact) return launch2d_tiled<T, ORDER, true>(A, L.tile_cfg, st);
+      return launch2d_tiled<T, ORDER>(A, L.tile_cfg, st);
+    };
+    auto shell = [&](cudaStream_t st) -> cudaError_t {
+      if (periodic) {
+        if (exact) return launch_shell_periodic<T, D, ORDER, true>(A, st);
+        return launch_shell_periodic<T, D, ORDER>(A, st);
+      }
+      if (exact) return launch_split<T, D, ORDER, true>(A, st, false, false);
+      return launch_split<T, D, ORDER>(A, st, false, false);
+    };
+    return launch_deep_and_shell(L, stream, has_deep(D, A.f.m), deep, shell);
+  }
+  return cudaErrorInvalidValue;
 }
 
 #define INST(T, O) template cudaError_t launch_stage<T, 2, O>(const StageArgs<T>&, const LaunchCfg&, cudaStream_t);

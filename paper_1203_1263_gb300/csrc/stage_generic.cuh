@@ -1,8 +1,6 @@
-// Generic stage kernel: one thread per interior site, all reads through the
-// read-only cache.  Simple and dimension-agnostic; it is the correctness
-// baseline that the tiled kernels are checked against, the kernel used for
-// 1D grids, and the default for 3D grids too small to fill the GPU with the
-// z-marching kernel's tiles (latency, not bandwidth, bounds those).
+// Per-site kernels that read through the read-only cache: one thread per
+// interior site (1D lines; planes and grids take stage_split.cuh), the periodic
+// grids' sites and shells, and the enumeration of the sites next to the walls.
 #pragma once
 #include "nlse_device.cuh"
 
@@ -35,9 +33,8 @@ __global__ void __launch_bounds__(256) k_stage_generic(const StageArgs<T> A) {
 // ---------------------------------------------------------------------------
 // Wall shell: the interior sites within one cell of a wall (some index equal
 // to 1 or N-2).  The tiled kernels compute only the deep interior (every
-// index in [2, N-3]), where the stencil never reaches past a wall and no
-// boundary site is served; the shell kernel computes the rest with the
-// generic per-site code.  Sites are enumerated exactly, face by face: with
+// index in [2, N-3]), where the stencil never reaches past a wall; the rest are
+// the shell's.  Sites are enumerated exactly, face by face: with
 // interior extents a_k = N_k - 2, deep extents d_k = max(a_k - 2, 0) and
 // c_k = a_k - d_k (2, or 1 when a_k == 1), the shell is
 //   {i_0 in the c_0 outer layers} x a_1 x a_2
@@ -118,19 +115,6 @@ inline bool has_deep(int D, const int* m) {
   return true;
 }
 
-template <class T, int D, int ORDER, bool EXACT, class I>
-__global__ void __launch_bounds__(256) k_stage_shell(const StageArgs<T> A, int64_t nshell) {
-  const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  unsigned int ex = 0;
-  if (t < nshell) {
-    int idx[D];
-    const int64_t c = shell_decode<T, D, I>(A.f, I(t), idx);
-    const GAcc<T, D> acc(A.f, c);
-    ex = process_site<T, D, ORDER, EXACT>(A, acc, idx, c);
-  }
-  if (A.emax) emax_commit(A.emax, ex);
-}
-
 // CTA size of the one-thread-per-site kernels: 256 threads, halved (down to
 // one warp) while the grid would give fewer than two CTAs per SM.  On small
 // grids this spreads the sites over all SMs, which matters most on the FP64
@@ -180,17 +164,6 @@ __global__ void __launch_bounds__(256) k_stage_generic_periodic(const StageArgs<
     ex = process_site_periodic<T, D, ORDER, EXACT>(A, idx, c);
   }
   if (A.emax) emax_commit(A.emax, ex);
-}
-
-template <class T, int D, int ORDER, bool EXACT = false>
-cudaError_t launch_shell(const StageArgs<T>& A, cudaStream_t stream) {
-  const int64_t ns = shell_count(D, A.f.m);
-  if (ns <= 0) return cudaSuccess;
-  const int threads = site_kernel_threads(ns);
-  const dim3 grid((unsigned)((ns + threads - 1) / threads));
-  if (A.f.ninterior < (int64_t(1) << 31)) k_stage_shell<T, D, ORDER, EXACT, uint32_t><<<grid, threads, 0, stream>>>(A, ns);
-  else k_stage_shell<T, D, ORDER, EXACT, uint64_t><<<grid, threads, 0, stream>>>(A, ns);
-  return cudaGetLastError();
 }
 
 template <class T, int D, int ORDER, bool EXACT = false>

@@ -33,6 +33,7 @@
 #include <vector>
 
 #include "../../include/nlse.h"
+#include "wide_sum.cuh"
 
 namespace nlse {
 void record_last_error(const char* msg);
@@ -510,6 +511,8 @@ __global__ void __launch_bounds__(WM * WN * 32) k_conv_fast(const ConvArgs a, co
 struct TcArgs {
   Geo g;
   int cg;              // gathered channels = K per tap (multiple of 16)
+  int slices;          // 16-channel K slices of a tap that hold channels; the rest are the padding's zeros, whose
+                       //   products add nothing (the network's two ends: 1 of 4)
   int nout;            // output channels = N (multiple of 16, <= 256)
   int dil;
   const bf16* act;     // gathered activation, channels-last [P][cg]
@@ -769,11 +772,12 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_conv_tc(const TcArgs a, const
             const uint64_t bd0 = sdesc_sw128(sm_base + (uint32_t)(t * nout * 128));
 #pragma unroll
             for (int kk = 0; kk < 4; ++kk)
-              tc_mma(tmem + (uint32_t)(st * nout), ad0 + 2u * kk, bd0 + 2u * kk, idesc, (t | kk) != 0);
+              if (kk < a.slices)
+                tc_mma(tmem + (uint32_t)(st * nout), ad0 + 2u * kk, bd0 + 2u * kk, idesc, (t | kk) != 0);
           } else {
             const uint32_t aoff = a0 + (uint32_t)(((1 + sy) * RW + d + sx * d) * 16);
             const uint32_t boff = sm_base + (uint32_t)(t * planes * nout * 16);
-            for (int kk = 0; kk < planes / 2; ++kk) {
+            for (int kk = 0; kk < a.slices; ++kk) {
               const uint64_t ad = sdesc(aoff + 2 * kk * LBOA, LBOA, 128);
               const uint64_t bd = sdesc(boff + 2 * kk * nout * 16, nout * 16, 128);
               tc_mma(tmem + (uint32_t)(st * nout), ad, bd, idesc, (t | kk) != 0);
@@ -827,17 +831,20 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_conv_tc(const TcArgs a, const
         if (!ok) continue;
         for (int c1 = 0; c1 < nc; c1 += 8) {
           const int cc = c0 + c1;
+          if (MODE == MODE_FWD && a.z) {   // the network's output: two channels (a sector) of the padded ones
+            if (cc == 0) {
+              float4* zd = reinterpret_cast<float4*>(a.z + p * nout);
+              zd[0] = make_float4(v[0] + sbias[0], v[1] + sbias[1], v[2] + sbias[2], v[3] + sbias[3]);
+              zd[1] = make_float4(v[4] + sbias[4], v[5] + sbias[5], v[6] + sbias[6], v[7] + sbias[7]);
+            }
+            break;
+          }
           if (MODE == MODE_FWD) {
             float zz[8], sg[8];
 #pragma unroll
             for (int e = 0; e < 8; ++e) {
               zz[e] = v[c1 + e] + sbias[cc + e];
               sg[e] = __fdividef(1.f, 1.f + __expf(-zz[e]));   // sigmoid, shared by silu and silu'
-            }
-            if (a.z) {
-              float4* zd = reinterpret_cast<float4*>(a.z + p * nout + cc);
-              zd[0] = make_float4(zz[0], zz[1], zz[2], zz[3]);
-              zd[1] = make_float4(zz[4], zz[5], zz[6], zz[7]);
             }
             if (a.h) {
               __nv_bfloat162 hb[4];
@@ -1048,8 +1055,9 @@ __global__ void __launch_bounds__(kWgThreads, 1) k_wgrad_tc(const WgArgs a, cons
 __global__ void k_sum_parts(const float* __restrict__ part, int nparts, float* __restrict__ dw,
                             float* __restrict__ db) {
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < kWgPart; i += (int64_t)gridDim.x * blockDim.x) {
-    float acc = 0.f;
-    for (int b = 0; b < nparts; ++b) acc += part[(int64_t)b * kWgPart + i];
+    float acc = 0.f;   // in order; sixteen loads in flight (13.5 us with the compiler's four)
+#pragma unroll 16
+    for (int b = 0; b < nparts; ++b) acc += __ldg(part + (int64_t)b * kWgPart + i);
     if (i < 64 * 9 * 64) dw[i] += acc;
     else db[i - 64 * 9 * 64] += acc;
   }
@@ -1067,29 +1075,38 @@ __global__ void k_transpose_w(const bf16* __restrict__ w, bf16* __restrict__ wt,
 // Per-state sums of |psi_in|^2 and |psi_out|^2 (FP64): grid (kMassBlocks, nb), 256 threads;
 // partial sums to part[(n * kMassBlocks + block) * 2 + {0, 1}].
 constexpr int kMassBlocks = 32;
-__global__ void k_state_mass(const float2* __restrict__ in, const float2* __restrict__ out, int64_t HW,
-                             double* __restrict__ part) {
-  __shared__ double r0[256], r1[256];
+__global__ void __launch_bounds__(256) k_state_mass(const float2* __restrict__ in, const float2* __restrict__ out,
+                                                    int64_t HW, double* __restrict__ part) {
+  // sums of squares of FP32 values, exact on the integer pipe (27 us for 16 256^2 states in FP64)
   const int64_t base = (int64_t)blockIdx.y * HW;
-  double a = 0.0, b = 0.0;
+  nlse::WideSum a, b;
+  bool oka = true, okb = true;
   for (int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; p < HW; p += (int64_t)gridDim.x * blockDim.x) {
     const float2 u = in[base + p], v = out[base + p];
-    a += double(u.x) * u.x + double(u.y) * u.y;
-    b += double(v.x) * v.x + double(v.y) * v.y;
-  }
-  r0[threadIdx.x] = a;
-  r1[threadIdx.x] = b;
-  __syncthreads();
-  for (int o = blockDim.x / 2; o > 0; o >>= 1) {
-    if ((int)threadIdx.x < o) {
-      r0[threadIdx.x] += r0[threadIdx.x + o];
-      r1[threadIdx.x] += r1[threadIdx.x + o];
+    if (isfinite(u.x) && isfinite(u.y)) {
+      a.add_square(u.x);
+      a.add_square(u.y);
+    } else {
+      oka = false;
     }
-    __syncthreads();
+    if (isfinite(v.x) && isfinite(v.y)) {
+      b.add_square(v.x);
+      b.add_square(v.y);
+    } else {
+      okb = false;
+    }
   }
+  oka = __syncthreads_and(oka);
+  okb = __syncthreads_and(okb);
+  a = nlse::block_wide_sum<256>(a);
+  b = nlse::block_wide_sum<256>(b);
   if (threadIdx.x == 0) {
-    part[((int64_t)blockIdx.y * kMassBlocks + blockIdx.x) * 2] = r0[0];
-    part[((int64_t)blockIdx.y * kMassBlocks + blockIdx.x) * 2 + 1] = r1[0];
+    double sa, sb, c;
+    const double nan = __longlong_as_double(0x7FF8000000000000ll);
+    a.pair(&sa, &c);
+    b.pair(&sb, &c);
+    part[((int64_t)blockIdx.y * kMassBlocks + blockIdx.x) * 2] = oka ? sa : nan;
+    part[((int64_t)blockIdx.y * kMassBlocks + blockIdx.x) * 2 + 1] = okb ? sb : nan;
   }
 }
 
@@ -1218,11 +1235,13 @@ constexpr int kIn = 4;
 
 // complex state -> pc-channel BF16 input (the kIn features, zeros); one thread per 16-byte chunk
 __global__ void k_pack_input(const float2* __restrict__ psi, int64_t P, int pc, bf16* __restrict__ h) {
-  const int cpp = pc / 8;
+  // a site's first two 8-channel chunks (a memory sector); the other padding channels stay as created, zero
+  const int cpp = pc / 8, w = cpp < 2 ? cpp : 2;
   uint4* dst = reinterpret_cast<uint4*>(h);
-  for (int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; q < P * cpp; q += (int64_t)gridDim.x * blockDim.x) {
+  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < P * w; i += (int64_t)gridDim.x * blockDim.x) {
+    const int64_t q = (i / w) * cpp + i % w;
     uint4 v = make_uint4(0u, 0u, 0u, 0u);
-    if (q % cpp == 0) {   // channels 0..3: hi parts, 4..7: lo parts of the kIn features
+    if (i % w == 0) {   // channels 0..3: hi parts, 4..7: lo parts of the kIn features
       const float2 z = psi[q / cpp];
       const float r = fmaf(z.x, z.x, z.y * z.y);
       const float f[4] = {z.x, z.y, r * z.x, r * z.y};
@@ -1308,40 +1327,53 @@ __global__ void k_residual(const float2* __restrict__ psi, const float* __restri
 // output gradient of the last layer (pc-channel rows, channels 2.. zero); one
 // thread per 16-byte chunk of that gradient
 // With coef (the mass term, k_mass_coef), coef[p / HW] psi_out[p] is added to the gradient.
-__global__ void k_mse(const float2* __restrict__ psi, const float* __restrict__ y, const float2* __restrict__ target,
-                      int64_t P, int pc, bf16* __restrict__ dz, double* __restrict__ loss_acc,
-                      const double* __restrict__ coef, int64_t HW) {
-  __shared__ double red[256];
-  double s = 0.0;
+__global__ void __launch_bounds__(256) k_mse(const float2* __restrict__ psi, const float* __restrict__ y,
+                                             const float2* __restrict__ target, int64_t P, int pc, bf16* __restrict__ dz,
+                                             double* __restrict__ loss_acc, const double* __restrict__ coef, int64_t HW) {
+  // a warp per 32 sites, a lane per site for the arithmetic (the squares exact on the integer pipe), then the whole
+  // warp for the sites' pc / 8 chunks in memory order (96 us with a thread per chunk and FP64 sums in one lane of 8)
+  nlse::WideSum sum;
+  bool ok = true;
   const float scale = 2.f / float(2 * P);
-  const int cpp = pc / 8;
+  const int cpp = pc / 8, lane = threadIdx.x & 31;
   uint4* dst = reinterpret_cast<uint4*>(dz);
-  for (int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; q < P * cpp; q += (int64_t)gridDim.x * blockDim.x) {
-    uint4 v = make_uint4(0u, 0u, 0u, 0u);
-    if (q % cpp == 0) {
-      const int64_t p = q / cpp;
+  const int64_t warps = (int64_t)gridDim.x * (blockDim.x / 32);
+  for (int64_t p0 = 32 * ((int64_t)blockIdx.x * (blockDim.x / 32) + (threadIdx.x >> 5)); p0 < P; p0 += 32 * warps) {
+    const int64_t p = p0 + lane;
+    uint32_t g = 0;
+    if (p < P) {
       const float2 u = psi[p], t = target[p];
       const float2 d = *reinterpret_cast<const float2*>(y + p * pc);
       const float ex = u.x + d.x - t.x, ey = u.y + d.y - t.y;
-      s += double(ex) * ex + double(ey) * ey;
+      if (isfinite(ex) && isfinite(ey)) {
+        sum.add_square(ex);
+        sum.add_square(ey);
+      } else {
+        ok = false;
+      }
       float gx = scale * ex, gy = scale * ey;
       if (coef) {
         const float cb = float(coef[p / HW]);
         gx = fmaf(cb, u.x + d.x, gx);
         gy = fmaf(cb, u.y + d.y, gy);
       }
-      const __nv_bfloat162 g = __floats2bfloat162_rn(gx, gy);
-      v.x = *reinterpret_cast<const uint32_t*>(&g);
+      const __nv_bfloat162 gb = __floats2bfloat162_rn(gx, gy);
+      g = *reinterpret_cast<const uint32_t*>(&gb);
     }
-    dst[q] = v;
+    const int n = int(P - p0 < 32 ? P - p0 : 32) * cpp;
+    for (int c0 = 0; c0 < 32 * cpp; c0 += 32) {
+      const int c = c0 + lane, site = c / cpp;
+      const uint32_t gs = __shfl_sync(0xffffffffu, g, site & 31);
+      if (c < n) dst[p0 * cpp + c] = make_uint4(c - site * cpp == 0 ? gs : 0u, 0u, 0u, 0u);
+    }
   }
-  red[threadIdx.x] = s;
-  __syncthreads();
-  for (int o = blockDim.x / 2; o > 0; o >>= 1) {
-    if ((int)threadIdx.x < o) red[threadIdx.x] += red[threadIdx.x + o];
-    __syncthreads();
+  ok = __syncthreads_and(ok);
+  sum = nlse::block_wide_sum<256>(sum);
+  if (threadIdx.x == 0) {
+    double a, c;
+    sum.pair(&a, &c);
+    atomicAdd(loss_acc, (ok ? a : __longlong_as_double(0x7FF8000000000000ll)) / double(2 * P));
   }
-  if (threadIdx.x == 0) atomicAdd(loss_acc, red[0] / double(2 * P));
 }
 
 // db[c] += sum over pixels of dz[p * stride + c] for c < creal (stride <= 256;
@@ -1620,6 +1652,9 @@ cudaError_t conv(const nlse_sur* s, int mode, int l, int nb, const bf16* x, cons
       memset(&t, 0, sizeof(t));
       t.g = a.g;
       t.cg = cg;
+      t.slices = cg / 16;
+      if (mode == MODE_FWD && l == 0) t.slices = 1;                     // the packed features, hi and lo parts
+      if (mode == MODE_BWD_DATA && l == s->L - 1) t.slices = 1;         // the two output channels
       t.nout = nout;
       t.dil = a.dil;
       t.act = mode == MODE_FWD ? x : dz;
@@ -1716,7 +1751,7 @@ cudaError_t refresh_bf16(const nlse_sur* s, bool copy) {
 // training = false (inference): the inner layers keep only silu(z); true: also silu'(z)
 cudaError_t forward(const nlse_sur* s, int nb, const float2* psi_in, bool training) {
   const int64_t P = (int64_t)nb * s->H * s->W;
-  k_pack_input<<<grid1d(P * s->pc / 8), 256, 0, s->stream>>>(psi_in, P, s->pc, s->hin);
+  k_pack_input<<<grid1d(P * (s->pc / 8 < 2 ? 1 : 2)), 256, 0, s->stream>>>(psi_in, P, s->pc, s->hin);
   cudaError_t e = cudaGetLastError();
   const bf16* x = s->hin;
   for (int l = 0; l < s->L && e == cudaSuccess; ++l) {
@@ -1742,7 +1777,7 @@ cudaError_t backward(const nlse_sur* s, int nb, const float2* psi_in, const floa
                                                                              s->mass_part);
     k_mass_coef<<<(nb + 31) / 32, 32, 0, s->stream>>>(s->mass_part, nb, s->mass_weight, s->mstat, s->loss);
   }
-  k_mse<<<grid1d(P * s->pc / 8), 256, 0, s->stream>>>(psi_in, s->y, target, P, s->pc, dz, s->loss,
+  k_mse<<<grid1d(P), 256, 0, s->stream>>>(psi_in, s->y, target, P, s->pc, dz, s->loss,
                                                       s->mass_weight > 0.0 ? s->mstat : nullptr, HW);
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
   for (int l = s->L - 1; l >= 0 && e == cudaSuccess; --l) {
@@ -1878,6 +1913,7 @@ int nlse_sur_create(nlse_sur_t* out, int H, int W, int channels, int layers, con
   if (e == cudaSuccess) e = cudaMemsetAsync(s->err, 0, sizeof(int), s->stream);
   if (e == cudaSuccess) e = cudaMemsetAsync(s->m1, 0, s->nparam * 4, s->stream);
   if (e == cudaSuccess) e = cudaMemsetAsync(s->m2, 0, s->nparam * 4, s->stream);
+  if (e == cudaSuccess) e = cudaMemsetAsync(s->hin, 0, (size_t)P * pc * 2, s->stream);   // its padding channels
   if (e == cudaSuccess) e = refresh_bf16(s, true);
   if (e != cudaSuccess) {
     delete s;
