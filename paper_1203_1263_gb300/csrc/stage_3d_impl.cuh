@@ -7,6 +7,7 @@
 #pragma once
 #include "stage_generic.cuh"
 #include "stage_march.cuh"
+#include "stage_pair.cuh"
 #include "stage_slab.cuh"
 #include "stage_split.cuh"
 #include "stage_tiled.cuh"
@@ -26,6 +27,11 @@ cudaError_t launch_stage(const StageArgs<T>& A, const LaunchCfg& L, cudaStream_t
       return launch_generic_periodic<T, D, ORDER>(A, stream);
     }
     if constexpr (fp64) if (exact) return launch_split<T, D, ORDER, true>(A, stream, true, true);
+    if constexpr (std::is_same<T, P64>::value) {
+      // see the figures in stage_pair.cuh
+      const int64_t sites = (int64_t)A.f.n[0] * A.f.n[1] * A.f.n[2];
+      if (sites <= (ORDER == 4 ? 600000 : 16384)) return launch_pair<ORDER>(A, stream);
+    }
     return launch_split<T, D, ORDER>(A, stream, true, true);
   }
   if constexpr (!fp64) {
