@@ -14,8 +14,11 @@ constexpr int kMaxReduceBlocks = 1024;
 
 // A kernel that may start while the kernel before it in the stream still runs (programmatic dependent
 // launch): it calls grid_wait() before it touches anything an earlier kernel wrote or still reads, and
-// grid_launch_dependents() where the next kernel may start.  On a dependency that is not such a kernel
-// this is an ordinary launch.
+// grid_launch_dependents() where the next kernel may start (otherwise as its CTAs end).  The early start pays
+// where a CTA fills an SM or CTAs are many; where a grid is less than a wave of small CTAs, the next
+// kernel's pile up on the SMs that are done first (64^3 FP32 columns 26.7 against 21.1 us per step without, 46^3
+// one thread per site 20.2 and 16.6, 512^2 FP32 12.8 and 10.9; but 256^2 FP64 21.7 and 22.4, a batch 594
+// and 602).  On a dependency that is not such a kernel this is an ordinary launch.
 __device__ __forceinline__ void grid_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void grid_launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 

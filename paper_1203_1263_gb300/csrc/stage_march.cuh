@@ -29,7 +29,6 @@ template <class T, int ORDER, int S>
 __global__ void __launch_bounds__(256, 4) k_stage3d_march(const StageArgs<T> A, int ntx, int nty, int zc, unsigned b1,
                                                           unsigned b2, unsigned b3, int64_t n2, int64_t n3, bool walls_first) {
   const Field<T>& f = A.f;
-  grid_launch_dependents();
   grid_wait();
   unsigned bi = blockIdx.x;
   if (walls_first) bi = bi < b3 - b1 ? bi + b1 : bi - (b3 - b1);

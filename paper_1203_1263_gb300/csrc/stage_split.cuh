@@ -10,7 +10,8 @@
 // evaluates F at its interior neighbour once more (MSD; Eq. msd) instead of
 // waiting for that site's thread.  The arithmetic is site_rhs, serve_walls and
 // rk_apply as everywhere, so results are bit-for-bit those of one thread per
-// interior site (21^3 FP64 2SHOC MSD: 38.6 against 60.5 us per step).
+// interior site (21^3 FP64 2SHOC MSD: 37.7 against 60.5 us per step; small FP64
+// grids: stage_pair.cuh).
 #pragma once
 #include "nlse_internal.h"
 #include "stage_generic.cuh"
@@ -127,7 +128,6 @@ __global__ void __launch_bounds__(256) k_stage_split(const StageArgs<T> A, unsig
   using C2 = typename V2<R>::t;
   const Field<T>& f = A.f;
   unsigned int ex = 0;
-  grid_launch_dependents();
   grid_wait();
   if (blockIdx.x < b1) {
     const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;

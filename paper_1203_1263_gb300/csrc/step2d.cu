@@ -9,7 +9,6 @@ __global__ void __launch_bounds__(NT, MINB) k_step2d(const __grid_constant__ Ste
   extern __shared__ __align__(16) unsigned char step2_smem[];
   Step2Tile<T, ORDER, TX, NT, RY> tile(A, ty, blockIdx.x % ntx, blockIdx.x / ntx, step2_smem);
   // launched while the step before still runs: V is not its output, Psi^n is
-  grid_launch_dependents();
   tile.load_potential();
   grid_wait();
   tile.run();
