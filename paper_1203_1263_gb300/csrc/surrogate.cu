@@ -34,6 +34,7 @@
 
 #include "../../include/nlse.h"
 #include "wide_sum.cuh"
+#include <algorithm>
 
 namespace nlse {
 void record_last_error(const char* msg);
@@ -1055,9 +1056,15 @@ __global__ void __launch_bounds__(kWgThreads, 1) k_wgrad_tc(const WgArgs a, cons
 __global__ void k_sum_parts(const float* __restrict__ part, int nparts, float* __restrict__ dw,
                             float* __restrict__ db) {
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < kWgPart; i += (int64_t)gridDim.x * blockDim.x) {
-    float acc = 0.f;   // in order; sixteen loads in flight (13.5 us with the compiler's four)
-#pragma unroll 16
-    for (int b = 0; b < nparts; ++b) acc += __ldg(part + (int64_t)b * kWgPart + i);
+    // in order, 32 loads in flight; the last group's missing parts add 0 (13.5 us with the compiler's four in flight)
+    float acc = 0.f;
+    for (int b = 0; b < nparts; b += 32) {
+      float v[32];
+#pragma unroll
+      for (int j = 0; j < 32; ++j) v[j] = b + j < nparts ? __ldg(part + (int64_t)(b + j) * kWgPart + i) : 0.f;
+#pragma unroll
+      for (int j = 0; j < 32; ++j) acc += v[j];
+    }
     if (i < 64 * 9 * 64) dw[i] += acc;
     else db[i - 64 * 9 * 64] += acc;
   }
@@ -1081,8 +1088,19 @@ __global__ void __launch_bounds__(256) k_state_mass(const float2* __restrict__ i
   const int64_t base = (int64_t)blockIdx.y * HW;
   nlse::WideSum a, b;
   bool oka = true, okb = true;
-  for (int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; p < HW; p += (int64_t)gridDim.x * blockDim.x) {
-    const float2 u = in[base + p], v = out[base + p];
+  const int64_t step = (int64_t)gridDim.x * blockDim.x;
+  int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  float2 u1 = {0.f, 0.f}, v1 = u1;   // the next site's values, requested a site ahead
+  if (p < HW) {
+    u1 = in[base + p];
+    v1 = out[base + p];
+  }
+  for (; p < HW; p += step) {
+    const float2 u = u1, v = v1;
+    if (p + step < HW) {
+      u1 = in[base + p + step];
+      v1 = out[base + p + step];
+    }
     if (isfinite(u.x) && isfinite(u.y)) {
       a.add_square(u.x);
       a.add_square(u.y);
@@ -1098,15 +1116,25 @@ __global__ void __launch_bounds__(256) k_state_mass(const float2* __restrict__ i
   }
   oka = __syncthreads_and(oka);
   okb = __syncthreads_and(okb);
-  a = nlse::block_wide_sum<256>(a);
-  b = nlse::block_wide_sum<256>(b);
-  if (threadIdx.x == 0) {
-    double sa, sb, c;
-    const double nan = __longlong_as_double(0x7FF8000000000000ll);
-    a.pair(&sa, &c);
-    b.pair(&sb, &c);
-    part[((int64_t)blockIdx.y * kMassBlocks + blockIdx.x) * 2] = oka ? sa : nan;
-    part[((int64_t)blockIdx.y * kMassBlocks + blockIdx.x) * 2 + 1] = okb ? sb : nan;
+  // lane 0 of every warp holds the warp's sums; warp 0 finishes the first, warp 1 the second
+  __shared__ unsigned long long sl[2][8];
+  __shared__ long long sh[2][8];
+  __shared__ int se[2][8];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  a = nlse::warp_wide_sum(a);
+  b = nlse::warp_wide_sum(b);
+  if (lane == 0) {
+    sl[0][warp] = a.lo; sh[0][warp] = a.hi; se[0][warp] = a.E;
+    sl[1][warp] = b.lo; sh[1][warp] = b.hi; se[1][warp] = b.E;
+  }
+  __syncthreads();
+  if (warp < 2) {
+    a = nlse::WideSum();
+    if (lane < 8) { a.lo = sl[warp][lane]; a.hi = sh[warp][lane]; a.E = se[warp][lane]; }
+    a = nlse::warp_wide_sum(a);
+    if (lane == 0)
+      part[((int64_t)blockIdx.y * kMassBlocks + blockIdx.x) * 2 + warp] =
+          (warp == 0 ? oka : okb) ? a.value() : __longlong_as_double(0x7FF8000000000000ll);
   }
 }
 
@@ -1370,9 +1398,7 @@ __global__ void __launch_bounds__(256) k_mse(const float2* __restrict__ psi, con
   ok = __syncthreads_and(ok);
   sum = nlse::block_wide_sum<256>(sum);
   if (threadIdx.x == 0) {
-    double a, c;
-    sum.pair(&a, &c);
-    atomicAdd(loss_acc, (ok ? a : __longlong_as_double(0x7FF8000000000000ll)) / double(2 * P));
+    atomicAdd(loss_acc, (ok ? sum.value() : __longlong_as_double(0x7FF8000000000000ll)) / double(2 * P));
   }
 }
 
@@ -1696,7 +1722,9 @@ cudaError_t conv(const nlse_sur* s, int mode, int l, int nb, const bf16* x, cons
     w.part = s->wgpart;
     w.err = s->err;
     w.spin_limit = 1ll << 24;
-    const int grid = s->num_sms < kWgMaxParts ? s->num_sms : kWgMaxParts;
+    // a CTA without a tile would only write zeros for k_sum_parts to read
+    const int64_t tiles = (int64_t)nb * s->H * ((s->W + 127) / 128);
+    const int grid = (int)std::min<int64_t>(tiles, std::min(s->num_sms, kWgMaxParts));
     k_wgrad_tc<<<grid, kWgThreads, kWgSmem, s->stream>>>(w, th, tz);
     k_sum_parts<<<grid1d(kWgPart), 256, 0, s->stream>>>(s->wgpart, grid, a.dw, layer_ops(s, l).db);
     if (bias_done) *bias_done = true;

@@ -70,6 +70,15 @@ struct WideSum {
     const unsigned int m = (u & 0x7FFFFFu) | (e ? 0x800000u : 0u);
     add((unsigned long long)m * m, 2 * (int(e ? e : 1) - 150) + 1075, false);
   }
+  // a non-negative total, rounded: one conversion and one scaling (pair() is some forty dependent FP64 instructions)
+  __device__ __forceinline__ double value() const {
+    const unsigned long long h = (unsigned long long)hi;
+    const int q = E - 1075 - kGuard;
+    if (h == 0) return ldexp(double(lo), q);
+    const int z = __clzll((long long)h), r = 64 - z;   // z >= 1
+    const unsigned long long top = (h << z) | (lo >> r);
+    return ldexp(double(top | ((lo << z) != 0 ? 1ull : 0ull)), q + r);   // 64 bits, the last one sticky
+  }
   // the total as a rounded sum and what the rounding left
   __device__ __forceinline__ void pair(double* s, double* c) const {
     const bool neg = hi < 0;
@@ -91,6 +100,21 @@ struct WideSum {
   }
 };
 
+// The sum over a warp, in lane 0: one exponent for all first, so that a level is two shuffles and a 128-bit add (pairs
+// rescaled at every level: 16 states of 64^2, two masses each, 4 us more).
+__device__ __forceinline__ WideSum warp_wide_sum(WideSum v) {
+  v.raise(__reduce_max_sync(0xffffffffu, v.E));
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    const unsigned long long l = __shfl_down_sync(0xffffffffu, v.lo, o);
+    const long long h = __shfl_down_sync(0xffffffffu, v.hi, o);   // lanes past the end add values nobody reads
+    const unsigned long long t = v.lo + l;
+    v.hi = (long long)((unsigned long long)v.hi + (unsigned long long)h + (t < l ? 1ull : 0ull));
+    v.lo = t;
+  }
+  return v;
+}
+
 // The sum over a block of THREADS threads, in thread 0.
 template <int THREADS>
 __device__ __forceinline__ WideSum block_wide_sum(WideSum v) {
@@ -98,23 +122,14 @@ __device__ __forceinline__ WideSum block_wide_sum(WideSum v) {
   __shared__ long long sh[THREADS / 32];
   __shared__ unsigned long long sl[THREADS / 32];
   __shared__ int se[THREADS / 32];
-  auto lanes = [&](int n) {
-    for (int o = n / 2; o > 0; o >>= 1) {
-      WideSum b;
-      b.lo = __shfl_down_sync(0xffffffffu, v.lo, o);
-      b.hi = __shfl_down_sync(0xffffffffu, v.hi, o);
-      b.E = __shfl_down_sync(0xffffffffu, v.E, o);
-      v.merge(b);   // lanes past the end add values nobody reads
-    }
-  };
-  lanes(32);
+  v = warp_wide_sum(v);
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   if (lane == 0) { sh[warp] = v.hi; sl[warp] = v.lo; se[warp] = v.E; }
   __syncthreads();
   if (warp == 0) {
     v = WideSum();
     if (lane < THREADS / 32) { v.hi = sh[lane]; v.lo = sl[lane]; v.E = se[lane]; }
-    lanes(THREADS / 32);
+    v = warp_wide_sum(v);
   }
   __syncthreads();   // the arrays may be used again
   return v;
