@@ -60,8 +60,8 @@ FP64_FLOPS_PER_SITE_STEP = 15 + 19 + 19 + 17
 CHUNK = 56   # steps per frame in the end-to-end measurement (the 87x87x203 run's chunk size)
 
 
-# Kernel launches per RK4 step of the 3D tiled path (every extent >= 7, x >= 10): per stage one
-# deep-interior kernel and three wall-slab kernels; the FP64 exact-sum form adds the one-thread kernel
+# Kernel launches per RK4 step of the 3D tiled path (every extent >= 7, x >= 10; the FP32 forms above
+# 3,000,000 sites): per stage one deep-interior kernel and three wall-slab kernels; the FP64 exact-sum form adds the one-thread kernel
 # that sets the next step's fixed-point scale.
 LAUNCHES_PER_STEP = {"c128": 17, "c64": 16, "c64_acc64": 16}
 
@@ -77,8 +77,8 @@ TRAFFIC_PER_STEP = {  # dtype -> (bytes per step, csrc hash of the capture)
 # The sources the 3D stage path (deep kernels, wall slabs, scale update, step loop) is built from.
 STAGE3D_SOURCES = ("api.cu", "reduce.cu", "nlse_device.cuh", "nlse_internal.h", "stage_3d_impl.cuh",
                    "stage_3d_p32_o2.cu", "stage_3d_p32_o4.cu", "stage_3d_p64_o2.cu", "stage_3d_p64_o4.cu",
-                   "stage_3d_pmix_o2.cu", "stage_3d_pmix_o4.cu", "stage_generic.cuh", "stage_slab.cuh",
-                   "stage_tiled.cuh", "stage_tma.cuh")
+                   "stage_3d_pmix_o2.cu", "stage_3d_pmix_o4.cu", "stage_generic.cuh", "stage_march.cuh", "stage_pair.cuh",
+                   "stage_slab.cuh", "stage_split.cuh", "stage_step2d.cuh", "stage_tiled.cuh", "stage_tma.cuh")
 
 
 def workload_dt(p):

@@ -632,12 +632,13 @@ int nlse_create(nlse_t* out, int dims, const int64_t* N, double h, double a, dou
   // Default kernel per form and size, from timings of the paper's workloads (MSD, 2SHOC, us per step):
   // FP64 takes the exact-sum stencil on the tiled kernels, except where the grid is so small that a
   // step is bound by latency, not by the FP64 pipe's throughput, and the plain FP64 stencil's shorter
-  // instruction chain wins: 3D grids of at most 2^15 sites (one thread per site; 21^3: 38.6 against
-  // 94.1 for the tiled exact-sum kernel, 32^3: 62.1 against 93.6) and 1D lines up to 2^15 sites, which run several steps per launch (2001 sites: 8.6 with MSD walls
-  // against 19.2 for a launch per stage and 23.8 with the exact-sum stencil on a cluster; 32,000: 18.6 against 24.4
-  // for the exact-sum stencil one thread per site; 49,000: 23.5 against 25.7).
-  // The FP32 forms take the tiled kernel on 3D grids above 2^17 sites (64^3: 26.6 against 30.0 for one
-  // thread per site, 128^3: 67.5 against 105; 40^3: 17.1 against 15.3).
+  // instruction chain wins: 3D grids of at most 2^15 sites (per-site kernels; 21^3: 21.8 against
+  // 94.1 for the tiled exact-sum kernel, 32^3: 38.8 against 93.6) and 1D lines up to 2^15 sites, which run
+  // several steps per launch (2001 sites: 8.6 with MSD walls against 19.2 for a launch per stage and 23.8
+  // with the exact-sum stencil on a cluster; 32,000: 18.6 against 24.4 for the exact-sum stencil one thread
+  // per site; 49,000: 23.5 against 25.7).
+  // The FP32 forms take the tiled kernel on 3D grids above 2^17 sites (64^3: 21.2 against 29.8 for one
+  // thread per site, 128^3: 67.5 against 105; 40^3: 16.1 against 16.0).
   c->variant = (dtype == NLSE_C128) ? 2 : 1;
   if (dims == 3 && total <= (dtype == NLSE_C128 ? (int64_t(1) << 15) : (int64_t(1) << 17))) c->variant = 0;
   if (dims == 1 && dtype == NLSE_C128)

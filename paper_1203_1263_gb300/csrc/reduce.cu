@@ -8,10 +8,12 @@
 //
 // The energy's Laplacian is summed in 64-bit fixed point too, at a scale taken
 // from the site's own operands, one per component; the sites next to a wall
-// take the FP64 form, enumerated apart so that whole warps take it.  256^3 FP64 state with V, mass and energy together: 677
-// us; with FP64 sums throughout (about 10 and 70 FP64 instructions per site)
-// 3,180.  What bounds them now: the mass the HBM read, the energy the integer
-// pipe (26 operands converted per site).
+// take the FP64 form, enumerated apart so that whole warps take it.  256^3 FP64
+// state with V, mass and energy together: 649 us; with FP64 sums throughout
+// (about 10 and 70 FP64 instructions per site) 3,180.  What bounds them now: the
+// mass the FP64 pipe (79 % busy with the two instructions a site's |Psi|^2
+// takes), the energy the FP64 pipe and the issue of the 26 conversions per site
+// together (62 % and 45 % busy).
 #include "nlse_device.cuh"
 #include "nlse_internal.h"
 #include "stage_generic.cuh"
