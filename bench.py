@@ -158,12 +158,13 @@ def fp64_peak():
     return _FP64_PEAK
 
 
-def roofline_for(dtype, sites, step_s, with_v):
+def roofline_for(dtype, sites, step_s, with_v, bytes_site=None):
     """HBM roofline of one RK4 step on the stage-streaming bytes (304 B per site with V for FP64, 152 B
     for FP32, 176 B for FP32 stages with the FP64 master), and, for FP64, the FP64-pipe view (the pipe
-    that binds that form on GB300) as a second figure."""
+    that binds that form on GB300) as a second figure. bytes_site: of a form that moves fewer."""
     hbm_peak, kind = peaks()
-    bytes_site = ALG_BYTES[dtype][0 if with_v else 1]
+    if bytes_site is None:
+        bytes_site = ALG_BYTES[dtype][0 if with_v else 1]
     gbs = sites * bytes_site / step_s / 1e9
     hbm = {"bound": "hbm", "achieved": round(gbs, 1), "peak": hbm_peak, "unit": "GB/s",
            "frac": round(gbs / hbm_peak, 4), "peak_kind": kind + " (MEASURED_PEAKS.json copy bandwidth)",
@@ -649,7 +650,8 @@ def batch_form(args, dev, K, Wm):
             "f64_sequential": round(v64, 4), "f32_sequential": round(v32, 4),
             "speedup_vs_f32_sequential": round(v_batch / v32, 3),
             "max_rel_l2_vs_f64_gpu": max(errs), "dtype": "f32",
-            "roofline": roofline_for("c64", sites, t_batch / K, True)}
+            # a step is one pass: Psi in and out, V in
+            "roofline": roofline_for("c64", sites, t_batch / K, True, 20)}
 
 
 def cpu_model():
