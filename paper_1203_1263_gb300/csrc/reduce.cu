@@ -234,6 +234,7 @@ cudaError_t launch_fix_update(const double* psi, int64_t n, unsigned int* emax, 
 // the mass kernel, two of the energy's (three blocks per SM).
 constexpr int kReduceBlocks = 6 * 152;
 static_assert(kReduceBlocks <= kMaxReduceBlocks, "a pair of partials per block");
+static_assert((int64_t(1) << 40) / kReduceBlocks + 1024 < (int64_t(1) << 31), "a block's terms of the largest grid (wide_sum.cuh)");
 static int reduce_blocks(int64_t work) {
   int64_t b = (work + 255) / 256;
   if (b < 1) b = 1;

@@ -3,8 +3,8 @@
 // GB300 issues FP64 at 1/64 of the FP32 rate, so a compensated FP64 sum (six
 // FP64 instructions a term) bounds a reduction long before HBM does.  A term
 // m 2^(e - 1075) (53-bit m) is instead added, shifted to a common exponent, to
-// a 128-bit integer per thread: exact while the bits kept reach 2^52 below the
-// last bit of the largest term seen, and otherwise off by less than 2^-104 of
+// a 128-bit integer per thread: exact while the bits kept reach 2^42 below the
+// last bit of the largest term seen, and otherwise off by less than 2^-94 of
 // that term per addition.  A block's threads are combined as integers too; its
 // total becomes an FP64 pair (sum, compensation) once.
 #pragma once
@@ -14,9 +14,10 @@
 namespace nlse {
 
 struct WideSum {
-  static constexpr int kGuard = 52;       // bits kept below the last bit of the largest term
-  // Room: 2^(53 + 52) per term and 2^22 terms per block stay below 2^127, so 2^14 for each of 256 threads; a
-  // reduction of 1024 blocks reaches that beyond the sites that fit the device's memory.
+  static constexpr int kGuard = 42;       // bits kept below the last bit of the largest term
+  // Room: a term is below 2^(53 + 42) units, so up to 2^32 terms stay below 2^127.  A block of the 912 that a large
+  // reduction has (kReduceBlocks) gets fewer than 2^31 of the 2^40 sites that a grid may have; the squares of FP32
+  // components, two terms a site, are below 2^(48 + 42).
   unsigned long long lo = 0;
   long long hi = 0;                       // (hi:lo) in units of 2^(E - 1075 - kGuard)
   int E = 0;
