@@ -21,8 +21,8 @@
 
 namespace nlse {
 
-// The block's pair into partials; the last block to get there adds all pairs and writes scale x the total.
-// `done` counts the blocks (0 before and after).
+// The block's pair into partials; the last block to get there adds all pairs and writes scale x the total, NaN if a
+// block's sum left the FP64 range (the terms themselves are finite).  `done` counts the blocks (0 before and after).
 __device__ __forceinline__ void finish(WideSum w, double* partials, unsigned int* done, double scale, double* result) {
   __shared__ bool last;
   w = block_wide_sum<256>(w);
@@ -38,15 +38,18 @@ __device__ __forceinline__ void finish(WideSum w, double* partials, unsigned int
   if (!last) return;
   __threadfence();
   WideSum t;
+  bool ok = true;
   for (int i = threadIdx.x; i < 2 * (int)gridDim.x; i += 256) {
     const double x = __ldcg(partials + i);
     if (finite_bits(x)) t.add(x);
+    else ok = false;
   }
+  ok = __syncthreads_and(ok);
   t = block_wide_sum<256>(t);
   if (threadIdx.x == 0) {
     double s, c;
     t.pair(&s, &c);
-    result[0] = scale * (s + c);
+    result[0] = ok ? scale * (s + c) : __longlong_as_double(0x7FF8000000000000ll);
     *done = 0u;
   }
 }
