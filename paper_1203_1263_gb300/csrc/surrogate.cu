@@ -1079,6 +1079,12 @@ __global__ void k_transpose_w(const bf16* __restrict__ w, bf16* __restrict__ wt,
   }
 }
 
+// The sum over a block of its threads' non-finite terms: Inf, NaN, or 0 where there are none (every thread calls).
+__device__ __forceinline__ double block_non_finite(double odd) {
+  const bool nan = __syncthreads_or(isnan(odd)), inf = __syncthreads_or(isinf(odd));
+  return nan ? __longlong_as_double(0x7FF8000000000000ll) : (inf ? __longlong_as_double(0x7FF0000000000000ll) : 0.0);
+}
+
 // Per-state sums of |psi_in|^2 and |psi_out|^2 (FP64): grid (kMassBlocks, nb), 256 threads;
 // partial sums to part[(n * kMassBlocks + block) * 2 + {0, 1}].
 constexpr int kMassBlocks = 32;
@@ -1087,7 +1093,7 @@ __global__ void __launch_bounds__(256) k_state_mass(const float2* __restrict__ i
   // sums of squares of FP32 values, exact on the integer pipe (27 us for 16 256^2 states in FP64)
   const int64_t base = (int64_t)blockIdx.y * HW;
   nlse::WideSum a, b;
-  bool oka = true, okb = true;
+  double odda = 0.0, oddb = 0.0;   // the non-finite terms
   const int64_t step = (int64_t)gridDim.x * blockDim.x;
   int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   float2 u1 = {0.f, 0.f}, v1 = u1;   // the next site's values, requested a site ahead
@@ -1105,17 +1111,19 @@ __global__ void __launch_bounds__(256) k_state_mass(const float2* __restrict__ i
       a.add_square(u.x);
       a.add_square(u.y);
     } else {
-      oka = false;
+      odda += double(u.x) * u.x + double(u.y) * u.y;
     }
     if (isfinite(v.x) && isfinite(v.y)) {
       b.add_square(v.x);
       b.add_square(v.y);
     } else {
-      okb = false;
+      oddb += double(v.x) * v.x + double(v.y) * v.y;
     }
   }
-  oka = __syncthreads_and(oka);
-  okb = __syncthreads_and(okb);
+  if (__syncthreads_or(odda != 0.0 || oddb != 0.0)) {
+    odda = block_non_finite(odda);
+    oddb = block_non_finite(oddb);
+  }
   // lane 0 of every warp holds the warp's sums; warp 0 finishes the first, warp 1 the second
   __shared__ unsigned long long sl[2][8];
   __shared__ long long sh[2][8];
@@ -1133,8 +1141,7 @@ __global__ void __launch_bounds__(256) k_state_mass(const float2* __restrict__ i
     if (lane < 8) { a.lo = sl[warp][lane]; a.hi = sh[warp][lane]; a.E = se[warp][lane]; }
     a = nlse::warp_wide_sum(a);
     if (lane == 0)
-      part[((int64_t)blockIdx.y * kMassBlocks + blockIdx.x) * 2 + warp] =
-          (warp == 0 ? oka : okb) ? a.value() : __longlong_as_double(0x7FF8000000000000ll);
+      part[((int64_t)blockIdx.y * kMassBlocks + blockIdx.x) * 2 + warp] = a.value() + (warp == 0 ? odda : oddb);
   }
 }
 
@@ -1361,7 +1368,7 @@ __global__ void __launch_bounds__(256) k_mse(const float2* __restrict__ psi, con
   // a warp per 32 sites, a lane per site for the arithmetic (the squares exact on the integer pipe), then the whole
   // warp for the sites' pc / 8 chunks in memory order (96 us with a thread per chunk and FP64 sums in one lane of 8)
   nlse::WideSum sum;
-  bool ok = true;
+  double odd = 0.0;   // the non-finite terms
   const float scale = 2.f / float(2 * P);
   const int cpp = pc / 8, lane = threadIdx.x & 31;
   uint4* dst = reinterpret_cast<uint4*>(dz);
@@ -1377,7 +1384,7 @@ __global__ void __launch_bounds__(256) k_mse(const float2* __restrict__ psi, con
         sum.add_square(ex);
         sum.add_square(ey);
       } else {
-        ok = false;
+        odd += double(ex) * ex + double(ey) * ey;
       }
       float gx = scale * ex, gy = scale * ey;
       if (coef) {
@@ -1395,11 +1402,9 @@ __global__ void __launch_bounds__(256) k_mse(const float2* __restrict__ psi, con
       if (c < n) dst[p0 * cpp + c] = make_uint4(c - site * cpp == 0 ? gs : 0u, 0u, 0u, 0u);
     }
   }
-  ok = __syncthreads_and(ok);
+  if (__syncthreads_or(odd != 0.0)) odd = block_non_finite(odd);
   sum = nlse::block_wide_sum<256>(sum);
-  if (threadIdx.x == 0) {
-    atomicAdd(loss_acc, (ok ? sum.value() : __longlong_as_double(0x7FF8000000000000ll)) / double(2 * P));
-  }
+  if (threadIdx.x == 0) atomicAdd(loss_acc, (sum.value() + odd) / double(2 * P));
 }
 
 // db[c] += sum over pixels of dz[p * stride + c] for c < creal (stride <= 256;
