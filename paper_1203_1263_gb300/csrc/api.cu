@@ -637,10 +637,16 @@ int nlse_create(nlse_t* out, int dims, const int64_t* N, double h, double a, dou
   // several steps per launch (2001 sites: 8.6 with MSD walls against 19.2 for a launch per stage and 23.8
   // with the exact-sum stencil on a cluster; 32,000: 18.6 against 24.4 for the exact-sum stencil one thread
   // per site; 49,000: 23.5 against 25.7).
+  // FP64 planes take the exact-sum stencil where a whole step is one launch (step2x_fits) and above 80,000 sites;
+  // the planes between (274^2 to 282^2, and long or narrow ones) the FP64 stencil, whose error is the smaller one
+  // where the operands' rounding is not taken back (Field::fine) and which is the faster one by launches per stage
+  // (282^2: 49.7 against 56.6; 316^2: 61.1 against 54.0).
   // The FP32 forms take the tiled kernel on 3D grids above 2^17 sites (64^3: 21.2 against 29.8 for one
   // thread per site, 128^3: 67.5 against 105; 40^3: 16.1 against 16.0).
   c->variant = (dtype == NLSE_C128) ? 2 : 1;
   if (dims == 3 && total <= (dtype == NLSE_C128 ? (int64_t(1) << 15) : (int64_t(1) << 17))) c->variant = 0;
+  if (dims == 2 && dtype == NLSE_C128 && total <= 80000 && !step2x_fits(int(N[0]), int(N[1]), bc == NLSE_BC_PERIODIC))
+    c->variant = 1;
   if (dims == 1 && dtype == NLSE_C128)
     c->variant = (total <= 2500 && line_ok(int(N[0]), true)) ? 1 : (total <= (int64_t(1) << 15) ? 0 : 3);
   c->tile_cfg = -1;
