@@ -253,7 +253,9 @@ size_t nlse_batch_workspace_bytes(int nruns, const nlse_run_desc *runs);
 int nlse_batch_create(nlse_batch_t *out, int nruns, const nlse_run_desc *runs, void *workspace, size_t ws_bytes,
                       void *stream);
 
-/* Advance every run by nsteps RK4 steps of its own dt; asynchronous. */
+/* Advance every run by nsteps RK4 steps of its own dt; asynchronous.  The
+ * runs' Psi and V are read as the stream's earlier work left them; neither
+ * may be written while the steps run. */
 int nlse_batch_step(nlse_batch_t b, int64_t nsteps);
 
 /* Tile shape of the batched step kernel: 0 = 32x28 cells with strips of 2 rows per thread, 1 = 64x24 with

@@ -375,17 +375,19 @@ int steps_per_launch(const nlse_ctx* c) {
 }
 
 template <class T>
-cudaError_t launch_steps1(const nlse_ctx* c, double dt, int steps, cudaStream_t st, const void* cur, void* nxt) {
+cudaError_t launch_steps1(const nlse_ctx* c, double dt, int steps, cudaStream_t st, const void* cur, void* nxt, bool early) {
   Step1Args<T> A = step_args<T, Step1Args<T>>(c, dt, cur, nxt);
   A.n = int(c->n[0]);
-  return launch_steps1d<T>(A, c->order, steps, st);
+  return launch_steps1d<T>(A, c->order, steps, early, st);
 }
 
-cudaError_t launch_steps1_any(const nlse_ctx* c, double dt, int steps, cudaStream_t st, const void* cur, void* nxt) {
+// (early: not a call's first launch, see launch_early)
+cudaError_t launch_steps1_any(const nlse_ctx* c, double dt, int steps, cudaStream_t st, const void* cur, void* nxt,
+                              bool early) {
   switch (c->dtype) {
-    case NLSE_C128: return launch_steps1<P64>(c, dt, steps, st, cur, nxt);
-    case NLSE_C64: return launch_steps1<P32>(c, dt, steps, st, cur, nxt);
-    default: return launch_steps1<PMix>(c, dt, steps, st, cur, nxt);
+    case NLSE_C128: return launch_steps1<P64>(c, dt, steps, st, cur, nxt, early);
+    case NLSE_C64: return launch_steps1<P32>(c, dt, steps, st, cur, nxt, early);
+    default: return launch_steps1<PMix>(c, dt, steps, st, cur, nxt, early);
   }
 }
 
@@ -411,14 +413,15 @@ bool step2_path(const nlse_ctx* c) {
 }
 
 template <class T>
-cudaError_t launch_step2(const nlse_ctx* c, double dt, cudaStream_t st, const void* cur, void* nxt) {
+cudaError_t launch_step2(const nlse_ctx* c, double dt, cudaStream_t st, const void* cur, void* nxt, bool early) {
   Step2Args<T> A = step_args<T, Step2Args<T>>(c, dt, cur, nxt);
   A.n[0] = int(c->n[0]);
   A.n[1] = int(c->n[1]);
-  return launch_step2d<T>(A, c->order, c->tile_cfg, st);
+  return launch_step2d<T>(A, c->order, c->tile_cfg, early, st);
 }
 
-cudaError_t launch_step2x_any(const nlse_ctx* c, double dt, cudaStream_t st, const void* cur, void* nxt, int turn) {
+cudaError_t launch_step2x_any(const nlse_ctx* c, double dt, cudaStream_t st, const void* cur, void* nxt, int turn,
+                              bool early) {
   const Field<P64> f = make_field<P64>(c, cur);
   Step2xArgs A = step_args<P64, Step2xArgs>(c, dt, cur, nxt);
   A.n[0] = int(c->n[0]);
@@ -432,15 +435,15 @@ cudaError_t launch_step2x_any(const nlse_ctx* c, double dt, cudaStream_t st, con
   A.turn = turn & 3;
   A.F0 = c->fixF;
   A.fix_offset = c->fix_offset;
-  return launch_step2x(A, c->order, st);
+  return launch_step2x(A, c->order, early, st);
 }
 
-// Step i of a run of steps.
-cudaError_t launch_step2_any(const nlse_ctx* c, double dt, cudaStream_t st, const void* cur, void* nxt, int i = 0) {
+// Step i of a run of steps (the first one an ordinary launch).
+cudaError_t launch_step2_any(const nlse_ctx* c, double dt, cudaStream_t st, const void* cur, void* nxt, int i) {
   switch (c->dtype) {
-    case NLSE_C128: return launch_step2x_any(c, dt, st, cur, nxt, i);
-    case NLSE_C64: return launch_step2<P32>(c, dt, st, cur, nxt);
-    default: return launch_step2<PMix>(c, dt, st, cur, nxt);
+    case NLSE_C128: return launch_step2x_any(c, dt, st, cur, nxt, i, i > 0);
+    case NLSE_C64: return launch_step2<P32>(c, dt, st, cur, nxt, i > 0);
+    default: return launch_step2<PMix>(c, dt, st, cur, nxt, i > 0);
   }
 }
 
@@ -497,7 +500,8 @@ int ensure_graph(nlse_ctx* c, double dt) {
     if (lines) {   // ping-pong as below
       void* a = c->psi;
       void* b = step_alt(c);
-      le = (i % 2 == 0) ? launch_steps1_any(c, dt, per, c->cap, a, b) : launch_steps1_any(c, dt, per, c->cap, b, a);
+      le = (i % 2 == 0) ? launch_steps1_any(c, dt, per, c->cap, a, b, i > 0)
+                        : launch_steps1_any(c, dt, per, c->cap, b, a, true);
     } else if (step2) {
       void* a = c->psi;
       void* b = step_alt(c);
@@ -777,9 +781,11 @@ int nlse_step(nlse_t c, int64_t nsteps, double dt) {
   if (lines_path(c) && left > 0) {   // launches of up to `per` steps; an odd number of them ends in the copy
     void *cur = c->psi, *nxt = step_alt(c);
     const int per = steps_per_launch(c);
+    bool early = false;
     while (left > 0 && e == cudaSuccess) {
       const int k = left < per ? int(left) : per;
-      e = launch_steps1_any(c, dt, k, c->stream, cur, nxt);
+      e = launch_steps1_any(c, dt, k, c->stream, cur, nxt, early);
+      early = true;
       void* t = cur;
       cur = nxt;
       nxt = t;
@@ -943,12 +949,12 @@ int nlse_autotune(nlse_t c, int* best_tile_cfg, float* best_ms) {
     for (int t = 0; t < 4 && e == cudaSuccess; ++t) {
       c->tile_cfg = t;
       const bool step2 = step2_path(c);   // one whole step, into Psi's ping-pong copy
-      if (step2) e = launch_step2_any(c, 1e-12, c->stream, c->psi, step_alt(c));
+      if (step2) e = launch_step2_any(c, 1e-12, c->stream, c->psi, step_alt(c), 0);
       else e = launch_stage_any(c, 1, 1e-12, c->stream);
       if (e == cudaSuccess && !step2) e = launch_stage_any(c, 2, 1e-12, c->stream);
       if (e == cudaSuccess) e = cudaEventRecord(e0, c->stream);
       for (int r = 0; r < 3 && e == cudaSuccess; ++r)
-        e = step2 ? launch_step2_any(c, 1e-12, c->stream, c->psi, step_alt(c)) : launch_stage_any(c, 2, 1e-12, c->stream);
+        e = step2 ? launch_step2_any(c, 1e-12, c->stream, c->psi, step_alt(c), 1) : launch_stage_any(c, 2, 1e-12, c->stream);
       if (e == cudaSuccess) e = cudaEventRecord(e1, c->stream);
       if (e == cudaSuccess) e = cudaEventSynchronize(e1);
       float ms = 0.f;

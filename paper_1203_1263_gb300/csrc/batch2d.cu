@@ -144,23 +144,23 @@ struct nlse_batch {
 namespace {
 
 template <int CFG>
-cudaError_t launch_shape(const nlse_batch* b, bool back, cudaStream_t st) {
+cudaError_t launch_shape(const nlse_batch* b, bool back, bool early, cudaStream_t st) {
   constexpr Shape s = kShapes[CFG];
   const size_t smem = step2_smem<s.tx>(s.ty, true);
   auto kern = k_batch2d_step<CFG>;
   static const cudaError_t attr = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
   if (attr != cudaSuccess) return attr;
-  return launch_early(kern, dim3((unsigned)b->lay.nitems), dim3(s.nt), smem, st,
+  return launch_early(early, kern, dim3((unsigned)b->lay.nitems), dim3(s.nt), smem, st,
                       (const BatchRun*)(b->ws + b->lay.runs_off), (const Item*)(b->ws + b->lay.items_off), back ? 1 : 0);
 }
 
-// One step of every run, from Psi into the copies or back.
-cudaError_t launch_batch_step(const nlse_batch* b, bool back, cudaStream_t st) {
+// One step of every run, from Psi into the copies or back (early: not a call's first, see launch_early).
+cudaError_t launch_batch_step(const nlse_batch* b, bool back, bool early, cudaStream_t st) {
   switch (b->tile_cfg < 0 ? kDefaultShape : b->tile_cfg) {
-    case 0: return launch_shape<0>(b, back, st);
-    case 1: return launch_shape<1>(b, back, st);
-    case 2: return launch_shape<2>(b, back, st);
-    default: return launch_shape<3>(b, back, st);
+    case 0: return launch_shape<0>(b, back, early, st);
+    case 1: return launch_shape<1>(b, back, early, st);
+    case 2: return launch_shape<2>(b, back, early, st);
+    default: return launch_shape<3>(b, back, early, st);
   }
 }
 
@@ -310,7 +310,7 @@ int nlse_batch_step(nlse_batch_t b, int64_t nsteps) {
       e = cudaStreamBeginCapture(b->cap, cudaStreamCaptureModeThreadLocal);
       cudaError_t le = cudaSuccess;
       for (int i = 0; i < kGraphSteps && le == cudaSuccess && e == cudaSuccess; ++i)   // an even count ends in Psi
-        le = launch_batch_step(b, i % 2 == 1, b->cap);
+        le = launch_batch_step(b, i % 2 == 1, i > 0, b->cap);
       cudaGraph_t g = nullptr;
       cudaError_t ee = cudaStreamEndCapture(b->cap, &g);
       if (e == cudaSuccess) e = (le != cudaSuccess) ? le : ee;
@@ -323,9 +323,10 @@ int nlse_batch_step(nlse_batch_t b, int64_t nsteps) {
     }
     for (; left >= kGraphSteps && e == cudaSuccess; left -= kGraphSteps) e = cudaGraphLaunch(b->exec, b->stream);
   }
-  for (; left > 0 && e == cudaSuccess; left -= 2) {   // pairs end in Psi; an odd step is copied back
-    e = launch_batch_step(b, false, b->stream);
-    if (e == cudaSuccess) e = left > 1 ? launch_batch_step(b, true, b->stream) : launch_batch_copy(b, b->stream);
+  bool early = false;
+  for (; left > 0 && e == cudaSuccess; left -= 2, early = true) {   // pairs end in Psi; an odd step is copied back
+    e = launch_batch_step(b, false, early, b->stream);
+    if (e == cudaSuccess) e = left > 1 ? launch_batch_step(b, true, true, b->stream) : launch_batch_copy(b, b->stream);
   }
   if (e != cudaSuccess) return bfail(NLSE_ECUDA, cudaGetErrorString(e));
   return NLSE_OK;
@@ -357,7 +358,7 @@ int nlse_batch_autotune(nlse_batch_t b, int* best_tile_cfg, float* best_ms) {
       rc = nlse_batch_set_tile(b, t);
       if (rc != NLSE_OK) break;
       cudaError_t e = cudaEventRecord(e0, b->stream);
-      for (int q = 0; q < 3 && e == cudaSuccess; ++q) e = launch_batch_step(b, false, b->stream);
+      for (int q = 0; q < 3 && e == cudaSuccess; ++q) e = launch_batch_step(b, false, q > 0, b->stream);
       if (e == cudaSuccess) e = cudaEventRecord(e1, b->stream);
       if (e == cudaSuccess) e = cudaEventSynchronize(e1);
       float ms = 0.f;

@@ -18,12 +18,15 @@ constexpr int kMaxReduceBlocks = 1024;
 // where a CTA fills an SM or CTAs are many; where a grid is less than a wave of small CTAs, the next
 // kernel's pile up on the SMs that are done first (64^3 FP32 columns 26.7 against 21.1 us per step without, 46^3
 // one thread per site 20.2 and 16.6, 512^2 FP32 12.8 and 10.9; but 256^2 FP64 21.7 and 22.4, a batch 594
-// and 602).  On a dependency that is not such a kernel this is an ordinary launch.
+// and 602).  Before grid_wait() a kernel may read only what nobody writes while the call's kernels run (V, tables).  What
+// wrote that before the call is ordered with it by an ordinary launch alone: the early start needs no more of the
+// launch before than its CTAs' end, not that their stores are visible.  So the first launch of a call is an ordinary
+// one (early = false; in a captured graph the first node has nothing before it).
 __device__ __forceinline__ void grid_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void grid_launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
 template <class... P, class... Q>
-inline cudaError_t launch_early(void (*kern)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t stream,
+inline cudaError_t launch_early(bool early, void (*kern)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t stream,
                                 Q&&... args) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = grid;
@@ -34,7 +37,7 @@ inline cudaError_t launch_early(void (*kern)(P...), dim3 grid, dim3 block, size_
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
-  cfg.numAttrs = 1;
+  cfg.numAttrs = early ? 1 : 0;
   return cudaLaunchKernelEx(&cfg, kern, static_cast<P>(args)...);
 }
 
@@ -58,21 +61,22 @@ bool fused_grid_ok(int d, const int* n);
 // the fused kernel's TMA box: 64 + 8 complex values by 8 + 8 rows
 constexpr int kFusedBoxX = 2 * (64 + 8), kFusedBoxY = 8 + 8;
 
-// One RK4 step of a 2D grid in one launch, Psi^n in A.in to Psi^{n+1} in A.out (stage_step2d.cuh).
+// One RK4 step of a 2D grid in one launch, Psi^n in A.in to Psi^{n+1} in A.out (stage_step2d.cuh).  early, here and
+// below: not a call's first launch (launch_early).
 template <class T>
-cudaError_t launch_step2d(const Step2Args<T>& A, int order, int tile_cfg, cudaStream_t stream);
+cudaError_t launch_step2d(const Step2Args<T>& A, int order, int tile_cfg, bool early, cudaStream_t stream);
 
 // The same for FP64 with the exact-sum stencil (stage_step2x.cuh); launch_max_expo puts the largest exponent of a
 // complex128 array (n components) into the word of the first step.
 bool step2x_fits(int ny, int nx, bool periodic);   // grids it is the faster one for
-cudaError_t launch_step2x(const Step2xArgs& A, int order, cudaStream_t stream);
+cudaError_t launch_step2x(const Step2xArgs& A, int order, bool early, cudaStream_t stream);
 cudaError_t launch_max_expo(const double* psi, int64_t n, unsigned int* expo, cudaStream_t stream);
 
 // Up to steps1d_per_launch(n) RK4 steps of an n-site line in one launch, from A.in to A.out (stage_step1d.cuh).
 template <class T>
 int steps1d_per_launch(int n);
 template <class T>
-cudaError_t launch_steps1d(const Step1Args<T>& A, int order, int steps, cudaStream_t stream);
+cudaError_t launch_steps1d(const Step1Args<T>& A, int order, int steps, bool early, cudaStream_t stream);
 
 // 1D lines on one thread-block cluster (stage_line1d.cuh): nsteps RK4 steps of
 // an n-site line in one launch; A[0..3] are stages 1..4 with Psi updated in

@@ -122,7 +122,7 @@ cudaError_t launch_march_stage(const StageArgs<T>& A, cudaStream_t stream) {
   const int64_t deep = (int64_t)planes * (A.f.n[1] - 4) * (A.f.n[2] - 4);
   const int64_t n2 = A.f.ninterior - deep, n3 = boundary_count(3, A.f.n, A.f.m);
   const unsigned b1 = (unsigned)(ntx * nty * nzc), b2 = b1 + (unsigned)((n2 + 255) / 256), b3 = b2 + (unsigned)((n3 + 255) / 256);
-  return launch_early(kern, dim3(b3), dim3(256), 0, stream, A, ntx, nty, zc, b1, b2, b3, n2, n3, !one_wave);
+  return launch_early(true, kern, dim3(b3), dim3(256), 0, stream, A, ntx, nty, zc, b1, b2, b3, n2, n3, !one_wave);
 }
 
 // Walls on every side and a deep interior (every extent >= 5); fewer than 2^31 sites.

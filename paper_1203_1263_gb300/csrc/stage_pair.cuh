@@ -211,7 +211,7 @@ cudaError_t launch_pair(const StageArgs<P64>& A, cudaStream_t stream) {
   const int n2 = (int)A.f.ninterior - n1, n3 = (int)boundary_count(3, A.f.n, A.f.m);
   constexpr int threads = 128, per = threads / 2;
   const unsigned b1 = (n3 + per - 1) / per, b2 = b1 + (n2 + per - 1) / per, b3 = b2 + (n1 + per - 1) / per;
-  return launch_early(k_stage_pair<ORDER>, dim3(b3), dim3(threads), 0, stream, A, b1, b2, n1, n2, n3);
+  return launch_early(true, k_stage_pair<ORDER>, dim3(b3), dim3(threads), 0, stream, A, b1, b2, n1, n2, n3);
 }
 
 }  // namespace nlse

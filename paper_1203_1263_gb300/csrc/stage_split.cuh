@@ -171,9 +171,7 @@ cudaError_t launch_split(const StageArgs<T>& A, cudaStream_t stream, bool deep, 
   auto blocks = [&](int64_t n) { return (unsigned)((n + threads - 1) / threads); };
   const unsigned b1 = blocks(n1), b2 = b1 + blocks(n2), b3 = b2 + blocks(n3);
   auto run = [&](auto kern) -> cudaError_t {
-    if (early) return launch_early(kern, dim3(b3), dim3((unsigned)threads), 0, stream, A, b1, b2, n1, n2, n3);
-    kern<<<b3, threads, 0, stream>>>(A, b1, b2, n1, n2, n3);
-    return cudaGetLastError();
+    return launch_early(early, kern, dim3(b3), dim3((unsigned)threads), 0, stream, A, b1, b2, n1, n2, n3);
   };
   if (A.f.ninterior + n3 < (int64_t(1) << 31)) return run(k_stage_split<T, D, ORDER, EXACT, uint32_t>);
   return run(k_stage_split<T, D, ORDER, EXACT, uint64_t>);

@@ -101,9 +101,10 @@ __global__ void __launch_bounds__(2 * SITES + 32) k_steps1d_split(const __grid_c
 namespace {
 
 template <class K, class T>
-cudaError_t launch_shape(K kern, int sites, int threads, const Step1Args<T>& A, int halo, int steps, cudaStream_t stream) {
+cudaError_t launch_shape(K kern, int sites, int threads, const Step1Args<T>& A, int halo, int steps, bool early, cudaStream_t stream) {
   const int own = sites - 2 * halo;
-  return launch_early(kern, dim3((unsigned)line_ctas(A.n, own, A.bc == BC_PERIODIC)), dim3((unsigned)threads + 32), 0, stream, A, halo, steps);
+  return launch_early(early, kern, dim3((unsigned)line_ctas(A.n, own, A.bc == BC_PERIODIC)), dim3((unsigned)threads + 32), 0,
+                      stream, A, halo, steps);
 }
 
 // The sites per CTA and the most steps per launch (a power of two up to 8) of an n-site line.
@@ -140,22 +141,22 @@ Plan plan32(int n, bool mixed) {
 }
 
 template <int ORDER>
-cudaError_t launch_order(const Step1Args<P64>& A, int steps, cudaStream_t stream) {
+cudaError_t launch_order(const Step1Args<P64>& A, int steps, bool early, cudaStream_t stream) {
   const Plan p = plan64(A.n);
   const int halo = 8 * p.steps;
   switch (p.sites) {
-    case 48: return launch_shape(k_steps1d_split<ORDER, 48>, 48, 96, A, halo, steps, stream);
-    default: return launch_shape(k_steps1d_split<ORDER, 112>, 112, 224, A, halo, steps, stream);
+    case 48: return launch_shape(k_steps1d_split<ORDER, 48>, 48, 96, A, halo, steps, early, stream);
+    default: return launch_shape(k_steps1d_split<ORDER, 112>, 112, 224, A, halo, steps, early, stream);
   }
 }
 template <int ORDER, class T>
-cudaError_t launch_order(const Step1Args<T>& A, int steps, cudaStream_t stream) {
+cudaError_t launch_order(const Step1Args<T>& A, int steps, bool early, cudaStream_t stream) {
   const Plan p = plan32(A.n, !std::is_same<T, P32>::value);
   const int halo = 8 * p.steps;
   switch (p.sites) {
-    case 256: return launch_shape(k_steps1d<T, ORDER, 256, 1>, 256, 256, A, halo, steps, stream);
-    case 512: return launch_shape(k_steps1d<T, ORDER, 256, 2>, 512, 256, A, halo, steps, stream);
-    default: return launch_shape(k_steps1d<T, ORDER, 256, 4>, 1024, 256, A, halo, steps, stream);
+    case 256: return launch_shape(k_steps1d<T, ORDER, 256, 1>, 256, 256, A, halo, steps, early, stream);
+    case 512: return launch_shape(k_steps1d<T, ORDER, 256, 2>, 512, 256, A, halo, steps, early, stream);
+    default: return launch_shape(k_steps1d<T, ORDER, 256, 4>, 1024, 256, A, halo, steps, early, stream);
   }
 }
 
@@ -168,13 +169,13 @@ int steps1d_per_launch(int n) {
 }
 
 template <class T>
-cudaError_t launch_steps1d(const Step1Args<T>& A, int order, int steps, cudaStream_t stream) {
-  return order == 4 ? launch_order<4>(A, steps, stream) : launch_order<2>(A, steps, stream);
+cudaError_t launch_steps1d(const Step1Args<T>& A, int order, int steps, bool early, cudaStream_t stream) {
+  return order == 4 ? launch_order<4>(A, steps, early, stream) : launch_order<2>(A, steps, early, stream);
 }
 
-#define INST(T)                                                                        \
-  template int steps1d_per_launch<T>(int);                                             \
-  template cudaError_t launch_steps1d<T>(const Step1Args<T>&, int, int, cudaStream_t);
+#define INST(T)                                                                              \
+  template int steps1d_per_launch<T>(int);                                                   \
+  template cudaError_t launch_steps1d<T>(const Step1Args<T>&, int, int, bool, cudaStream_t);
 INST(P64) INST(P32) INST(PMix)
 #undef INST
 

@@ -8,7 +8,7 @@ template <class T, int ORDER, int TX, int NT, int RY, int MINB>
 __global__ void __launch_bounds__(NT, MINB) k_step2d(const __grid_constant__ Step2Args<T> A, int ty, int ntx) {
   extern __shared__ __align__(16) unsigned char step2_smem[];
   Step2Tile<T, ORDER, TX, NT, RY> tile(A, ty, blockIdx.x % ntx, blockIdx.x / ntx, step2_smem);
-  // launched while the step before still runs: V is not its output, Psi^n is
+  // may start while the step before still runs: V is not its output, Psi^n is
   tile.load_potential();
   grid_wait();
   tile.run();
@@ -56,7 +56,7 @@ int plan(const Shape& s, int ny, int nx, bool periodic, bool with_v) {
 }
 
 template <class T, int ORDER, int CFG>
-cudaError_t launch_shape(const Step2Args<T>& A, int ty, cudaStream_t stream) {
+cudaError_t launch_shape(const Step2Args<T>& A, int ty, bool early, cudaStream_t stream) {
   constexpr Shape s = kShapes[CFG];
   const size_t smem = step2_smem<s.tx>(ty, A.V != nullptr);
   auto kern = k_step2d<T, ORDER, s.tx, s.nt, s.ry, s.per_sm>;
@@ -64,31 +64,31 @@ cudaError_t launch_shape(const Step2Args<T>& A, int ty, cudaStream_t stream) {
   if (attr != cudaSuccess) return attr;
   int ntx, nty;
   step2_tiles(A.n[0], A.n[1], A.bc == BC_PERIODIC, s.tx, ty, &ntx, &nty);
-  return launch_early(kern, dim3((unsigned)(ntx * nty)), dim3(s.nt), smem, stream, A, ty, ntx);
+  return launch_early(early, kern, dim3((unsigned)(ntx * nty)), dim3(s.nt), smem, stream, A, ty, ntx);
 }
 
 template <class T, int ORDER>
-cudaError_t launch_order(const Step2Args<T>& A, int tile_cfg, cudaStream_t stream) {
+cudaError_t launch_order(const Step2Args<T>& A, int tile_cfg, bool early, cudaStream_t stream) {
   // 64 columns (a smaller share of halo) where the grid fills the chip with them, 32 below: 400^2 9.3 against
   // 11.1 us per step, 600^2 12.9 against 12.1, 1300^2 32.5 against 30.2
   const int cfg = tile_cfg >= 0 ? tile_cfg : ((long long)A.n[0] * A.n[1] > 250000 ? 1 : 0);
   const int ty = plan(kShapes[cfg], A.n[0], A.n[1], A.bc == BC_PERIODIC, A.V != nullptr);
   switch (cfg) {
-    case 0: return launch_shape<T, ORDER, 0>(A, ty, stream);
-    case 1: return launch_shape<T, ORDER, 1>(A, ty, stream);
-    case 2: return launch_shape<T, ORDER, 2>(A, ty, stream);
-    default: return launch_shape<T, ORDER, 3>(A, ty, stream);
+    case 0: return launch_shape<T, ORDER, 0>(A, ty, early, stream);
+    case 1: return launch_shape<T, ORDER, 1>(A, ty, early, stream);
+    case 2: return launch_shape<T, ORDER, 2>(A, ty, early, stream);
+    default: return launch_shape<T, ORDER, 3>(A, ty, early, stream);
   }
 }
 
 }  // namespace
 
 template <class T>
-cudaError_t launch_step2d(const Step2Args<T>& A, int order, int tile_cfg, cudaStream_t stream) {
-  return order == 4 ? launch_order<T, 4>(A, tile_cfg, stream) : launch_order<T, 2>(A, tile_cfg, stream);
+cudaError_t launch_step2d(const Step2Args<T>& A, int order, int tile_cfg, bool early, cudaStream_t stream) {
+  return order == 4 ? launch_order<T, 4>(A, tile_cfg, early, stream) : launch_order<T, 2>(A, tile_cfg, early, stream);
 }
 
-template cudaError_t launch_step2d<P32>(const Step2Args<P32>&, int, int, cudaStream_t);
-template cudaError_t launch_step2d<PMix>(const Step2Args<PMix>&, int, int, cudaStream_t);
+template cudaError_t launch_step2d<P32>(const Step2Args<P32>&, int, int, bool, cudaStream_t);
+template cudaError_t launch_step2d<PMix>(const Step2Args<PMix>&, int, int, bool, cudaStream_t);
 
 }  // namespace nlse

@@ -25,11 +25,11 @@ int tiles(int ny, int nx, bool periodic, int ty, int* ntx) {
 }
 
 template <int ORDER>
-cudaError_t launch_order(const Step2xArgs& A, int ty, int ntx, int n, cudaStream_t stream) {
+cudaError_t launch_order(const Step2xArgs& A, int ty, int ntx, int n, bool early, cudaStream_t stream) {
   auto kern = k_step2x<ORDER>;
   static const cudaError_t attr = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
   if (attr != cudaSuccess) return attr;
-  return launch_early(kern, dim3((unsigned)n), dim3(kNT), step2x_smem(kTX, ty, A.V != nullptr), stream, A, ty, ntx);
+  return launch_early(early, kern, dim3((unsigned)n), dim3(kNT), step2x_smem(kTX, ty, A.V != nullptr), stream, A, ty, ntx);
 }
 
 }  // namespace
@@ -41,12 +41,12 @@ bool step2x_fits(int ny, int nx, bool periodic) {
   return (int64_t)ny * nx < (int64_t(1) << 20) && tiles(ny, nx, periodic, 16, &ntx) <= kPerSm * 152;
 }
 
-cudaError_t launch_step2x(const Step2xArgs& A, int order, cudaStream_t stream) {
+cudaError_t launch_step2x(const Step2xArgs& A, int order, bool early, cudaStream_t stream) {
   // 8-row tiles while those are one wave too (128^2: 16.7 against 19.1 us)
   const bool periodic = A.bc == BC_PERIODIC;
   int ntx, ty = 8, n = tiles(A.n[0], A.n[1], periodic, ty, &ntx);
   if (n > kPerSm * 152) n = tiles(A.n[0], A.n[1], periodic, ty = 16, &ntx);
-  return order == 4 ? launch_order<4>(A, ty, ntx, n, stream) : launch_order<2>(A, ty, ntx, n, stream);
+  return order == 4 ? launch_order<4>(A, ty, ntx, n, early, stream) : launch_order<2>(A, ty, ntx, n, early, stream);
 }
 
 }  // namespace nlse
