@@ -79,6 +79,14 @@ __device__ __forceinline__ typename V2<R>::t ld2(const C* __restrict__ p, int64_
   const C v = __ldg(p + i);
   return {widen<R>(v.x), widen<R>(v.y)};
 }
+// The same through an ordinary load, for kernels that may start before the kernel that writes the field has ended
+// (launch_early): the read-only path above is for data that nobody writes while the kernel runs, and keeps no order
+// with the wait for that kernel.
+template <class R, class C>
+__device__ __forceinline__ typename V2<R>::t ld2_ordered(const C* p, int64_t i) {
+  const C v = p[i];
+  return {widen<R>(v.x), widen<R>(v.y)};
+}
 template <class R, class VR>
 __device__ __forceinline__ R ldv(const VR* __restrict__ V, int64_t i) {
   return V ? widen<R>(__ldg(V + i)) : R(0);
@@ -119,31 +127,34 @@ struct Field {
 // Operand access for the stencil.  An accessor is positioned at one interior
 // site c and returns Psi at c plus small offsets: at1(k, s) = Psi(c + s e_k),
 // at2(k, s, j, t) = Psi(c + s e_k + t e_j), atv(o) = Psi(c + sum_k o_k e_k).
-// GAcc reads global memory; the tiled kernels supply shared-memory accessors.
-// The arithmetic below never depends on which accessor is used.
-template <class T, int D>
+// GAcc reads global memory (ORDERED: by ld2_ordered); the tiled kernels supply
+// shared-memory accessors.  The arithmetic below never depends on which
+// accessor is used.
+template <class T, int D, bool ORDERED = false>
 struct GAcc {
   using R = typename T::R;
   using C2 = typename V2<R>::t;
   const Field<T>& f;
   int64_t c;
   __device__ __forceinline__ GAcc(const Field<T>& f_, int64_t c_) : f(f_), c(c_) {}
-  __device__ __forceinline__ C2 at0() const { return ld2<R>(f.in, c); }
-  __device__ __forceinline__ C2 at1(int k, int s) const { return ld2<R>(f.in, c + s * f.st[k]); }
-  __device__ __forceinline__ C2 at2(int k, int s, int j, int t) const {
-    return ld2<R>(f.in, c + s * f.st[k] + t * f.st[j]);
+  __device__ __forceinline__ C2 at(int64_t i) const {
+    if constexpr (ORDERED) return ld2_ordered<R>(f.in, i);
+    else return ld2<R>(f.in, i);
   }
+  __device__ __forceinline__ C2 at0() const { return at(c); }
+  __device__ __forceinline__ C2 at1(int k, int s) const { return at(c + s * f.st[k]); }
+  __device__ __forceinline__ C2 at2(int k, int s, int j, int t) const { return at(c + s * f.st[k] + t * f.st[j]); }
   __device__ __forceinline__ C2 atv(const int* o) const {
     int64_t q = c;
 #pragma unroll
     for (int k = 0; k < D; ++k) q += o[k] * f.st[k];
-    return ld2<R>(f.in, q);
+    return at(q);
   }
   // fixed-point operands of the exact-sum stencil (FP64 fields only)
   __device__ __forceinline__ longlong2 fx0() const;
   __device__ __forceinline__ longlong2 fx1(int k, int s) const;
   __device__ __forceinline__ longlong2 fx2(int k, int s, int j, int t) const;
-  __device__ __forceinline__ int fixF() const { return cur_fix(f); }   // this step's fraction bits
+  __device__ __forceinline__ int fixF() const;                         // this step's fraction bits
 };
 
 // h^2 D_b at the face boundary site nb = c + dir e_k (Eqs. BCDlap, BCMSDlap;
@@ -280,8 +291,11 @@ __device__ __forceinline__ longlong2 fix2(double2 v, int F) { return make_longlo
 // 2^-F always follows the state's own scale.  The stencil sums are formed at
 // that scale and converted to units of cLF = cL 2^-F0 (F0: the reference
 // scale fixed at creation) by an exact power-of-two exponent shift.
-template <class T>
-__device__ __forceinline__ int cur_fix(const Field<T>& f) { return f.Fdev ? __ldg(f.Fdev) : f.F; }
+template <class T, bool ORDERED = false>
+__device__ __forceinline__ int cur_fix(const Field<T>& f) {
+  if (!f.Fdev) return f.F;
+  return ORDERED ? *f.Fdev : __ldg(f.Fdev);
+}
 
 // Biased IEEE-754 exponent of |v|: 0 for zero and subnormals, 2047 for Inf/NaN.
 __device__ __forceinline__ unsigned int expo_bits(double v) { return (unsigned int)(__double2hiint(v) >> 20) & 0x7FFu; }
@@ -300,7 +314,7 @@ __device__ __forceinline__ unsigned int range_bits(float v) { return 0u; }
 // large).  Every lane of the warp must call it.
 __device__ __forceinline__ void emax_commit(unsigned int* p, unsigned int e) {
   e = __reduce_max_sync(0xffffffffu, e);
-  if ((threadIdx.x & 31) == 0 && e > __ldcg(p)) atomicMax(p, e);
+  if ((threadIdx.x & 31) == 0 && e > *(volatile const unsigned int*)p) atomicMax(p, e);
 }
 __device__ __forceinline__ bool fbad(longlong2 v) { return (v.x == kFixBad) | (v.y == kFixBad); }
 
@@ -549,15 +563,15 @@ __device__ __forceinline__ double2 a_lap_exact_deep(const Field<T>& f, const Acc
   return {i2d_rn(Sx, eadj), i2d_rn(Sy, eadj)};
 }
 
-template <class T, int D>
-__device__ __forceinline__ longlong2 GAcc<T, D>::fx0() const { return fix2(ld2<double>(f.in, c), cur_fix(f)); }
-template <class T, int D>
-__device__ __forceinline__ longlong2 GAcc<T, D>::fx1(int k, int s) const {
-  return fix2(ld2<double>(f.in, c + s * f.st[k]), cur_fix(f));
-}
-template <class T, int D>
-__device__ __forceinline__ longlong2 GAcc<T, D>::fx2(int k, int s, int j, int t) const {
-  return fix2(ld2<double>(f.in, c + s * f.st[k] + t * f.st[j]), cur_fix(f));
+template <class T, int D, bool ORDERED>
+__device__ __forceinline__ int GAcc<T, D, ORDERED>::fixF() const { return cur_fix<T, ORDERED>(f); }
+template <class T, int D, bool ORDERED>
+__device__ __forceinline__ longlong2 GAcc<T, D, ORDERED>::fx0() const { return fix2(at0(), fixF()); }
+template <class T, int D, bool ORDERED>
+__device__ __forceinline__ longlong2 GAcc<T, D, ORDERED>::fx1(int k, int s) const { return fix2(at1(k, s), fixF()); }
+template <class T, int D, bool ORDERED>
+__device__ __forceinline__ longlong2 GAcc<T, D, ORDERED>::fx2(int k, int s, int j, int t) const {
+  return fix2(at2(k, s, j, t), fixF());
 }
 
 // Everything a stage writes, on top of the field it reads.

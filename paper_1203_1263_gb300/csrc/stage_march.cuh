@@ -48,10 +48,10 @@ __global__ void __launch_bounds__(256, 4) k_stage3d_march(const StageArgs<T> A, 
   const int64_t plane = (int64_t)f.n[1] * nx;
   int64_t c = zb * plane + (int64_t)gy * nx + gx;
   const float2* in = f.in + c;
-  float2 w[5];   // the column's planes z-2 .. z+2
+  float2 w[5];   // the column's planes z-2 .. z+2 (ordinary loads, see ld2_ordered)
 #pragma unroll
-  for (int d = 0; d < 4; ++d) w[d] = (ORDER == 4 || d > 0) ? __ldg(in + (d - 2) * plane) : float2{0.f, 0.f};
-  float2 next = __ldg(in + (ORDER == 4 ? 2 : 1) * plane);
+  for (int d = 0; d < 4; ++d) w[d] = (ORDER == 4 || d > 0) ? in[(d - 2) * plane] : float2{0.f, 0.f};
+  float2 next = in[(ORDER == 4 ? 2 : 1) * plane];
   if (ORDER == 2) { w[3] = next; }
   const bool with_v = f.V != nullptr;
   PointVals<T> pn = load_point<T, S>(A, c, with_v);
@@ -60,15 +60,15 @@ __global__ void __launch_bounds__(256, 4) k_stage3d_march(const StageArgs<T> A, 
   // the eight in-plane neighbours, loaded a plane ahead
   float2 xm, xp, ym, yp, xm2, xp2, ym2, yp2;
   auto neighbours = [&]() {
-    xm = __ldg(in - 1);
-    xp = __ldg(in + 1);
-    ym = __ldg(in - nx);
-    yp = __ldg(in + nx);
+    xm = in[-1];
+    xp = in[1];
+    ym = in[-nx];
+    yp = in[nx];
     if constexpr (ORDER == 4) {
-      xm2 = __ldg(in - 2);
-      xp2 = __ldg(in + 2);
-      ym2 = __ldg(in - 2 * nx);
-      yp2 = __ldg(in + 2 * nx);
+      xm2 = in[-2];
+      xp2 = in[2];
+      ym2 = in[-2 * nx];
+      yp2 = in[2 * nx];
     }
   };
   neighbours();
@@ -77,7 +77,7 @@ __global__ void __launch_bounds__(256, 4) k_stage3d_march(const StageArgs<T> A, 
     if (ORDER == 4) w[4] = next;
     else w[3] = next;
     if (z + 1 < ze) {
-      next = __ldg(in + (ORDER == 4 ? 3 : 2) * plane);
+      next = in[(ORDER == 4 ? 3 : 2) * plane];
       pn = load_point<T, S>(A, c + plane, with_v);
     }
     const float2 pc = w[2];

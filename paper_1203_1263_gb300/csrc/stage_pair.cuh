@@ -34,8 +34,8 @@ template <int ORDER, bool WALL>
 __device__ __forceinline__ double pair_rhs(const Field<P64>& f, const int* idx, int64_t c, int k, double2* pc_out, double* m2_out) {
   constexpr int D = 3;
   const double* in = reinterpret_cast<const double*>(f.in) + k;   // component k of the field
-  auto at = [&](int64_t i) { return __ldg(in + 2 * i); };
-  const double2 pc = __ldg(f.in + c);
+  auto at = [&](int64_t i) { return in[2 * i]; };   // ordinary loads, see ld2_ordered
+  const double2 pc = f.in[c];
   const double v = ldv<double>(f.V, c);
   double u1[D], w1[D], hi[D], lo[D];
   double2 pb[D];
@@ -55,7 +55,7 @@ __device__ __forceinline__ double pair_rhs(const Field<P64>& f, const int* idx, 
   // a wall's ghost operands, of the lower wall first
   auto load_wall = [&](int a, int64_t d) {
     const int64_t b = c + d;
-    pb[a] = __ldg(f.in + b);
+    pb[a] = f.in[b];
     vb[a] = ldv<double>(f.V, b);
 #pragma unroll
     for (int j = 0; j < D; ++j) {
@@ -187,7 +187,7 @@ __global__ void __launch_bounds__(128) k_stage_pair(const StageArgs<P64> A, unsi
     F = pair_rhs<ORDER, true>(f, idx, c, k, &pc, &m2);
   }
   if (kind == 0 && f.bc != BC_DIRICHLET) {   // see serve_walls
-    const double2 pb = __ldg(f.in + site);
+    const double2 pb = f.in[site];
     double th = 0.0;                         // what turns Psi_b into F_b / i
     if (f.bc == BC_MSD) {
       const double o = __shfl_xor_sync(0xffffffffu, F, 1);

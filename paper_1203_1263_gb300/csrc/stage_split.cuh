@@ -11,7 +11,8 @@
 // waiting for that site's thread.  The arithmetic is site_rhs, serve_walls and
 // rk_apply as everywhere, so results are bit-for-bit those of one thread per
 // interior site (21^3 FP64 2SHOC MSD: 37.7 against 60.5 us per step; small FP64
-// grids: stage_pair.cuh).
+// grids: stage_pair.cuh).  The kernel may start before the one before it has
+// ended, so it reads what that wrote by ordinary loads (ld2_ordered).
 #pragma once
 #include "nlse_internal.h"
 #include "stage_generic.cuh"
@@ -78,7 +79,7 @@ __device__ __forceinline__ unsigned int shell_site(const StageArgs<T>& A, int64_
   if (t >= n) return 0u;
   int idx[D];
   const int64_t c = shell_decode<T, D, I>(A.f, I(t), idx);
-  const GAcc<T, D> acc(A.f, c);
+  const GAcc<T, D, true> acc(A.f, c);
   const PointVals<T> p = load_point<T, -1, EXACT>(A, c, true);
   typename V2<typename T::R>::t pc;
   typename T::R m2w;
@@ -97,14 +98,14 @@ __device__ __forceinline__ unsigned int boundary_site(const StageArgs<T>& A, int
   const PointVals<T> p = load_point<T, -1, EXACT>(A, b, true);
   C2 Fb = {R(0), R(0)};
   if (f.bc == BC_MSD) {   // see serve_walls
-    const C2 pb = ld2<R>(f.in, b);
+    const C2 pb = ld2_ordered<R>(f.in, b);
     int64_t c = 0;
 #pragma unroll
     for (int k = 0; k < D; ++k) {
       idx[k] = min(max(idx[k], 1), f.n[k] - 2);
       c += idx[k] * f.st[k];
     }
-    const GAcc<T, D> acc(f, c);
+    const GAcc<T, D, true> acc(f, c);
     C2 pc;
     R m2w;
     const C2 F = site_rhs<T, D, ORDER, EXACT>(f, acc, idx, c, ldv<R>(EXACT ? A.Vs : f.V, c), &pc, &m2w);
@@ -113,7 +114,7 @@ __device__ __forceinline__ unsigned int boundary_site(const StageArgs<T>& A, int
     if (EXACT ? m2 > R(0) : m2 > f.tiny) theta = fma(F.y, pc.x, -(F.x * pc.y)) / m2;
     Fb = {-theta * pb.y, theta * pb.x};
   } else if (f.bc == BC_L0) {
-    const C2 pb = ld2<R>(f.in, b);
+    const C2 pb = ld2_ordered<R>(f.in, b);
     const R Nb = fma(EXACT ? f.sG : f.s, norm2(pb), -p.v);
     Fb = {-Nb * pb.y, Nb * pb.x};
   }
@@ -142,13 +143,13 @@ __global__ void __launch_bounds__(256) k_stage_split(const StageArgs<T> A, unsig
         rem = q;
         c += idx[k] * f.st[k];
       }
-      const GAcc<T, D> acc(f, c);
+      const GAcc<T, D, true> acc(f, c);
       const PointVals<T> p = load_point<T, -1, EXACT>(A, c, true);
       const C2 pc = acc.at0();
       const R N = fma(EXACT ? f.sG : f.s, norm2(pc), -p.v);
       C2 aL;
       if constexpr (EXACT) aL = a_lap_exact_deep<T, D, ORDER>(f, acc, idx, c, pc, N);
-      else aL = a_lap_body<T, D, ORDER, GAcc<T, D>, false>(f, acc, idx, c, pc, N);
+      else aL = a_lap_body<T, D, ORDER, GAcc<T, D, true>, false>(f, acc, idx, c, pc, N);
       ex = rk_apply<T>(A, c, {-fma(N, pc.y, aL.y), fma(N, pc.x, aL.x)}, p);
     }
   } else if (blockIdx.x < b2) {

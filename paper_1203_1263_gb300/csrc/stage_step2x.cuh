@@ -122,7 +122,7 @@ struct Step2xTile {
     rows([&](int e, int64_t g) {
       Step2Tile<P32, ORDER, TX, NT, 2>::template copy_async<16>(smem_addr(P + e), A.in + (g < 0 ? 0 : g), g < 0 ? 0 : 16);
     });
-    const unsigned int E = __ldcg(A.expo + A.turn);
+    const unsigned int E = *(volatile const unsigned int*)(A.expo + A.turn);   // after grid_wait()
     F = (E > 0u && E < 2047u ? 1077 - int(E) : A.F0) + A.fix_offset;
     eadj = A.F0 - F;
     if (blockIdx.x == 0 && threadIdx.x == 0) A.expo[(A.turn + 2) & 3] = 0u;
