@@ -33,6 +33,6 @@ def test_an_overflowing_mass_is_not_finite(n, at, dtype):
 @pytest.mark.parametrize("shape", [(257,), (60, 70), (11, 20, 30)])
 @pytest.mark.parametrize("bc", ["dirichlet", "periodic"])
 def test_an_overflowing_energy_is_not_finite(shape, bc):
-    psi = np.full(shape, 0.9e154, complex)     # a smooth state: V |Psi|^2 = 0.81e308 at each interior site, s = 0
-    g = Integrator(psi, 1.0, 1e-3, 0.0, np.ones(shape), bc, 4, "c128")
+    # V |Psi|^2 = 0.6e308 at each interior site; |Psi|^4 and a |Psi Lap Psi| stay in range
+    g = Integrator(np.full(shape, 1e74, complex), 1.0, 1e160, 0.0, np.full(shape, 0.6e160), bc, 4, "c128")
     assert not math.isfinite(g.energy())
