@@ -28,16 +28,17 @@ cudaError_t launch_stage(const StageArgs<T>& A, const LaunchCfg& L, cudaStream_t
     }
     if constexpr (fp64) if (exact) return launch_split<T, D, ORDER, true>(A, stream, true, true);
     if constexpr (std::is_same<T, P64>::value) {
-      // see the figures in stage_pair.cuh
+      // see the figures in stage_pair.cuh, and walls_apart
       const int64_t sites = (int64_t)A.f.n[0] * A.f.n[1] * A.f.n[2];
-      if (sites <= (ORDER == 4 ? 600000 : 16384)) return launch_pair<ORDER>(A, stream);
+      if (sites <= (ORDER == 4 ? 600000 : 16384) && walls_apart<T, D, ORDER, false>(A.f, true))
+        return launch_pair<ORDER>(A, stream);
     }
     return launch_split<T, D, ORDER>(A, stream, true, true);
   }
   if constexpr (!fp64) {
     // a few million sites, or rows TMA cannot take: one launch (see the figures in stage_march.cuh; the hook that
     // drives the TMA kernels' bounded waits keeps those)
-    const bool small = (int64_t)A.f.n[0] * A.f.n[1] * A.f.n[2] <= 3000000;
+    const bool small = (int64_t)A.f.n[0] * A.f.n[1] * A.f.n[2] <= 3000000 && !march_thin<ORDER>(A.f);
     if (A.stage >= 1 && (small || !L.tmap) && march_ok(A.f.n, A.f.bc) && !L.extra_tx)
       return launch_march<T, ORDER>(A, stream);
   }

@@ -115,6 +115,18 @@ inline bool has_deep(int D, const int* m) {
   return true;
 }
 
+template <class T, int D, int ORDER, bool EXACT, class I>
+__global__ void __launch_bounds__(256) k_stage_shell(const StageArgs<T> A, int64_t nshell) {
+  const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  unsigned int ex = 0;
+  if (t < nshell) {
+    int idx[D];
+    const int64_t c = shell_decode<T, D, I>(A.f, I(t), idx);
+    ex = process_site<T, D, ORDER, EXACT>(A, GAcc<T, D>(A.f, c), idx, c);
+  }
+  if (A.emax) emax_commit(A.emax, ex);
+}
+
 // CTA size of the one-thread-per-site kernels: 256 threads, halved (down to
 // one warp) while the grid would give fewer than two CTAs per SM.  On small
 // grids this spreads the sites over all SMs, which matters most on the FP64
@@ -164,6 +176,17 @@ __global__ void __launch_bounds__(256) k_stage_generic_periodic(const StageArgs<
     ex = process_site_periodic<T, D, ORDER, EXACT>(A, idx, c);
   }
   if (A.emax) emax_commit(A.emax, ex);
+}
+
+template <class T, int D, int ORDER, bool EXACT = false>
+cudaError_t launch_shell(const StageArgs<T>& A, cudaStream_t stream) {
+  const int64_t ns = shell_count(D, A.f.m);
+  if (ns <= 0) return cudaSuccess;
+  const int threads = site_kernel_threads(ns);
+  const dim3 grid((unsigned)((ns + threads - 1) / threads));
+  if (A.f.ninterior < (int64_t(1) << 31)) k_stage_shell<T, D, ORDER, EXACT, uint32_t><<<grid, threads, 0, stream>>>(A, ns);
+  else k_stage_shell<T, D, ORDER, EXACT, uint64_t><<<grid, threads, 0, stream>>>(A, ns);
+  return cudaGetLastError();
 }
 
 template <class T, int D, int ORDER, bool EXACT = false>

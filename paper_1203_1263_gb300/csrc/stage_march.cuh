@@ -130,6 +130,14 @@ inline bool march_ok(const int* n, int bc) {
   return bc != BC_PERIODIC && n[0] >= 5 && n[1] >= 5 && n[2] >= 5 && (int64_t)n[0] * n[1] * n[2] < (int64_t(1) << 31);
 }
 
+// Flat grids that are mostly MSD walls: with a thread per boundary site (walls_apart) they are slower than the tiles
+// with a thread per wall site (2SHOC, this form and that: 6x600x700 142 and 131, 700x6x700 198 and 173; 6x300x300 38
+// and 43, 700x700x6 410 and 470).
+template <int ORDER, class T>
+inline bool march_thin(const Field<T>& f) {
+  return ORDER == 4 && f.bc == BC_MSD && (f.n[0] < 8 || f.n[1] < 8) && boundary_count(3, f.n, f.m) > 500000;
+}
+
 template <class T, int ORDER>
 cudaError_t launch_march(const StageArgs<T>& A, cudaStream_t stream) {
   switch (A.stage) {

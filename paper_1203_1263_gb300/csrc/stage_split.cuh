@@ -8,7 +8,7 @@
 // deep sites, the sites next to a wall and the boundary sites are three ranges of
 // blocks: warps hold one kind, and a boundary site has a thread of its own, which
 // evaluates F at its interior neighbour once more (MSD; Eq. msd) instead of
-// waiting for that site's thread.  The arithmetic is site_rhs, serve_walls and
+// waiting for that site's thread (where that pays: walls_apart).  The arithmetic is site_rhs, serve_walls and
 // rk_apply as everywhere, so results are bit-for-bit those of one thread per
 // interior site (21^3 FP64 2SHOC MSD: 37.7 against 60.5 us per step; small FP64
 // grids: stage_pair.cuh).  The kernel may start before the one before it has
@@ -160,10 +160,49 @@ __global__ void __launch_bounds__(256) k_stage_split(const StageArgs<T> A, unsig
   if (A.emax) emax_commit(A.emax, ex);
 }
 
+// Whether the boundary sites get threads of their own, in a launch of every site (deep) or of the walls alone.  With
+// MSD walls such a thread evaluates its interior neighbour's F a second time: that pays while the walls are latency
+// beside the rest, and costs once they are work for the whole chip.  us per step, 2SHOC, MSD, one thread per interior
+// site and this form:
+//   every site, FP64 stencil   12x5000 48 / 42, 5x6000 37 / 33, 64^3 282 / 173; 3x20000 40 / 61, 9x200x300 324 / 369
+//   every site, exact sums     21^3 89 / 81, 46^3 129 / 99, 64^3 222 / 144; 33^3 85 / 95, 5x6000 48 / 59
+//   walls, exact sums          500^2 59 / 57, 3x40x40 91 / 78; 60x4000 61 / 65, 12x5000 51 / 63, 6x300x300 202 / 287
+//   walls, FP64 stencil, 3D    3x40x40 65 / 37, 3x100x100 64 / 54; 100x5x100 68 / 72, 6x300x300 331 / 434
+//   FP32                       700x700x9 (every site) 400 / 329; 6x600x700 (walls) 131 / 145
+// (central differences, whose F is cheaper, later: walls, exact sums 200x200x4 53 / 45, 6x300x300 112 / 118).  The other
+// boundaries' sites are a few instructions, apart in all but the largest exact-sum shells (Dirichlet 6x200000 262 / 303,
+// 3x300x400 159 / 128).  Planes of the FP64 stencil: the tiles' CTAs pile up on the SMs that short wall CTAs leave free,
+// from 40,000 to 110,000 sites (Dirichlet 128^2 30 / 22, 256^2 47 / 48, 100x700 48 / 83, 282^2 48 / 61, 500^2 110 / 107).
+template <class T, int D, int ORDER, bool EXACT>
+inline bool walls_apart(const Field<T>& f, bool deep) {
+  int64_t total = 1;
+  bool has_tiles = true;
+  for (int k = 0; k < D; ++k) {
+    total *= f.n[k];
+    has_tiles &= f.n[k] >= 5;
+  }
+  const int64_t n3 = boundary_count(D, f.n, f.m);
+  const bool msd = f.bc == BC_MSD;
+  if constexpr (!std::is_same<typename T::R, double>::value) return !msd || n3 <= (deep && D == 3 ? total : 300000);
+  if (deep) {
+    if (!msd) return true;
+    if (EXACT) return n3 <= (ORDER == 4 ? 1500 : 600000) || n3 * (D == 2 ? 16 : 8) <= total;
+    return n3 <= 24000 || n3 * (D == 2 ? 16 : 10) <= total;
+  }
+  if (EXACT) {
+    if (!msd) return n3 <= (D == 2 ? 100000 : 250000);
+    return n3 <= (ORDER == 4 ? 3500 : (D == 2 ? 16000 : 100000));
+  }
+  if (D == 2 && has_tiles && total > 32768) return false;
+  return !msd || n3 <= (has_tiles && ORDER == 4 && D == 3 ? 4000 : 24000);
+}
+
 // Every site (deep: the tiled kernels' part left out).  `early`: on the step's own stream, where the kernel before may
 // still run.
 template <class T, int D, int ORDER, bool EXACT = false>
 cudaError_t launch_split(const StageArgs<T>& A, cudaStream_t stream, bool deep, bool early) {
+  if (!walls_apart<T, D, ORDER, EXACT>(A.f, deep))
+    return deep ? launch_generic<T, D, ORDER, EXACT>(A, stream) : launch_shell<T, D, ORDER, EXACT>(A, stream);
   int64_t n1 = 1;
   for (int k = 0; k < D; ++k) n1 *= A.f.n[k] > 4 ? A.f.n[k] - 4 : 0;
   const int64_t n2 = A.f.ninterior - n1, n3 = boundary_count(D, A.f.n, A.f.m);
