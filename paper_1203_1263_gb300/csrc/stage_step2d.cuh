@@ -176,20 +176,21 @@ struct Step2Tile {
     const int lane = threadIdx.x & 31;
     const uint32_t d0 = static_cast<uint32_t>(__cvta_generic_to_shared(dst));
     const char* s0 = static_cast<const char*>(src);
-    if (A.bc == BC_PERIODIC) {
-      for (int r = threadIdx.x >> 5; r < H; r += NT / 32) {
-        const int gy = (((oy + r) % ny) + ny) % ny;
-        for (int q = lane; q < W; q += 32) {
-          const int gx = (((ox + q) % nx) + nx) % nx;
-          copy_async<B>(d0 + (r * W + q) * B, s0 + ((int64_t)gy * nx + gx) * B, B);
-        }
-      }
-      return;
-    }
+    const bool periodic = A.bc == BC_PERIODIC;
+    const bool wrap_x = periodic && (ox < 0 || ox + W > nx);
+    const int x0 = wrap_x ? ((ox % nx) + nx) % nx : ox;   // column of the tile's first one
     for (int r = threadIdx.x >> 5; r < H; r += NT / 32) {
-      const int gy = oy + r;
+      int gy = oy + r;
+      if (periodic && (gy < 0 || gy >= ny)) gy = ((gy % ny) + ny) % ny;
       const bool in_y = gy >= 0 && gy < ny;
       const char* row = s0 + ((int64_t)(in_y ? gy : 0) * nx) * B;
+      if (wrap_x) {   // only the tiles at an end of the rows (1000^2 FP32: 37 us per step with every column wrapped)
+        for (int q = lane; q < W; q += 32) {
+          const int g = x0 + q, gx = nx >= W ? (g >= nx ? g - nx : g) : g % nx;
+          copy_async<B>(d0 + (r * W + q) * B, row + (int64_t)gx * B, B);
+        }
+        continue;
+      }
 #pragma unroll
       for (int q0 = 0; q0 < W; q0 += 32) {
         const int q = q0 + lane, gx = ox + q;
