@@ -328,11 +328,18 @@ bool line_path(const nlse_ctx* c) {
 
 // 1D lines that run several steps per launch: variant 1 (and what runs as it) with the FP64 stencil up to the
 // length the cluster path has, with FP32 stages at any length; and FP64 lines whose default is one thread per site
-// with the FP64 stencil (variant 0: the same arithmetic).
+// with the FP64 stencil (variant 0: the same arithmetic), up to the length where a launch per stage is the faster
+// one: central differences 14,000 sites 7.2 against 9.7 us per step, 18,000 10.6 against 9.9 (MSD 22,000 11.4 and
+// 12.9, 24,000 14.4 and 13.0); 2SHOC periodic 12,000 8.2 and 10.7, 16,000 13.4 and 11.0; 2SHOC between walls 32,768
+// 15.0 and 19.1.
 bool lines_path(const nlse_ctx* c) {
   if (c->d != 1) return false;
   if (c->dtype == NLSE_C128) {
-    if (c->variant == 0) return !c->chosen;
+    if (c->variant == 0) {
+      const bool msd = c->bc == NLSE_BC_MSD;
+      const int64_t longest = c->order == 2 ? (msd ? 22500 : 14500) : (c->bc == NLSE_BC_PERIODIC ? 12500 : int64_t(1) << 15);
+      return !c->chosen && c->n[0] <= longest;
+    }
     return (c->variant == 1 || c->variant == 4) && line_ok(int(c->n[0]), true);
   }
   return c->variant == 1 || c->variant == 2 || c->variant == 4;
