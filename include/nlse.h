@@ -137,7 +137,9 @@ int nlse_energy(nlse_t ctx, double *out_host);
  * state psi_in (same dtype, shape and device as the context's Psi; for
  * NLSE_C64_ACC64 it is float2), written to F_out (same type).  Boundary sites
  * get the boundary condition's time derivative (Eqs. BCDdt, msd).
- * Asynchronous.  For testing the right-hand side on its own.
+ * With the default kernel of an NLSE_C128 plane of up to 80,000 sites it is
+ * the FP64 stencil's.  Asynchronous.  For testing the right-hand side on its
+ * own.
  */
 int nlse_rhs(nlse_t ctx, const void *psi_in, void *F_out);
 

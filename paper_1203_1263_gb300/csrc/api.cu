@@ -184,9 +184,10 @@ Field<T> make_field(const nlse_ctx* c, const void* in) {
 LaunchCfg launch_cfg(const nlse_ctx* c);
 
 template <class T>
-cudaError_t dispatch_stage(const nlse_ctx* c, const StageArgs<T>& A, const void* tmap, cudaStream_t st) {
+cudaError_t dispatch_stage(const nlse_ctx* c, const StageArgs<T>& A, const void* tmap, cudaStream_t st, int variant = -1) {
   LaunchCfg L = launch_cfg(c);
-  L.variant = (c->variant == 4) ? 1 : c->variant;   // single stages of the fused variant: the tiled kernel
+  if (variant < 0) variant = c->variant;
+  L.variant = (variant == 4) ? 1 : variant;   // single stages of the fused variant: the tiled kernel
   L.tmap = tmap;
   switch (c->d * 10 + c->order) {
     case 12: return launch_stage<T, 1, 2>(A, L, st);
@@ -648,16 +649,23 @@ int nlse_create(nlse_t* out, int dims, const int64_t* N, double h, double a, dou
   // several steps per launch (2001 sites: 8.6 with MSD walls against 19.2 for a launch per stage and 23.8
   // with the exact-sum stencil on a cluster; 32,000: 18.6 against 24.4 for the exact-sum stencil one thread
   // per site; 49,000: 23.5 against 25.7).
-  // FP64 planes take the exact-sum stencil where a whole step is one launch (step2x_fits) and above 80,000 sites;
-  // the planes between (274^2 to 282^2, and long or narrow ones) the FP64 stencil, whose error is the smaller one
-  // where the operands' rounding is not taken back (Field::fine) and which is the faster one by launches per stage
-  // (282^2: 49.7 against 56.6; 316^2: 61.1 against 54.0).
+  // FP64 planes take the exact-sum stencil where a whole step is one launch (step2x_fits) and above 80,000 sites
+  // (316^2: 61.1 with the FP64 stencil, 54.0).  The planes between (274^2 to 282^2, and long or narrow ones) take the
+  // FP64 stencil: where the operands' rounding is not taken back (Field::fine) its error is the smaller one (32 steps,
+  // against 64 bits: 100x700 2.3e-16 and 3.0e-16, 5x6000 4.1e-16 and 9.2e-16).  Of its two forms the tiles (100x700
+  // 48.7 against 53 for the exact-sum stencil then, 5x15000 43 against 51 for one thread per site), except on narrow
+  // planes (12x5000: 86 with the tiles, 42 with one thread per site; 100x700 44).  A periodic plane of three or four
+  // rows or columns is too narrow for the whole-step kernel's tiles (3x3 8.2 against 11.4, 3x4800 11.4 against 14.0
+  // us with central differences).
   // The FP32 forms take the tiled kernel on 3D grids above 2^17 sites (64^3: 21.2 against 29.8 for one
   // thread per site, 128^3: 67.5 against 105; 40^3: 16.1 against 16.0).
   c->variant = (dtype == NLSE_C128) ? 2 : 1;
   if (dims == 3 && total <= (dtype == NLSE_C128 ? (int64_t(1) << 15) : (int64_t(1) << 17))) c->variant = 0;
-  if (dims == 2 && dtype == NLSE_C128 && total <= 80000 && !step2x_fits(int(N[0]), int(N[1]), bc == NLSE_BC_PERIODIC))
-    c->variant = 1;
+  if (dims == 2 && dtype == NLSE_C128 && total <= 80000) {
+    const int64_t side = N[0] < N[1] ? N[0] : N[1];
+    if (!step2x_fits(int(N[0]), int(N[1]), bc == NLSE_BC_PERIODIC)) c->variant = side >= 8 && side <= 128 ? 0 : 1;
+    else if (bc == NLSE_BC_PERIODIC && side < 5) c->variant = 1;
+  }
   if (dims == 1 && dtype == NLSE_C128)
     c->variant = (total <= 2500 && line_ok(int(N[0]), true)) ? 1 : (total <= (int64_t(1) << 15) ? 0 : 3);
   c->tile_cfg = -1;
@@ -824,7 +832,11 @@ int nlse_step(nlse_t c, int64_t nsteps, double dt) {
 int nlse_rhs(nlse_t c, const void* psi_in, void* F_out) {
   if (!c || !psi_in || !F_out) return fail(NLSE_EINVAL, "NULL argument");
   cudaError_t e;
-  if (c->exact() && (e = update_fix(c, psi_in, c->stream)) != cudaSuccess) return cuda_fail(e, "scale");
+  // A small plane whose whole step is one launch takes the exact sums for its steps alone (unless the caller chose
+  // them): F by itself is the FP64 stencil, one launch instead of three (256^2 2SHOC 10.5 us, 27 with exact sums).
+  const bool plain = !c->chosen && step2x_path(c);
+  const bool exact = c->exact() && !plain;
+  if (exact && (e = update_fix(c, psi_in, c->stream)) != cudaSuccess) return cuda_fail(e, "scale");
   auto run = [&](auto tag) {
     using T = decltype(tag);
     StageArgs<T> A;
@@ -833,10 +845,10 @@ int nlse_rhs(nlse_t c, const void* psi_in, void* F_out) {
     A.out = (typename T::C*)F_out;
     A.stage = 0;
     A.flag = c->flag();
-    const bool g = std::is_same<T, P64>::value && c->variant >= 2;   // F in units of cLF: scale it back
+    const bool g = std::is_same<T, P64>::value && c->variant >= 2 && !plain;   // F in units of cLF: scale it back
     A.dtc = typename T::R(g ? A.f.cLF : 1.0);
     A.Vs = (g && c->V) ? (const typename T::VR*)c->at(c->lay.vs) : nullptr;
-    return dispatch_stage<T>(c, A, nullptr, c->stream);
+    return dispatch_stage<T>(c, A, nullptr, c->stream, plain ? 0 : -1);
   };
   if (c->dtype == NLSE_C128) e = run(P64{});
   else if (c->dtype == NLSE_C64) e = run(P32{});
