@@ -845,7 +845,7 @@ int nlse_rhs(nlse_t c, const void* psi_in, void* F_out) {
     A.out = (typename T::C*)F_out;
     A.stage = 0;
     A.flag = c->flag();
-    const bool g = std::is_same<T, P64>::value && c->variant >= 2 && !plain;   // F in units of cLF: scale it back
+    const bool g = std::is_same<T, P64>::value && exact;   // F in units of cLF: scale it back
     A.dtc = typename T::R(g ? A.f.cLF : 1.0);
     A.Vs = (g && c->V) ? (const typename T::VR*)c->at(c->lay.vs) : nullptr;
     return dispatch_stage<T>(c, A, nullptr, c->stream, plain ? 0 : -1);
