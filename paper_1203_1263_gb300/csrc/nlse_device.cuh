@@ -116,7 +116,8 @@ struct Field {
   int F;             // exact-sum stencil: the reference fraction bits F0 that cLF and V / cLF are scaled by
   const int* Fdev;   // exact-sum stencil: device word holding the fraction bits of the current state
                      //   (derived from max |Psi| every step; nullptr: use F)
-  int fine;          // exact-sum stencil, 2D: the operands' rounding is taken back (fix_correction)
+  int fine;          // exact-sum stencil, 2D: the operands' rounding is taken back (fix_correction), by kernels of
+                     //   their own (per site and the whole step)
   double cLF;        // exact-sum stencil: cL * 2^-F
   R sG;              // exact-sum stencil: s / cLF
   R invcLF;          // exact-sum stencil: 1 / cLF
@@ -129,9 +130,10 @@ struct Field {
 // at2(k, s, j, t) = Psi(c + s e_k + t e_j), atv(o) = Psi(c + sum_k o_k e_k).
 // GAcc reads global memory (ORDERED: by ld2_ordered); the tiled kernels supply
 // shared-memory accessors.  The arithmetic below never depends on which
-// accessor is used.
-template <class T, int D, bool ORDERED = false>
+// accessor is used (FINE: whether the kernel is built for planes with Field::fine).
+template <class T, int D, bool ORDERED = false, bool FINE = false>
 struct GAcc {
+  static constexpr bool kFine = FINE;
   using R = typename T::R;
   using C2 = typename V2<R>::t;
   const Field<T>& f;
@@ -318,6 +320,13 @@ __device__ __forceinline__ void emax_commit(unsigned int* p, unsigned int e) {
 }
 __device__ __forceinline__ bool fbad(longlong2 v) { return (v.x == kFixBad) | (v.y == kFixBad); }
 
+// Whether a kernel's 2D accessor asks for the correction below.
+template <int D, class Acc>
+__host__ __device__ constexpr bool is_fine() {
+  if constexpr (D == 2) return Acc::kFine;
+  else return false;
+}
+
 // What rounding component v to fixed point left out, in 1/256 of the resolution (-128 .. 127).
 __device__ __forceinline__ int fix_low(double v, int F) {
   const unsigned long long u = (unsigned long long)__double_as_longlong(v);
@@ -479,7 +488,7 @@ __device__ __forceinline__ double2 a_lap_exact(const Field<T>& f, const Acc& acc
       return {aL.x * f.invcLF, aL.y * f.invcLF};
     }
     longlong2 r = {0, 0};
-    if (D == 2 && f.fine) r = fix_correction<T, D, ORDER>(acc, pc, F);
+    if constexpr (is_fine<D, Acc>()) r = fix_correction<T, D, ORDER>(acc, pc, F);
     return {i2d_rn(s1x - 2 * D * cc.x + ((r.x + 128) >> 8), eadj), i2d_rn(s1y - 2 * D * cc.y + ((r.y + 128) >> 8), eadj)};
   }
   const bool wall = near_wall2<D>(idx, f.n);
@@ -505,7 +514,7 @@ __device__ __forceinline__ double2 a_lap_exact(const Field<T>& f, const Acc& acc
   }
   long long Sx = 16 * s1x - s2x - 30 * D * cc.x;
   long long Sy = 16 * s1y - s2y - 30 * D * cc.y;
-  if (D == 2 && f.fine) {
+  if constexpr (is_fine<D, Acc>()) {
     const longlong2 r = fix_correction<T, D, ORDER>(acc, pc, F), r2 = fix_correction2<T, D>(f, acc, idx, wall, F);
     Sx += (r.x + r2.x + 128) >> 8;
     Sy += (r.y + r2.y + 128) >> 8;
@@ -537,7 +546,7 @@ __device__ __forceinline__ double2 a_lap_exact_deep(const Field<T>& f, const Acc
       return {aL.x * f.invcLF, aL.y * f.invcLF};
     }
     longlong2 r = {0, 0};
-    if (D == 2 && f.fine) r = fix_correction<T, D, ORDER>(acc, pc, acc.fixF());
+    if constexpr (is_fine<D, Acc>()) r = fix_correction<T, D, ORDER>(acc, pc, acc.fixF());
     return {i2d_rn(s1x - 2 * D * cc.x + ((r.x + 128) >> 8), eadj), i2d_rn(s1y - 2 * D * cc.y + ((r.y + 128) >> 8), eadj)};
   }
   long long s2x = 0, s2y = 0;
@@ -554,7 +563,7 @@ __device__ __forceinline__ double2 a_lap_exact_deep(const Field<T>& f, const Acc
   }
   long long Sx = 16 * s1x - s2x - 30 * D * cc.x;
   long long Sy = 16 * s1y - s2y - 30 * D * cc.y;
-  if (D == 2 && f.fine) {
+  if constexpr (is_fine<D, Acc>()) {
     const longlong2 r = fix_correction<T, D, ORDER>(acc, pc, acc.fixF()),
                     r2 = fix_correction2<T, D>(f, acc, idx, false, acc.fixF());
     Sx += (r.x + r2.x + 128) >> 8;
@@ -563,14 +572,16 @@ __device__ __forceinline__ double2 a_lap_exact_deep(const Field<T>& f, const Acc
   return {i2d_rn(Sx, eadj), i2d_rn(Sy, eadj)};
 }
 
-template <class T, int D, bool ORDERED>
-__device__ __forceinline__ int GAcc<T, D, ORDERED>::fixF() const { return cur_fix<T, ORDERED>(f); }
-template <class T, int D, bool ORDERED>
-__device__ __forceinline__ longlong2 GAcc<T, D, ORDERED>::fx0() const { return fix2(at0(), fixF()); }
-template <class T, int D, bool ORDERED>
-__device__ __forceinline__ longlong2 GAcc<T, D, ORDERED>::fx1(int k, int s) const { return fix2(at1(k, s), fixF()); }
-template <class T, int D, bool ORDERED>
-__device__ __forceinline__ longlong2 GAcc<T, D, ORDERED>::fx2(int k, int s, int j, int t) const {
+template <class T, int D, bool ORDERED, bool FINE>
+__device__ __forceinline__ int GAcc<T, D, ORDERED, FINE>::fixF() const { return cur_fix<T, ORDERED>(f); }
+template <class T, int D, bool ORDERED, bool FINE>
+__device__ __forceinline__ longlong2 GAcc<T, D, ORDERED, FINE>::fx0() const { return fix2(at0(), fixF()); }
+template <class T, int D, bool ORDERED, bool FINE>
+__device__ __forceinline__ longlong2 GAcc<T, D, ORDERED, FINE>::fx1(int k, int s) const {
+  return fix2(at1(k, s), fixF());
+}
+template <class T, int D, bool ORDERED, bool FINE>
+__device__ __forceinline__ longlong2 GAcc<T, D, ORDERED, FINE>::fx2(int k, int s, int j, int t) const {
   return fix2(at2(k, s, j, t), fixF());
 }
 
@@ -817,8 +828,9 @@ __device__ __forceinline__ unsigned int process_site(const StageArgs<T>& A, cons
 // is then an ordinary site, so 2SHOC is the five-point form everywhere (the
 // identity above needs no wall ghosts).
 // ---------------------------------------------------------------------------
-template <class T, int D>
+template <class T, int D, bool FINE = false>
 struct GAccP {
+  static constexpr bool kFine = FINE;
   using R = typename T::R;
   using C2 = typename V2<R>::t;
   const Field<T>& f;
@@ -861,9 +873,9 @@ __device__ __forceinline__ unsigned int process_site_periodic_acc(const StageArg
   return rk_apply<T>(A, c, {-fma(Nc, pc.y, aL.y), fma(Nc, pc.x, aL.x)}, p);
 }
 
-template <class T, int D, int ORDER, bool EXACT>
+template <class T, int D, int ORDER, bool EXACT, bool FINE = false>
 __device__ __forceinline__ unsigned int process_site_periodic(const StageArgs<T>& A, const int* idx, int64_t c) {
-  return process_site_periodic_acc<T, D, ORDER, EXACT>(A, GAccP<T, D>(A.f, c, idx), idx, c);
+  return process_site_periodic_acc<T, D, ORDER, EXACT>(A, GAccP<T, D, FINE>(A.f, c, idx), idx, c);
 }
 
 // How a stage is launched: kernel variant, CTA tile, and (3D tiled kernel)

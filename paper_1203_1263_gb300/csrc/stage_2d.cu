@@ -12,8 +12,9 @@ cudaError_t launch_stage(const StageArgs<T>& A, const LaunchCfg& L, cudaStream_t
   const int variant = (!fp64 && L.variant >= 2) ? L.variant - 2 : L.variant;   // exact sums are FP64 only
   const bool exact = variant >= 2;
   const bool periodic = A.f.bc == BC_PERIODIC;
-  // (the FP32 forms' tiled steps are step2d.cu's; here their one thread per site, and nlse_rhs)
-  if (!fp64 || variant == 0 || variant == 3) {
+  // (the FP32 forms' tiled steps are step2d.cu's, small FP64 planes' exact-sum steps step2x.cu's; here their one thread
+  // per site, and nlse_rhs)
+  if (!fp64 || variant == 0 || variant == 3 || (exact && A.f.fine)) {
     if (periodic) {
       if constexpr (fp64) if (exact) return launch_generic_periodic<T, D, ORDER, true>(A, stream);
       return launch_generic_periodic<T, D, ORDER>(A, stream);

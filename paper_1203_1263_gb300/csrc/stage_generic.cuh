@@ -8,7 +8,7 @@ namespace nlse {
 
 // I = index type of the site decode: uint32_t whenever the count fits
 // (64-bit integer division is a long software sequence on the GPU).
-template <class T, int D, int ORDER, bool EXACT, class I>
+template <class T, int D, int ORDER, bool EXACT, class I, bool FINE = false>
 __global__ void __launch_bounds__(256) k_stage_generic(const StageArgs<T> A) {
   const int64_t t64 = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   unsigned int ex = 0;
@@ -24,7 +24,7 @@ __global__ void __launch_bounds__(256) k_stage_generic(const StageArgs<T> A) {
       idx[k] = int(q) + 1;
       c += idx[k] * A.f.st[k];
     }
-    const GAcc<T, D> acc(A.f, c);
+    const GAcc<T, D, false, FINE> acc(A.f, c);
     ex = process_site<T, D, ORDER, EXACT>(A, acc, idx, c);
   }
   if (A.emax) emax_commit(A.emax, ex);
@@ -158,7 +158,7 @@ __global__ void __launch_bounds__(256) k_stage_shell_periodic(const StageArgs<T>
   if (A.emax) emax_commit(A.emax, ex);
 }
 
-template <class T, int D, int ORDER, bool EXACT, class I>
+template <class T, int D, int ORDER, bool EXACT, class I, bool FINE = false>
 __global__ void __launch_bounds__(256) k_stage_generic_periodic(const StageArgs<T> A, int64_t total) {
   const int64_t t64 = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   unsigned int ex = 0;
@@ -173,7 +173,7 @@ __global__ void __launch_bounds__(256) k_stage_generic_periodic(const StageArgs<
       rem /= nk;
       c += idx[k] * A.f.st[k];
     }
-    ex = process_site_periodic<T, D, ORDER, EXACT>(A, idx, c);
+    ex = process_site_periodic<T, D, ORDER, EXACT, FINE>(A, idx, c);
   }
   if (A.emax) emax_commit(A.emax, ex);
 }
@@ -206,6 +206,12 @@ cudaError_t launch_generic_periodic(const StageArgs<T>& A, cudaStream_t stream) 
   for (int k = 0; k < D; ++k) total *= A.f.n[k];
   const int threads = site_kernel_threads(total);
   const int64_t blocks = (total + threads - 1) / threads;
+  if constexpr (D == 2 && EXACT) {   // fine planes are small
+    if (A.f.fine) {
+      k_stage_generic_periodic<T, D, ORDER, EXACT, uint32_t, true><<<dim3((unsigned)blocks), threads, 0, stream>>>(A, total);
+      return cudaGetLastError();
+    }
+  }
   if (total < (int64_t(1) << 31))
     k_stage_generic_periodic<T, D, ORDER, EXACT, uint32_t><<<dim3((unsigned)blocks), threads, 0, stream>>>(A, total);
   else
@@ -218,6 +224,12 @@ cudaError_t launch_generic(const StageArgs<T>& A, cudaStream_t stream) {
   if (A.f.ninterior <= 0) return cudaSuccess;
   const int threads = site_kernel_threads(A.f.ninterior);
   const int64_t blocks = (A.f.ninterior + threads - 1) / threads;
+  if constexpr (D == 2 && EXACT) {
+    if (A.f.fine) {
+      k_stage_generic<T, D, ORDER, EXACT, uint32_t, true><<<dim3((unsigned)blocks), threads, 0, stream>>>(A);
+      return cudaGetLastError();
+    }
+  }
   if (A.f.ninterior < (int64_t(1) << 31))
     k_stage_generic<T, D, ORDER, EXACT, uint32_t><<<dim3((unsigned)blocks), threads, 0, stream>>>(A);
   else

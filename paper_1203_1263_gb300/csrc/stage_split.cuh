@@ -74,12 +74,12 @@ inline int64_t boundary_count(int D, const int* n, const int* m) {
 }
 
 // The t-th of n sites next to the walls, without the boundary sites it serves.
-template <class T, int D, int ORDER, bool EXACT, class I>
+template <class T, int D, int ORDER, bool EXACT, class I, bool FINE = false>
 __device__ __forceinline__ unsigned int shell_site(const StageArgs<T>& A, int64_t t, int64_t n) {
   if (t >= n) return 0u;
   int idx[D];
   const int64_t c = shell_decode<T, D, I>(A.f, I(t), idx);
-  const GAcc<T, D, true> acc(A.f, c);
+  const GAcc<T, D, true, FINE> acc(A.f, c);
   const PointVals<T> p = load_point<T, -1, EXACT>(A, c, true);
   typename V2<typename T::R>::t pc;
   typename T::R m2w;
@@ -87,7 +87,7 @@ __device__ __forceinline__ unsigned int shell_site(const StageArgs<T>& A, int64_
 }
 
 // The t-th of n boundary sites.
-template <class T, int D, int ORDER, bool EXACT, class I>
+template <class T, int D, int ORDER, bool EXACT, class I, bool FINE = false>
 __device__ __forceinline__ unsigned int boundary_site(const StageArgs<T>& A, int64_t t, int64_t n) {
   using R = typename T::R;
   using C2 = typename V2<R>::t;
@@ -105,7 +105,7 @@ __device__ __forceinline__ unsigned int boundary_site(const StageArgs<T>& A, int
       idx[k] = min(max(idx[k], 1), f.n[k] - 2);
       c += idx[k] * f.st[k];
     }
-    const GAcc<T, D, true> acc(f, c);
+    const GAcc<T, D, true, FINE> acc(f, c);
     C2 pc;
     R m2w;
     const C2 F = site_rhs<T, D, ORDER, EXACT>(f, acc, idx, c, ldv<R>(EXACT ? A.Vs : f.V, c), &pc, &m2w);
@@ -122,7 +122,7 @@ __device__ __forceinline__ unsigned int boundary_site(const StageArgs<T>& A, int
 }
 
 // Blocks [0, b1): the n1 deep sites; [b1, b2): the n2 shell sites; the rest: the n3 boundary sites.
-template <class T, int D, int ORDER, bool EXACT, class I>
+template <class T, int D, int ORDER, bool EXACT, class I, bool FINE = false>
 __global__ void __launch_bounds__(256) k_stage_split(const StageArgs<T> A, unsigned b1, unsigned b2, int64_t n1, int64_t n2,
                                                      int64_t n3) {
   using R = typename T::R;
@@ -143,19 +143,19 @@ __global__ void __launch_bounds__(256) k_stage_split(const StageArgs<T> A, unsig
         rem = q;
         c += idx[k] * f.st[k];
       }
-      const GAcc<T, D, true> acc(f, c);
+      const GAcc<T, D, true, FINE> acc(f, c);
       const PointVals<T> p = load_point<T, -1, EXACT>(A, c, true);
       const C2 pc = acc.at0();
       const R N = fma(EXACT ? f.sG : f.s, norm2(pc), -p.v);
       C2 aL;
       if constexpr (EXACT) aL = a_lap_exact_deep<T, D, ORDER>(f, acc, idx, c, pc, N);
-      else aL = a_lap_body<T, D, ORDER, GAcc<T, D, true>, false>(f, acc, idx, c, pc, N);
+      else aL = a_lap_body<T, D, ORDER, GAcc<T, D, true, FINE>, false>(f, acc, idx, c, pc, N);
       ex = rk_apply<T>(A, c, {-fma(N, pc.y, aL.y), fma(N, pc.x, aL.x)}, p);
     }
   } else if (blockIdx.x < b2) {
-    ex = shell_site<T, D, ORDER, EXACT, I>(A, (int64_t)(blockIdx.x - b1) * blockDim.x + threadIdx.x, n2);
+    ex = shell_site<T, D, ORDER, EXACT, I, FINE>(A, (int64_t)(blockIdx.x - b1) * blockDim.x + threadIdx.x, n2);
   } else {
-    ex = boundary_site<T, D, ORDER, EXACT, I>(A, (int64_t)(blockIdx.x - b2) * blockDim.x + threadIdx.x, n3);
+    ex = boundary_site<T, D, ORDER, EXACT, I, FINE>(A, (int64_t)(blockIdx.x - b2) * blockDim.x + threadIdx.x, n3);
   }
   if (A.emax) emax_commit(A.emax, ex);
 }
@@ -213,6 +213,9 @@ cudaError_t launch_split(const StageArgs<T>& A, cudaStream_t stream, bool deep, 
   auto run = [&](auto kern) -> cudaError_t {
     return launch_early(early, kern, dim3(b3), dim3((unsigned)threads), 0, stream, A, b1, b2, n1, n2, n3);
   };
+  if constexpr (D == 2 && EXACT) {   // fine planes are small
+    if (A.f.fine) return run(k_stage_split<T, D, ORDER, EXACT, uint32_t, true>);
+  }
   if (A.f.ninterior + n3 < (int64_t(1) << 31)) return run(k_stage_split<T, D, ORDER, EXACT, uint32_t>);
   return run(k_stage_split<T, D, ORDER, EXACT, uint64_t>);
 }
