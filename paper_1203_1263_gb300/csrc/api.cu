@@ -415,8 +415,11 @@ bool step2x_path(const nlse_ctx* c) {
          step2x_fits(int(c->n[0]), int(c->n[1]), c->bc == NLSE_BC_PERIODIC);
 }
 
-// The FP32 forms' 2D grids on the whole-step kernel (the tiled variants).
+// The FP32 forms' 2D grids on the whole-step kernel (the tiled variants); not the mixed form's long periodic planes of
+// three or four rows, whose tiles would be mostly wrapped halo, each row of it rounded from the FP64 master (3x20000
+// 11.9 us per step, one thread per site 9.4; 3x4800 5.5 and 9.8).
 bool step2_path(const nlse_ctx* c) {
+  if (c->dtype == NLSE_C64_ACC64 && c->bc == NLSE_BC_PERIODIC && c->n[0] < 5 && c->n[1] > 12000) return false;
   return c->d == 2 && c->dtype != NLSE_C128 && (c->variant == 1 || c->variant == 2 || c->variant == 4);
 }
 

@@ -13,8 +13,10 @@ cudaError_t launch_stage(const StageArgs<T>& A, const LaunchCfg& L, cudaStream_t
   const bool exact = variant >= 2;
   const bool periodic = A.f.bc == BC_PERIODIC;
   // (the FP32 forms' tiled steps are step2d.cu's, small FP64 planes' exact-sum steps step2x.cu's; here their one thread
-  // per site, and nlse_rhs)
-  if (!fp64 || variant == 0 || variant == 3 || (exact && A.f.fine)) {
+  // per site, and nlse_rhs, which takes the tiles on large periodic planes: F of 1500x1700 FP32 2SHOC 17 against 27 us,
+  // of 128^2 4.2 by either)
+  const bool tiles32 = !fp64 && variant == 1 && periodic && A.stage == 0 && (int64_t)A.f.n[0] * A.f.n[1] > 400000;
+  if ((!fp64 && !tiles32) || variant == 0 || variant == 3 || (exact && A.f.fine)) {
     if (periodic) {
       if constexpr (fp64) if (exact) return launch_generic_periodic<T, D, ORDER, true>(A, stream);
       return launch_generic_periodic<T, D, ORDER>(A, stream);
@@ -23,22 +25,22 @@ cudaError_t launch_stage(const StageArgs<T>& A, const LaunchCfg& L, cudaStream_t
     return launch_split<T, D, ORDER>(A, stream, true, true);
   }
   // tiled: deep interior + the wall shell (periodic grids: the two layers at each end of each axis)
-  if constexpr (fp64) {
-    auto deep = [&](cudaStream_t st) -> cudaError_t {
-      if (exact) return launch2d_tiled<T, ORDER, true>(A, L.tile_cfg, st);
-      return launch2d_tiled<T, ORDER>(A, L.tile_cfg, st);
-    };
-    auto shell = [&](cudaStream_t st) -> cudaError_t {
-      if (periodic) {
-        if (exact) return launch_shell_periodic<T, D, ORDER, true>(A, st);
-        return launch_shell_periodic<T, D, ORDER>(A, st);
-      }
+  auto deep = [&](cudaStream_t st) -> cudaError_t {
+    if constexpr (fp64) if (exact) return launch2d_tiled<T, ORDER, true>(A, L.tile_cfg, st);
+    return launch2d_tiled<T, ORDER>(A, L.tile_cfg, st);
+  };
+  auto shell = [&](cudaStream_t st) -> cudaError_t {
+    if (periodic) {
+      if constexpr (fp64) if (exact) return launch_shell_periodic<T, D, ORDER, true>(A, st);
+      return launch_shell_periodic<T, D, ORDER>(A, st);
+    }
+    if constexpr (fp64) {
       if (exact) return launch_split<T, D, ORDER, true>(A, st, false, false);
       return launch_split<T, D, ORDER>(A, st, false, false);
-    };
-    return launch_deep_and_shell(L, stream, has_deep(D, A.f.m), deep, shell);
-  }
-  return cudaErrorInvalidValue;
+    }
+    return cudaErrorInvalidValue;
+  };
+  return launch_deep_and_shell(L, stream, has_deep(D, A.f.m), deep, shell);
 }
 
 #define INST(T, O) template cudaError_t launch_stage<T, 2, O>(const StageArgs<T>&, const LaunchCfg&, cudaStream_t);
