@@ -261,7 +261,8 @@ int nlse_batch_create(nlse_batch_t *out, int nruns, const nlse_run_desc *runs, v
 int nlse_batch_step(nlse_batch_t b, int64_t nsteps);
 
 /* Tile shape of the batched step kernel: 0 = 32x28 cells with strips of 2 rows per thread, 1 = 64x24 with
- * 2, 2 = 32x28 with 4, 3 = 64x24 with 4, -1 = default (1); it never changes results. */
+ * 2, 2 = 32x28 with 4, 3 = 64x24 with 4, -1 = default (1, or 0 where most sites lie in runs of up to 33 columns);
+ * it never changes results. */
 int nlse_batch_set_tile(nlse_batch_t b, int tile_cfg);
 
 /* Autotuner: time steps of every tile shape on the batch's own runs (three

@@ -50,7 +50,6 @@ int bfail(int code, const char* msg) {
 // The tile shapes of tile_cfg 0..3: columns, largest rows, threads, rows per strip, CTAs per SM.
 struct Shape { int tx, ty, nt, ry, per_sm; };
 constexpr Shape kShapes[4] = {{32, 28, 256, 2, 3}, {64, 24, 256, 2, 2}, {32, 28, 256, 4, 3}, {64, 24, 384, 4, 2}};
-constexpr int kDefaultShape = 1;
 
 template <int CFG>
 __global__ void __launch_bounds__(kShapes[CFG].nt, kShapes[CFG].per_sm)
@@ -95,14 +94,32 @@ struct BatchLayout {
   std::vector<size_t> field_off;   // per run: Psi's copy
 };
 
+// The shape for tile_cfg -1: 64 columns (a smaller share of halo), or 32, three CTAs per SM, where most sites lie in runs
+// that one such column of tiles covers and there is more than a wave of those (us per step, MSD, 2SHOC, with V, shape 1
+// and 0: 20 runs of 4000x8 121.7 and 100.6, of 2000x32 70.6 and 61.2, of 2000x40 76.0 and 97.0; 200 of 16^2 8.8 and 10.8).
+int run_rows(const Shape& s, int64_t ny);
+int default_shape(int nruns, const nlse_run_desc* runs) {
+  int64_t narrow = 0, total = 0, items = 0;
+  for (int r = 0; r < nruns; ++r) {
+    const int64_t sites = runs[r].n[0] * runs[r].n[1];
+    total += sites;
+    if (runs[r].n[1] > 33) continue;
+    narrow += sites;
+    int ntx, nty;
+    step2_tiles(int(runs[r].n[0]), int(runs[r].n[1]), false, kShapes[0].tx, run_rows(kShapes[0], runs[r].n[0]), &ntx, &nty);
+    items += nty;
+  }
+  return 2 * narrow > total && items > 3 * 152 ? 0 : 1;
+}
+
 // Rows of a run's tiles under a shape: its interior in equal parts of at most the shape's rows.
 int run_rows(const Shape& s, int64_t ny) {
   const int64_t ext = ny - 1, parts = (ext + s.ty - 1) / s.ty;
   return int(((ext + parts - 1) / parts + 3) / 4 * 4);
 }
 
-bool layout_batch(int nruns, const nlse_run_desc* runs, int tile_cfg, BatchLayout* L) {
-  const Shape& s = kShapes[tile_cfg < 0 ? kDefaultShape : tile_cfg];
+bool layout_batch(int nruns, const nlse_run_desc* runs, int shape, BatchLayout* L) {
+  const Shape& s = kShapes[shape];
   size_t off = 256;   // bytes 0..255: the status word, at the same place for every tile shape
   auto al = [](size_t x) { return (x + 255) / 256 * 256; };
   L->runs_off = off;
@@ -137,7 +154,7 @@ struct nlse_batch {
   BatchLayout lay;
   cudaStream_t stream, cap;
   cudaGraphExec_t exec;
-  int tile_cfg;
+  int shape;   // of kShapes
   unsigned int* flag() const { return (unsigned int*)ws; }   // fixed: the layout after it depends on the tile shape
 };
 
@@ -156,7 +173,7 @@ cudaError_t launch_shape(const nlse_batch* b, bool back, bool early, cudaStream_
 
 // One step of every run, from Psi into the copies or back (early: not a call's first, see launch_early).
 cudaError_t launch_batch_step(const nlse_batch* b, bool back, bool early, cudaStream_t st) {
-  switch (b->tile_cfg < 0 ? kDefaultShape : b->tile_cfg) {
+  switch (b->shape) {
     case 0: return launch_shape<0>(b, back, early, st);
     case 1: return launch_shape<1>(b, back, early, st);
     case 2: return launch_shape<2>(b, back, early, st);
@@ -180,7 +197,7 @@ cudaError_t launch_batch_copy(const nlse_batch* b, cudaStream_t st) {
 
 // Build the run table and work lists on the host and copy them into the workspace.
 int upload_tables(nlse_batch* b) {
-  const Shape& sh = kShapes[b->tile_cfg < 0 ? kDefaultShape : b->tile_cfg];
+  const Shape& sh = kShapes[b->shape];
   std::vector<BatchRun> runs(b->nruns);
   std::vector<Item> items;
   items.reserve(b->lay.nitems);
@@ -256,7 +273,7 @@ extern "C" {
 size_t nlse_batch_workspace_bytes(int nruns, const nlse_run_desc* runs) {
   if (validate(nruns, runs) != NLSE_OK) return 0;
   BatchLayout L;
-  if (!layout_batch(nruns, runs, -1, &L)) return 0;
+  if (!layout_batch(nruns, runs, default_shape(nruns, runs), &L)) return 0;
   size_t worst = L.total;
   for (int t = 0; t < 4; ++t) {   // room for any tile shape
     BatchLayout Lt;
@@ -278,10 +295,10 @@ int nlse_batch_create(nlse_batch_t* out, int nruns, const nlse_run_desc* runs, v
   b->desc.assign(runs, runs + nruns);
   b->ws = (char*)workspace;
   b->stream = (cudaStream_t)stream;
-  b->tile_cfg = -1;
+  b->shape = default_shape(nruns, runs);
   b->cap = nullptr;
   b->exec = nullptr;
-  layout_batch(nruns, runs, b->tile_cfg, &b->lay);
+  layout_batch(nruns, runs, b->shape, &b->lay);
   cudaError_t e = cudaStreamCreateWithFlags(&b->cap, cudaStreamNonBlocking);
   if (e == cudaSuccess) e = cudaMemsetAsync(b->flag(), 0, 256, b->stream);
   if (e != cudaSuccess) {
@@ -300,8 +317,8 @@ int nlse_batch_create(nlse_batch_t* out, int nruns, const nlse_run_desc* runs, v
 int nlse_batch_set_tile(nlse_batch_t b, int tile_cfg) {
   if (!b) return bfail(NLSE_EINVAL, "NULL batch");
   if (tile_cfg < -1 || tile_cfg > 3) return bfail(NLSE_EINVAL, "tile_cfg must be -1..3");
-  b->tile_cfg = tile_cfg;
-  layout_batch(b->nruns, b->desc.data(), tile_cfg, &b->lay);
+  b->shape = tile_cfg < 0 ? default_shape(b->nruns, b->desc.data()) : tile_cfg;
+  layout_batch(b->nruns, b->desc.data(), b->shape, &b->lay);
   drop_graph(b);
   return upload_tables(b);
 }

@@ -1,5 +1,5 @@
-"""Odd step counts of a batch end in a copy back into every run's Psi: one large run, many tiny ones, and both together
-must match the runs integrated alone, bit for bit."""
+"""Odd step counts of a batch end in a copy back into every run's Psi: one large run, many tiny ones, both together, and
+narrow runs (tiles of 32 columns) must match the runs integrated alone, bit for bit."""
 import numpy as np
 import pytest
 
@@ -8,7 +8,8 @@ from paper_1203_1263_gb300.integrator import BatchIntegrator, Integrator, max_dt
 pytestmark = pytest.mark.gpu
 
 
-@pytest.mark.parametrize("shapes", [[(1501, 903)], [(3, 3)] * 40 + [(5, 17)] * 300, [(1200, 800), (3, 4), (64, 64)]])
+@pytest.mark.parametrize("shapes", [[(1501, 903)], [(3, 3)] * 40 + [(5, 17)] * 300, [(1200, 800), (3, 4), (64, 64)],
+                                    [(2000, 9)] * 12 + [(900, 33), (60, 34)]])
 @pytest.mark.parametrize("steps", [1, 3])
 def test_odd_counts_reach_every_site(shapes, steps):
     dt = 0.2 * max_dt(2, 0.3, 0.7, 4, 0.0, 2.0)
