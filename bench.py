@@ -78,7 +78,7 @@ TRAFFIC_PER_STEP = {  # dtype -> (bytes per step, csrc hash of the capture)
 STAGE3D_SOURCES = ("api.cu", "reduce.cu", "nlse_device.cuh", "nlse_internal.h", "stage_3d_impl.cuh",
                    "stage_3d_p32_o2.cu", "stage_3d_p32_o4.cu", "stage_3d_p64_o2.cu", "stage_3d_p64_o4.cu",
                    "stage_3d_pmix_o2.cu", "stage_3d_pmix_o4.cu", "stage_generic.cuh", "stage_march.cuh", "stage_pair.cuh",
-                   "stage_slab.cuh", "stage_split.cuh", "stage_step2d.cuh", "stage_tiled.cuh", "stage_tma.cuh")
+                   "smem_limit.h", "stage_slab.cuh", "stage_split.cuh", "stage_step2d.cuh", "stage_tiled.cuh", "stage_tma.cuh")
 
 
 def workload_dt(p):

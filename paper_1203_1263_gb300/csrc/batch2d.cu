@@ -165,8 +165,9 @@ cudaError_t launch_shape(const nlse_batch* b, bool back, bool early, cudaStream_
   constexpr Shape s = kShapes[CFG];
   const size_t smem = step2_smem<s.tx>(s.ty, true);
   auto kern = k_batch2d_step<CFG>;
-  static const cudaError_t attr = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
-  if (attr != cudaSuccess) return attr;
+  static SmemLimit limit;
+  const cudaError_t e = limit.allow(kern, 227 * 1024);
+  if (e != cudaSuccess) return e;
   return launch_early(early, kern, dim3((unsigned)b->lay.nitems), dim3(s.nt), smem, st,
                       (const BatchRun*)(b->ws + b->lay.runs_off), (const Item*)(b->ws + b->lay.items_off), back ? 1 : 0);
 }

@@ -4,6 +4,7 @@
 #include <stdint.h>
 
 #include "nlse_device.cuh"
+#include "smem_limit.h"
 #include "stage_step1d.cuh"
 #include "stage_step2d.cuh"
 #include "stage_step2x.cuh"

@@ -273,12 +273,11 @@ cudaError_t launch_fused_kernel(const StageArgs<P32>& A1, const StageArgs<P32>& 
   const int planes = nz - 4;
   const size_t smem = fused_smem_bytes();
   auto kern = k_stage3d_fused<ORDER, S1, TX, kFusedTYT, kFusedRY, kFusedP>;
+  static SmemLimit limit;
+  const cudaError_t e = limit.allow(kern, smem);
+  if (e != cudaSuccess) return e;
   static int per_sm = 0;
-  if (per_sm == 0) {
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-    per_sm = resident_per_sm(kern, TX * kFusedTYT, smem);
-  }
+  if (per_sm == 0) per_sm = resident_per_sm(kern, TX * kFusedTYT, smem);
   // six extra planes: a chunk's rings fill and drain
   int nzc = z_chunks(tiles, planes, per_sm, 6);
   const int zc = (planes + nzc - 1) / nzc;

@@ -411,14 +411,13 @@ cudaError_t launch3d_tma_exact_shape(const StageArgs<T>& A, const CUtensorMap* t
   const int planes = nz - 2;
   const size_t smem = (P + 1 + 6) * G::kSlot + (P + 1) * sizeof(uint64_t);
   auto kern = k_stage3d_tma_exact<T, ORDER, S, TX, TYT, RY, P>;
-  static int per_sm = 0;
-  if (per_sm == 0) {
-    if (smem > 48 * 1024) {
-      cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-      if (e != cudaSuccess) return e;
-    }
-    per_sm = resident_per_sm(kern, TX * TYT, smem);
+  static SmemLimit limit;
+  if (smem > 48 * 1024) {
+    const cudaError_t e = limit.allow(kern, smem);
+    if (e != cudaSuccess) return e;
   }
+  static int per_sm = 0;
+  if (per_sm == 0) per_sm = resident_per_sm(kern, TX * TYT, smem);
   int nzc = z_chunks(tiles, planes, per_sm, 4);
   const int zc = (planes + nzc - 1) / nzc;
   nzc = (planes + zc - 1) / zc;
@@ -437,14 +436,13 @@ cudaError_t launch3d_tma_shape(const StageArgs<T>& A, const CUtensorMap* tm, lon
   const int planes = nz - 2;
   const size_t smem = (5 + P) * G::kSlot + (5 + P) * sizeof(uint64_t);
   auto kern = k_stage3d_tma<T, ORDER, S, TX, TYT, RY, P>;
-  static int per_sm = 0;
-  if (per_sm == 0) {
-    if (smem > 48 * 1024) {
-      cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-      if (e != cudaSuccess) return e;
-    }
-    per_sm = resident_per_sm(kern, TX * TYT, smem);
+  static SmemLimit limit;
+  if (smem > 48 * 1024) {
+    const cudaError_t e = limit.allow(kern, smem);
+    if (e != cudaSuccess) return e;
   }
+  static int per_sm = 0;
+  if (per_sm == 0) per_sm = resident_per_sm(kern, TX * TYT, smem);
   int nzc = z_chunks(tiles, planes, per_sm, 4);
   const int zc = (planes + nzc - 1) / nzc;
   nzc = (planes + zc - 1) / zc;

@@ -60,8 +60,9 @@ cudaError_t launch_shape(const Step2Args<T>& A, int ty, bool early, cudaStream_t
   constexpr Shape s = kShapes[CFG];
   const size_t smem = step2_smem<s.tx>(ty, A.V != nullptr);
   auto kern = k_step2d<T, ORDER, s.tx, s.nt, s.ry, s.per_sm>;
-  static const cudaError_t attr = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
-  if (attr != cudaSuccess) return attr;
+  static SmemLimit limit;
+  const cudaError_t e = limit.allow(kern, 227 * 1024);
+  if (e != cudaSuccess) return e;
   int ntx, nty;
   step2_tiles(A.n[0], A.n[1], A.bc == BC_PERIODIC, s.tx, ty, &ntx, &nty);
   return launch_early(early, kern, dim3((unsigned)(ntx * nty)), dim3(s.nt), smem, stream, A, ty, ntx);

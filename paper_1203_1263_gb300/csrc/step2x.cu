@@ -27,8 +27,9 @@ int tiles(int ny, int nx, bool periodic, int ty, int* ntx) {
 template <int ORDER>
 cudaError_t launch_order(const Step2xArgs& A, int ty, int ntx, int n, bool early, cudaStream_t stream) {
   auto kern = k_step2x<ORDER>;
-  static const cudaError_t attr = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
-  if (attr != cudaSuccess) return attr;
+  static SmemLimit limit;
+  const cudaError_t e = limit.allow(kern, 227 * 1024);
+  if (e != cudaSuccess) return e;
   return launch_early(early, kern, dim3((unsigned)n), dim3(kNT), step2x_smem(kTX, ty, A.V != nullptr), stream, A, ty, ntx);
 }
 
