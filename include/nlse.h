@@ -223,7 +223,9 @@ int nlse_kernel_in_use(nlse_t ctx);
  * timing).  Synchronises the stream.  *best_tile_cfg receives the chosen
  * tile_cfg (-1 when there is none to choose: 1D grids, small FP64 2D grids, variants 0 and 3) and
  * *best_ms the measured stage-2 time (0 when taken from a cache); either
- * pointer may be NULL.  Tiles never change results.
+ * pointer may be NULL.  Where no launch of a step depends on the tile (3D
+ * grids of the FP32 forms on the columns kernel) the default tile is kept.
+ * Tiles never change results.
  */
 int nlse_autotune(nlse_t ctx, int *best_tile_cfg, float *best_ms);
 

@@ -14,6 +14,7 @@
 
 #include "../../include/nlse.h"
 #include "nlse_internal.h"
+#include "stage_march.cuh"
 
 using namespace nlse;
 
@@ -413,6 +414,15 @@ cudaError_t launch_step_fused(const nlse_ctx* c, double dt, cudaStream_t st, voi
 bool step2x_path(const nlse_ctx* c) {
   return c->d == 2 && c->dtype == NLSE_C128 && c->variant == 2 &&
          step2x_fits(int(c->n[0]), int(c->n[1]), c->bc == NLSE_BC_PERIODIC);
+}
+
+// FP32 forms' 3D grids whose steps take the columns kernel: its launches do not depend on the tile.
+bool columns_path(const nlse_ctx* c) {
+  if (c->d != 3 || c->dtype == NLSE_C128 || c->extra_tx) return false;
+  const Field<P32> f = make_field<P32>(c, c->psi);
+  const void* in = c->dtype == NLSE_C64_ACC64 ? c->at(c->lay.pn32) : c->psi;
+  const bool tma = stage_tmap(c, 0, in) != nullptr;
+  return c->order == 4 ? march_serves<4>(f, tma) : march_serves<2>(f, tma);
 }
 
 // The FP32 forms' 2D grids on the whole-step kernel (the tiled variants); not the mixed form's long periodic planes of
@@ -962,13 +972,14 @@ int nlse_autotune(nlse_t c, int* best_tile_cfg, float* best_ms) {
     cudaEvent_t e0, e1;
     cudaEventCreate(&e0);
     cudaEventCreate(&e1);
-    const int saved = c->tile_cfg;
+    const int saved = c->tile_cfg, only = columns_path(c) ? resolved_tile(c) : -1;   // nothing to compare: the default
     best = 1e30f;
     cudaError_t e = cudaSuccess;
     if (c->dtype == NLSE_C64_ACC64)
       e = launch_round_master((const double2*)c->psi, (float2*)c->at(c->lay.pn32), c->total, c->stream);
     if (e == cudaSuccess && c->exact()) e = update_fix(c, c->psi, c->stream);
     for (int t = 0; t < 4 && e == cudaSuccess; ++t) {
+      if (only >= 0 && t != only) continue;
       c->tile_cfg = t;
       const bool step2 = step2_path(c);   // one whole step, into Psi's ping-pong copy
       if (step2) e = launch_step2_any(c, 1e-12, c->stream, c->psi, step_alt(c), 0);

@@ -36,11 +36,8 @@ cudaError_t launch_stage(const StageArgs<T>& A, const LaunchCfg& L, cudaStream_t
     return launch_split<T, D, ORDER>(A, stream, true, true);
   }
   if constexpr (!fp64) {
-    // a few million sites, or rows TMA cannot take: one launch (see the figures in stage_march.cuh; the hook that
-    // drives the TMA kernels' bounded waits keeps those)
-    const bool small = (int64_t)A.f.n[0] * A.f.n[1] * A.f.n[2] <= 3000000 && !march_thin<ORDER>(A.f);
-    if (A.stage >= 1 && (small || !L.tmap) && march_ok(A.f.n, A.f.bc) && !L.extra_tx)
-      return launch_march<T, ORDER>(A, stream);
+    // one launch (the hook that drives the TMA kernels' bounded waits keeps those)
+    if (A.stage >= 1 && !L.extra_tx && march_serves<ORDER>(A.f, L.tmap != nullptr)) return launch_march<T, ORDER>(A, stream);
   }
   // tiled: deep interior (TMA-fed when the layout allows) + the wall shell, as
   // shared-memory slabs (FP32 stages: three x layers per x wall) or, for thin

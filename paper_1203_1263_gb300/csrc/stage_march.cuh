@@ -138,6 +138,13 @@ inline bool march_thin(const Field<T>& f) {
   return ORDER == 4 && f.bc == BC_MSD && (f.n[0] < 8 || f.n[1] < 8) && boundary_count(3, f.n, f.m) > 500000;
 }
 
+// Whether the steps of a grid take the columns: a few million sites, or rows that TMA cannot take (the figures above).
+template <int ORDER, class T>
+inline bool march_serves(const Field<T>& f, bool tma) {
+  const bool small = (int64_t)f.n[0] * f.n[1] * f.n[2] <= 3000000 && !march_thin<ORDER>(f);
+  return (small || !tma) && march_ok(f.n, f.bc);
+}
+
 template <class T, int ORDER>
 cudaError_t launch_march(const StageArgs<T>& A, cudaStream_t stream) {
   switch (A.stage) {
