@@ -20,5 +20,5 @@ def test_the_default_tile_is_kept(shape, default, dtype, chosen, tmp_path, monke
     cfg, ms = g.autotune()
     want = chosen if chosen >= 0 else default
     assert cfg == want and ms > 0
-    lines = (tmp_path / "tune.txt").read_text().split()
+    lines = (tmp_path / "tune.txt").read_text().splitlines()
     assert len(lines) == 1 and lines[0].endswith(f"={want}")
