@@ -325,7 +325,7 @@ LaunchCfg launch_cfg(const nlse_ctx* c) {
 
 // 1D lines that take the cluster path: FP64 with the exact-sum stencil (variant 2).
 bool line_path(const nlse_ctx* c) {
-  return c->d == 1 && !c->line_failed && c->dtype == NLSE_C128 && c->variant == 2 && line_ok(int(c->n[0]), true);
+  return c->d == 1 && !c->line_failed && c->dtype == NLSE_C128 && c->variant == 2 && line_ok(int(c->n[0]));
 }
 
 // 1D lines that run several steps per launch: variant 1 (and what runs as it) with the FP64 stencil up to the
@@ -342,7 +342,7 @@ bool lines_path(const nlse_ctx* c) {
       const int64_t longest = c->order == 2 ? (msd ? 22500 : 14500) : (c->bc == NLSE_BC_PERIODIC ? 12500 : int64_t(1) << 15);
       return !c->chosen && c->n[0] <= longest;
     }
-    return (c->variant == 1 || c->variant == 4) && line_ok(int(c->n[0]), true);
+    return (c->variant == 1 || c->variant == 4) && line_ok(int(c->n[0]));
   }
   return c->variant == 1 || c->variant == 2 || c->variant == 4;
 }
@@ -680,7 +680,7 @@ int nlse_create(nlse_t* out, int dims, const int64_t* N, double h, double a, dou
     else if (bc == NLSE_BC_PERIODIC && side < 5) c->variant = 1;
   }
   if (dims == 1 && dtype == NLSE_C128)
-    c->variant = (total <= 2500 && line_ok(int(N[0]), true)) ? 1 : (total <= (int64_t(1) << 15) ? 0 : 3);
+    c->variant = (total <= 2500 && line_ok(int(N[0]))) ? 1 : (total <= (int64_t(1) << 15) ? 0 : 3);
   c->tile_cfg = -1;
   c->spin_limit = kSpinLimit;
   c->graph_dt = -1.0;

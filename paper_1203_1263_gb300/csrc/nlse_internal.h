@@ -83,7 +83,7 @@ cudaError_t launch_steps1d(const Step1Args<T>& A, int order, int steps, bool ear
 // an n-site line in one launch; A[0..3] are stages 1..4 with Psi updated in
 // place.  cudaErrorInvalidConfiguration when the line does not fit or the
 // cluster cannot be co-scheduled (the caller then takes the per-site kernel).
-bool line_ok(int n, bool fp64);
+bool line_ok(int n);
 cudaError_t launch_line_steps(const StageArgs<P64>* A, int64_t nsteps, int n, int order, int F0, int fix_offset,
                               cudaStream_t stream);
 

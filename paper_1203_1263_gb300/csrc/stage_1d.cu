@@ -22,18 +22,18 @@ cudaError_t launch_stage(const StageArgs<T>& A, const LaunchCfg& L, cudaStream_t
 INST(P64, 2) INST(P64, 4) INST(P32, 2) INST(P32, 4) INST(PMix, 2) INST(PMix, 4)
 #undef INST
 
-bool line_ok(int n, bool fp64) {
+bool line_ok(int n) {
   int cl, seg;
   size_t smem;
-  return line_plan(n, fp64 ? 16 : 8, &cl, &seg, &smem);
+  return line_plan(n, &cl, &seg, &smem);
 }
 
 cudaError_t launch_line_steps(const StageArgs<P64>* A, int64_t nsteps, int n, int order, int F0, int fix_offset,
                               cudaStream_t stream) {
   int cl, seg;
   size_t smem;
-  if (!line_plan(n, sizeof(double2), &cl, &seg, &smem)) return cudaErrorInvalidConfiguration;
-  LineArgs<P64> L;
+  if (!line_plan(n, &cl, &seg, &smem)) return cudaErrorInvalidConfiguration;
+  LineArgs L;
   memset(&L, 0, sizeof(L));
   for (int s = 0; s < 4; ++s) L.A[s] = A[s];
   L.nsteps = nsteps;
@@ -41,7 +41,7 @@ cudaError_t launch_line_steps(const StageArgs<P64>* A, int64_t nsteps, int n, in
   L.seg = seg;
   L.F0 = F0;
   L.fix_offset = fix_offset;
-  return order == 4 ? launch_line1d<P64, 4, true>(L, cl, smem, stream) : launch_line1d<P64, 2, true>(L, cl, smem, stream);
+  return order == 4 ? launch_line1d<4>(L, cl, smem, stream) : launch_line1d<2>(L, cl, smem, stream);
 }
 
 }  // namespace nlse

@@ -114,7 +114,9 @@ cudaError_t launch_march_stage(const StageArgs<T>& A, cudaStream_t stream) {
   const int ntx = (A.f.n[2] - 4 + kMarchTX - 1) / kMarchTX, nty = (A.f.n[1] - 4 + kMarchTY - 1) / kMarchTY;
   const int planes = A.f.n[0] - 4;
   // The wall blocks first and the columns in two waves behind them, or the columns in one wave and the wall blocks
-  // after it (us per step: 64^3 FP32 27.2 and 32.8, 128^3 70.7 and 77.0; mixed form 203x87x87 76.9 and 73.1).
+  // after it: the second for the mixed form above 2^20 sites (us per step, two waves and one, MSD 2SHOC: 100^3 48.8 and
+  // 50.5, 104^3 63.3 and 63.6, 110^3 68.4 and 66.0, 203x87x87 75.9 and 73.2, 140x120x130 95.9 and 88.7, 143^3 141 and
+  // 132; against it 128^3 96.7 and 103.5, 300x64x64 71.0 and 78.0).  FP32: 128^3 72.6 and 81.4, 143^3 104.6 and 94.8.
   const bool one_wave = !std::is_same<typename T::M, typename T::C>::value && A.f.ninterior > (int64_t(1) << 20);
   int nzc = z_chunks(ntx * nty, planes, one_wave ? per_sm : 2 * per_sm, 3);
   const int zc = (planes + nzc - 1) / nzc;
