@@ -66,12 +66,12 @@ __global__ void __launch_bounds__(kShapes[CFG].nt, kShapes[CFG].per_sm)
   }
   const int ty = R.ty, ntx = R.ntx, tx_i = w.tile % ntx, ty_i = w.tile / ntx;
   if (R.order == 4) {
-    Step2Tile<P32, 4, s.tx, s.nt, s.ry> tile(A, ty, tx_i, ty_i, batch_smem);
+    Step2Tile<P32, 4, s.tx, s.nt, s.ry, false> tile(A, ty, tx_i, ty_i, batch_smem);
     tile.load_potential();
     grid_wait();
     tile.run();
   } else {
-    Step2Tile<P32, 2, s.tx, s.nt, s.ry> tile(A, ty, tx_i, ty_i, batch_smem);
+    Step2Tile<P32, 2, s.tx, s.nt, s.ry, false> tile(A, ty, tx_i, ty_i, batch_smem);
     tile.load_potential();
     grid_wait();
     tile.run();

@@ -135,8 +135,8 @@ __device__ __forceinline__ typename T::M final_value(typename T::R dtc, typename
   return q;
 }
 
-// ty (the tile's rows) is a multiple of RY.
-template <class T, int ORDER, int TX, int NT, int RY>
+// ty (the tile's rows) is a multiple of RY.  WRAP: the grid is periodic.
+template <class T, int ORDER, int TX, int NT, int RY, bool WRAP>
 struct Step2Tile {
   using LT = L32;
   using C = float2;
@@ -176,12 +176,11 @@ struct Step2Tile {
     const int lane = threadIdx.x & 31;
     const uint32_t d0 = static_cast<uint32_t>(__cvta_generic_to_shared(dst));
     const char* s0 = static_cast<const char*>(src);
-    const bool periodic = A.bc == BC_PERIODIC;
-    const bool wrap_x = periodic && (ox < 0 || ox + W > nx);
+    const bool wrap_x = WRAP && (ox < 0 || ox + W > nx);
     const int x0 = wrap_x ? ((ox % nx) + nx) % nx : ox;   // column of the tile's first one
     for (int r = threadIdx.x >> 5; r < H; r += NT / 32) {
       int gy = oy + r;
-      if (periodic && (gy < 0 || gy >= ny)) gy = ((gy % ny) + ny) % ny;
+      if (WRAP && (gy < 0 || gy >= ny)) gy = ((gy % ny) + ny) % ny;
       const bool in_y = gy >= 0 && gy < ny;
       const char* row = s0 + ((int64_t)(in_y ? gy : 0) * nx) * B;
       if (wrap_x) {   // only the tiles at an end of the rows (1000^2 FP32: 37 us per step with every column wrapped)
@@ -269,7 +268,7 @@ struct Step2Tile {
     Pair2 col[RY + 4];
 #pragma unroll
     for (int r = ORDER == 4 ? 0 : 1; r < (ORDER == 4 ? RY + 4 : RY + 3); ++r) col[r] = ld_pair(in + e + (r - 2) * W);
-    const int lo = A.bc == BC_PERIODIC ? 0 : 1;   // first updated index
+    const int lo = WRAP ? 0 : 1;   // first updated index
     const bool m0 = !WALLS || (gx >= lo && gx < A.n[1] - lo), m1 = !WALLS || (gx + 1 >= lo && gx + 1 < A.n[1] - lo);
 #pragma unroll
     for (int r = 0; r < RY; ++r) {
@@ -432,7 +431,7 @@ struct Step2Tile {
   __device__ __forceinline__ void strips(const C* in, C* out, bool vec) {
     constexpr int e0 = 2 * (4 - S), RW = TX + 2 * e0;   // the stage's region
     static_assert(12 % RY == 0 && 8 % RY == 0 && 4 % RY == 0, "whole strips");
-    if (WALLS && A.bc != BC_PERIODIC) {
+    if (WALLS && !WRAP) {
       // only the part of the region that holds interior sites (pairs and strips kept on the region's own grid)
       constexpr int R0 = HALO - e0;
       const int lx0 = max(R0, -ox), lx1 = min(R0 + RW, A.n[1] - 1 - ox);
@@ -464,7 +463,7 @@ struct Step2Tile {
   // One stage from `in` to `out` (in: not const, the ghosts go into its cells beyond the walls).
   template <int S, bool WALLS>
   __device__ __forceinline__ void whole(C* in, C* out, bool vec) {
-    const bool walls = WALLS && A.bc != BC_PERIODIC;
+    const bool walls = WALLS && !WRAP;
     if (ORDER == 4 && walls) {
       ghosts<S>(in);
       __syncthreads();

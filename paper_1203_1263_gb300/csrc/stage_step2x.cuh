@@ -111,8 +111,8 @@ struct Step2xTile {
   __device__ __forceinline__ void load_potential() {
     if (with_v)
       rows([&](int e, int64_t g) {
-        Step2Tile<P32, ORDER, TX, NT, 2>::template copy_async<8>(smem_addr(V + e), A.V + (g < 0 ? 0 : g), g < 0 ? 0 : 8);
-        Step2Tile<P32, ORDER, TX, NT, 2>::template copy_async<8>(smem_addr(Vs + e), A.Vs + (g < 0 ? 0 : g), g < 0 ? 0 : 8);
+        Step2Tile<P32, ORDER, TX, NT, 2, false>::template copy_async<8>(smem_addr(V + e), A.V + (g < 0 ? 0 : g), g < 0 ? 0 : 8);
+        Step2Tile<P32, ORDER, TX, NT, 2, false>::template copy_async<8>(smem_addr(Vs + e), A.Vs + (g < 0 ? 0 : g), g < 0 ? 0 : 8);
       });
   }
   __device__ __forceinline__ static uint32_t smem_addr(const void* p) {
@@ -120,7 +120,7 @@ struct Step2xTile {
   }
   __device__ __forceinline__ void load() {
     rows([&](int e, int64_t g) {
-      Step2Tile<P32, ORDER, TX, NT, 2>::template copy_async<16>(smem_addr(P + e), A.in + (g < 0 ? 0 : g), g < 0 ? 0 : 16);
+      Step2Tile<P32, ORDER, TX, NT, 2, false>::template copy_async<16>(smem_addr(P + e), A.in + (g < 0 ? 0 : g), g < 0 ? 0 : 16);
     });
     const unsigned int E = *(volatile const unsigned int*)(A.expo + A.turn);   // after grid_wait()
     F = (E > 0u && E < 2047u ? 1077 - int(E) : A.F0) + A.fix_offset;

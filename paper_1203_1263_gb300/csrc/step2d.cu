@@ -4,10 +4,10 @@
 
 namespace nlse {
 
-template <class T, int ORDER, int TX, int NT, int RY, int MINB>
+template <class T, int ORDER, int TX, int NT, int RY, int MINB, bool WRAP>
 __global__ void __launch_bounds__(NT, MINB) k_step2d(const __grid_constant__ Step2Args<T> A, int ty, int ntx) {
   extern __shared__ __align__(16) unsigned char step2_smem[];
-  Step2Tile<T, ORDER, TX, NT, RY> tile(A, ty, blockIdx.x % ntx, blockIdx.x / ntx, step2_smem);
+  Step2Tile<T, ORDER, TX, NT, RY, WRAP> tile(A, ty, blockIdx.x % ntx, blockIdx.x / ntx, step2_smem);
   // may start while the step before still runs: V is not its output, Psi^n is
   tile.load_potential();
   grid_wait();
@@ -55,17 +55,25 @@ int plan(const Shape& s, int ny, int nx, bool periodic, bool with_v) {
   return ty_best;
 }
 
-template <class T, int ORDER, int CFG>
-cudaError_t launch_shape(const Step2Args<T>& A, int ty, bool early, cudaStream_t stream) {
+// WRAP: a periodic grid's kernel (its wrapped loads cost the others 5 % in one kernel for both: 1000^2 FP32, MSD, central
+// differences 16.9 against 16.1 us per step).
+template <class T, int ORDER, int CFG, bool WRAP>
+cudaError_t launch_wrap(const Step2Args<T>& A, int ty, bool early, cudaStream_t stream) {
   constexpr Shape s = kShapes[CFG];
   const size_t smem = step2_smem<s.tx>(ty, A.V != nullptr);
-  auto kern = k_step2d<T, ORDER, s.tx, s.nt, s.ry, s.per_sm>;
+  auto kern = k_step2d<T, ORDER, s.tx, s.nt, s.ry, s.per_sm, WRAP>;
   static SmemLimit limit;
   const cudaError_t e = limit.allow(kern, 227 * 1024);
   if (e != cudaSuccess) return e;
   int ntx, nty;
-  step2_tiles(A.n[0], A.n[1], A.bc == BC_PERIODIC, s.tx, ty, &ntx, &nty);
+  step2_tiles(A.n[0], A.n[1], WRAP, s.tx, ty, &ntx, &nty);
   return launch_early(early, kern, dim3((unsigned)(ntx * nty)), dim3(s.nt), smem, stream, A, ty, ntx);
+}
+
+template <class T, int ORDER, int CFG>
+cudaError_t launch_shape(const Step2Args<T>& A, int ty, bool early, cudaStream_t stream) {
+  return A.bc == BC_PERIODIC ? launch_wrap<T, ORDER, CFG, true>(A, ty, early, stream)
+                             : launch_wrap<T, ORDER, CFG, false>(A, ty, early, stream);
 }
 
 template <class T, int ORDER>
