@@ -757,6 +757,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_conv_tc(const TcArgs a, const
     if (lane == 0) {
       const uint32_t idesc = idesc_bf16(128, nout);
       const uint32_t sm_base = smem_u32(tc_smem);
+      const bool whole = a.slices > 1;   // all four slices (LAYOUT 1: 64 channels), or the first alone
       int i = 0;
       for (int64_t tile = blockIdx.x; tile < T; tile += gridDim.x, ++i) {
         const int st = i & 1, k = i >> 1;
@@ -771,10 +772,11 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_conv_tc(const TcArgs a, const
             // one descriptor per tap; the K slices step the 16-byte start-address field by 2 (32 bytes)
             const uint64_t ad0 = sdesc_sw128(a0 + (uint32_t)(((1 + sy) * RW + d + sx * d) * 128));
             const uint64_t bd0 = sdesc_sw128(sm_base + (uint32_t)(t * nout * 128));
+            tc_mma(tmem + (uint32_t)(st * nout), ad0, bd0, idesc, t != 0);
+            if (whole) {
 #pragma unroll
-            for (int kk = 0; kk < 4; ++kk)
-              if (kk < a.slices)
-                tc_mma(tmem + (uint32_t)(st * nout), ad0 + 2u * kk, bd0 + 2u * kk, idesc, (t | kk) != 0);
+              for (int kk = 1; kk < 4; ++kk) tc_mma(tmem + (uint32_t)(st * nout), ad0 + 2u * kk, bd0 + 2u * kk, idesc, true);
+            }
           } else {
             const uint32_t aoff = a0 + (uint32_t)(((1 + sy) * RW + d + sx * d) * 16);
             const uint32_t boff = sm_base + (uint32_t)(t * planes * nout * 16);
