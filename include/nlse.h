@@ -118,9 +118,12 @@ int nlse_refresh_potential(nlse_t ctx);
 int nlse_step(nlse_t ctx, int64_t nsteps, double dt);
 
 /*
- * Mass  M = h^d sum_{all sites} |Psi|^2, in FP64 with compensated
- * (Neumaier) summation and a deterministic two-pass reduction.  Synchronises
- * the stream.  Returns NLSE_ENONFINITE if Psi holds a NaN or Inf.
+ * Mass  M = h^d sum_{all sites} |Psi|^2: the FP64 terms are added in 128-bit
+ * integers (what is left out stays below 2^-94 of the largest term per
+ * addition), in an order that never depends on scheduling, and rounded once
+ * per block and once at the end.  Synchronises the stream.  Returns
+ * NLSE_ENONFINITE if Psi holds a NaN or Inf; finite terms whose sum is beyond
+ * FP64 give a non-finite value.
  */
 int nlse_mass(nlse_t ctx, double *out_host);
 
@@ -179,10 +182,14 @@ const char *nlse_last_error(void);
  * Default: 2 for NLSE_C128 and 1 otherwise, except on grids small enough
  * that a step is bound by latency rather than by throughput: 3D grids of at
  * most 2^15 sites (NLSE_C128) or 2^17 sites (the FP32 forms) take 0,
- * and NLSE_C128 1D lines take 1 up to 2500 sites, 0 up to 2^15 sites and 3 beyond (the plain FP64
- * stencil's instruction chain is shorter than the exact-sum stencil's
- * conversions).  Where 0 is such a line's default rather than the caller's
- * choice, its steps run several per launch as with 1 (the same arithmetic).
+ * NLSE_C128 planes of at most 80,000 sites that 2 does not run in one launch
+ * per step (long or narrow ones, 274^2 to 282^2, periodic ones of three or
+ * four rows) take 1, or 0 with 8 to 128 sites along the shorter side,
+ * and NLSE_C128 1D lines take 1 up to 2500 sites, 0 up to 2^15 sites and 3
+ * beyond (the plain FP64 stencil's instruction chain is shorter than the
+ * exact-sum stencil's conversions).  Where 0 is such a line's default rather
+ * than the caller's choice, its steps run several per launch as with 1 (the
+ * same arithmetic), up to the lengths where that is the faster form.
  * The exact-sum stencil's fixed-point scale follows the state: before every
  * step it is taken from the largest component of Psi (below 1.6 2^54 in fixed
  * point, 1.25x or more below the accepted range, so the largest components
@@ -190,8 +197,8 @@ const char *nlse_last_error(void);
  * over Psi (the caller may have written it) and after each step from the
  * values the step wrote; a site whose operand is still out of range (a
  * stage state that far above the step's largest component) takes the FP64
- * stencil.  The resolution is thus 2^-54 or finer relative to max|Psi| for
- * any state, and results never depend on how steps are split into calls.
+ * stencil.  The resolution is thus 1.25 2^-54 or finer relative to the
+ * largest component for any state, and results never depend on how steps are split into calls.
  *   4 = NLSE_C64 on 3D grids: two RK4 stages per pass (stages 1+2 and 3+4,
  *       temporal blocking): the first stage's result for a tile plus a
  *       two-cell halo stays on chip and feeds the second stage, so the

@@ -140,9 +140,11 @@ namespace {
 
 // Tile shape in use: the caller's choice, else the measured default per form
 // and size (nlse_autotune can refine it): 32x8 for FP64; for the FP32 forms
-// in 3D, 64x8 on planes of at least 8192 sites (fewer, wider TMA boxes; 100^3:
-// 65.7 against 68.5 us per step, 128^3: 88.3 against 92.1) and 32x8 on smaller
-// planes (enough CTAs to fill the SMs; 64^3: 41.8 against 43.3); 32x16 in 2D.
+// in 3D, where the tiles serve them (above 3,000,000 sites, and periodic grids),
+// 64x8 on planes of at least 8192 sites (fewer, wider TMA boxes; FP32 512x256x256
+// 953 against 996 us per step with 32x8, periodic 128^3 70.2 against 72.8) and
+// 32x8 on smaller planes (enough CTAs to fill the SMs; periodic 80^3 37.8 against
+// 41.0, 88^3 41.5 against 46.9); 32x16 in 2D (F of large periodic planes).
 int resolved_tile(const nlse_ctx* c) {
   if (c->tile_cfg >= 0) return c->tile_cfg;
   if (c->dtype == NLSE_C128) return 0;
@@ -658,7 +660,8 @@ int nlse_create(nlse_t* out, int dims, const int64_t* N, double h, double a, dou
   // FP64 takes the exact-sum stencil on the tiled kernels, except where the grid is so small that a
   // step is bound by latency, not by the FP64 pipe's throughput, and the plain FP64 stencil's shorter
   // instruction chain wins: 3D grids of at most 2^15 sites (per-site kernels; 21^3: 21.8 against
-  // 94.1 for the tiled exact-sum kernel, 32^3: 38.8 against 93.6) and 1D lines up to 2^15 sites, which run
+  // 94.1 for the tiled exact-sum kernel, 32^3: 38.8 against 93.6; by time alone the line would lie higher, 46^3 74
+  // against 85, 64^3 162 against 92, but moving it changes the arithmetic of the grids between) and 1D lines up to 2^15 sites, which run
   // several steps per launch (2001 sites: 8.6 with MSD walls against 19.2 for a launch per stage and 23.8
   // with the exact-sum stencil on a cluster; 32,000: 18.6 against 24.4 for the exact-sum stencil one thread
   // per site; 49,000: 23.5 against 25.7).

@@ -7,7 +7,7 @@
 // items, the largest runs first.  A CTA takes one item through all four stages
 // with the single runs' code, so results are bit-for-bit those of integrating
 // each run alone.  Psi alternates between the caller's array and a copy in the
-// workspace.  96 runs of 64^2 to 1024^2 (3.5e7 sites): 0.587 ms per step, 60
+// workspace.  96 runs of 64^2 to 1024^2 (3.5e7 sites): 0.590 ms per step, 60
 // Gsite-step/s; a deep and a wall-shell kernel per stage, with K_tot, Psi_tmp
 // and Psi_out through memory (148 bytes per site and step), took 1.55 ms.
 #include <cuda_runtime.h>
@@ -138,7 +138,7 @@ bool layout_batch(int nruns, const nlse_run_desc* runs, int shape, BatchLayout* 
   L->field_off.resize(nruns);
   for (int r = 0; r < nruns; ++r) {
     L->field_off[r] = off;
-    // a run's share is at least two arrays, as callers may rely on; the copy takes the first
+    // a run's share is two arrays, the least that the ABI's test holds callers to; the copy takes the first
     off = al(off + 2 * sizeof(float2) * size_t(runs[r].n[0] * runs[r].n[1]));
   }
   L->total = al(off);

@@ -54,7 +54,7 @@ struct L64 { using R = double; using C = double2; using VR = OnChip<double>; usi
 struct L32 { using R = float;  using C = float2;  using VR = OnChip<float>;  using M = float2;  };
 
 // float <-> double on the integer pipe (GB300 issues FP64-pipe instructions,
-// conversions included, at 1/75 of the FP32 rate).  Both follow IEEE-754:
+// conversions included, at 1/64 of the FP32 rate).  Both follow IEEE-754:
 // widening is exact, narrowing rounds to nearest even; zeros, subnormals,
 // infinities and NaN take the hardware conversion.
 __device__ __forceinline__ double f2d_exact(float v) {
@@ -254,7 +254,7 @@ __device__ __forceinline__ typename V2<typename T::R>::t a_lap(const Field<T>& f
 
 // ---------------------------------------------------------------------------
 // Exact-sum stencil for the FP64 path.  GB300 issues FP64 arithmetic at
-// 1/75 of the FP32 rate, so the FP64 stage is bound by the FP64 pipe, and
+// 1/64 of the FP32 rate, so the FP64 stage is bound by the FP64 pipe, and
 // most of its FP64 instructions are the stencil's additions.  Here every
 // stencil operand is converted (on the integer pipe, from its IEEE-754 bits)
 // to a 64-bit fixed-point number v * 2^F rounded to nearest; the sums
@@ -305,8 +305,9 @@ __device__ __forceinline__ unsigned int expo_bits(float v) { return 0u; }
 
 // What the fixed-point scale follows: the biased exponent of |v|, one more from 1.6 times its power of two on, 2047
 // or more for Inf / NaN.  With F = 1077 - (the largest of the state) the largest component lies in
-// [0.8, 1.6) 2^54: 53 bits kept for every component down to a quarter of it, and a factor of 1.25 at least up to
-// the accepted range for the stages' intermediate states (beyond, a site takes the FP64 stencil).
+// [0.8, 1.6) 2^54: all 53 bits kept of every component of at least 2^52 in fixed point (5/16 of the largest or less),
+// and a factor of 1.25 at least up to the accepted range for the stages' intermediate states (beyond, a site takes the
+// FP64 stencil).
 __device__ __forceinline__ unsigned int range_bits(double v) {
   return (unsigned int)((__double2hiint(v) & 0x7FFFFFFF) + 0x66667) >> 20;
 }
@@ -340,8 +341,8 @@ __device__ __forceinline__ int fix_low(double v, int F) {
 }
 
 // The stencil sum of what rounding its operands left out, on small planes (Field::fine): there the FP64 stencil's
-// error is the measure (256^2, 32 steps, against 64 bits: 3.5e-16; the plain fixed-point sum 6.3e-16, with this
-// 3.5e-16).  All operands or none: the errors of a smooth field's neighbours cancel in the sum.
+// error is the measure (256^2 window, 32 steps, against 64 bits: 3.6e-16; the plain fixed-point sum 6.3e-16, with this
+// 3.6e-16; before the scale followed 1.6 times a power of two the plain sum had 1.6e-15).  All operands or none: the errors of a smooth field's neighbours cancel in the sum.
 template <class T, int D, int ORDER, class Acc>
 __device__ __forceinline__ longlong2 fix_correction(const Acc& acc, double2 pc, int F) {
   int x = (ORDER == 4 ? -30 : -2) * D * fix_low(pc.x, F), y = (ORDER == 4 ? -30 : -2) * D * fix_low(pc.y, F);

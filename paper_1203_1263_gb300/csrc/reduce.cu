@@ -9,7 +9,7 @@
 // The energy's Laplacian is summed in 64-bit fixed point too, at a scale taken
 // from the site's own operands, one per component; the sites next to a wall
 // take the FP64 form, enumerated apart so that whole warps take it.  256^3 FP64
-// state with V, mass and energy together: 649 us; with FP64 sums throughout
+// state with V, mass and energy together: 655 us; with FP64 sums throughout
 // (about 10 and 70 FP64 instructions per site) 3,180.  What bounds them now: the
 // mass the FP64 pipe (79 % busy with the two instructions a site's |Psi|^2
 // takes), the energy the FP64 pipe and the issue of the 26 conversions per site

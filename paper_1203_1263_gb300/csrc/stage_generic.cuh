@@ -1,6 +1,7 @@
 // Per-site kernels that read through the read-only cache: one thread per
-// interior site (1D lines; planes and grids take stage_split.cuh), the periodic
-// grids' sites and shells, and the enumeration of the sites next to the walls.
+// interior site (1D lines; planes and grids where the walls do not pay as
+// threads of their own, see stage_split.cuh), the periodic grids' sites and
+// shells, and the enumeration of the sites next to the walls.
 #pragma once
 #include "nlse_device.cuh"
 

@@ -12,7 +12,7 @@
 // and the issue slots are each 42 % busy, the rest is barriers at the end of a
 // stage), not memory: 20 bytes per site and step.  Measured, us per step, four
 // launches per stage pass before and now: 1000^2 FP32, central differences,
-// MSD, 30.6 and 16.3; on small grids the launches and the four stages' latency
+// MSD, 30.6 and 15.8; on small grids the launches and the four stages' latency
 // remain (100^2: 6.9).
 // Psi^{n+1} goes to another buffer than Psi^n, because neighbouring tiles
 // still read Psi^n.
