@@ -661,10 +661,10 @@ int nlse_create(nlse_t* out, int dims, const int64_t* N, double h, double a, dou
   // step is bound by latency, not by the FP64 pipe's throughput, and the plain FP64 stencil's shorter
   // instruction chain wins: 3D grids of at most 2^15 sites (per-site kernels; 21^3: 21.8 against
   // 94.1 for the tiled exact-sum kernel, 32^3: 38.8 against 93.6; by time alone the line would lie higher, 46^3 74
-  // against 85, 64^3 162 against 92, but moving it changes the arithmetic of the grids between) and 1D lines up to 2^15 sites, which run
-  // several steps per launch (2001 sites: 8.6 with MSD walls against 19.2 for a launch per stage and 23.8
-  // with the exact-sum stencil on a cluster; 32,000: 18.6 against 24.4 for the exact-sum stencil one thread
-  // per site; 49,000: 23.5 against 25.7).
+  // against 85, 64^3 162 against 92, but moving it changes the arithmetic of the grids between) and 1D lines up to
+  // 2^15 sites, several steps per launch where that is the faster form (lines_path; 2001 sites: 8.6 with MSD walls
+  // against 19.2 for a launch per stage and 23.8 with the exact-sum stencil on a cluster; 32,000: 18.6 against 24.4
+  // for the exact-sum stencil one thread per site; 49,000: 23.5 against 25.7).
   // FP64 planes take the exact-sum stencil where a whole step is one launch (step2x_fits) and above 80,000 sites
   // (316^2: 61.1 with the FP64 stencil, 54.0).  The planes between (274^2 to 282^2, and long or narrow ones) take the
   // FP64 stencil: where the operands' rounding is not taken back (Field::fine) its error is the smaller one (32 steps,
@@ -975,7 +975,9 @@ int nlse_autotune(nlse_t c, int* best_tile_cfg, float* best_ms) {
     cudaEvent_t e0, e1;
     cudaEventCreate(&e0);
     cudaEventCreate(&e1);
-    const int saved = c->tile_cfg, only = columns_path(c) ? resolved_tile(c) : -1;   // nothing to compare: the default
+    // the default where no launch of a step depends on the tile
+    const bool same = columns_path(c) || (c->d == 2 && c->dtype != NLSE_C128 && !step2_path(c));
+    const int saved = c->tile_cfg, only = same ? resolved_tile(c) : -1;
     best = 1e30f;
     cudaError_t e = cudaSuccess;
     if (c->dtype == NLSE_C64_ACC64)

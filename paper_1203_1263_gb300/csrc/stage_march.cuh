@@ -9,7 +9,7 @@
 // planes of its own column stay in registers, the eight in-plane neighbours are
 // L1 hits (their own columns' threads loaded them two planes ago), all loads
 // issued a plane ahead.  What bounds it is the latency of those loads (long
-// scoreboard, 41 % issue at four CTAs per SM); 173 instructions per site.  The sites
+// scoreboard, 48 % issue at four CTAs per SM); 173 instructions per site.  The sites
 // next to the walls and the boundary sites are further ranges of blocks, as in
 // stage_split.cuh.  The arithmetic is a_lap_body's and rk_apply's on packed FP32
 // pairs (stage_step2d.cuh) in the same order: bit-for-bit the other kernels'.

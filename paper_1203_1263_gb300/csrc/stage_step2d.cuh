@@ -9,7 +9,7 @@
 // from the one before in shared memory, and writes Psi^{n+1}.  What bounds it
 // is the shared-memory and issue rate of the stages (the halo costs a factor
 // 1.3-1.7 in evaluated sites; on a batch of uneven grids the shared-memory pipe
-// and the issue slots are each 42 % busy, the rest is barriers at the end of a
+// is 72 % busy and the issue slots 46 %, the rest is barriers at the end of a
 // stage), not memory: 20 bytes per site and step.  Measured, us per step, four
 // launches per stage pass before and now: 1000^2 FP32, central differences,
 // MSD, 30.6 and 15.8; on small grids the launches and the four stages' latency
