@@ -176,7 +176,10 @@ Field<T> make_field(const nlse_ctx* c, const void* in) {
   f.F = c->fixF;
   f.Fdev = (c->dtype == NLSE_C128) ? c->fdev() : nullptr;
   f.fine = c->d == 2 && step2x_fits(int(c->n[0]), int(c->n[1]), c->bc == NLSE_BC_PERIODIC);
-  f.cLF = ldexp(c->order == 4 ? c->a / (12.0 * c->h * c->h) : c->a / (c->h * c->h), -c->fixF);
+  const double cL = c->order == 4 ? c->a / (12.0 * c->h * c->h) : c->a / (c->h * c->h);
+  int ex = 0;
+  f.mL = 2.0 * frexp(cL, &ex);
+  f.cLF = f.fine ? ldexp(0.5, ex - c->fixF) : ldexp(cL, -c->fixF);
   f.invcLF = R(1.0 / f.cLF);
   f.sG = R(c->s / f.cLF);
   f.V = (const typename T::VR*)c->V;
@@ -451,6 +454,7 @@ cudaError_t launch_step2x_any(const nlse_ctx* c, double dt, cudaStream_t st, con
   A.n[1] = int(c->n[1]);
   A.cLF = f.cLF;
   A.invcLF = f.invcLF;
+  A.mL = f.mL;
   A.sG = f.sG;
   for (int i = 0; i < 4; ++i) A.dtc[i] = A.dtc[i] * f.cLF;
   A.Vs = c->V ? (const double*)c->at(c->lay.vs) : nullptr;

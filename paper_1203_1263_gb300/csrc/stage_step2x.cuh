@@ -5,7 +5,7 @@
 // thread per boundary site.  The tile holds every stage's input twice, in FP64
 // (the pointwise terms) and as the 64-bit fixed point that the stencil sums are
 // formed in, converted once where a stage produces it.  What bounds it is the
-// FP64 pipe, nine instructions per evaluated site and stage, of which the halo
+// FP64 pipe, eleven instructions per evaluated site and stage, of which the halo
 // adds 1.4-2.2 times; so it pays while a step is launches and latency, and the
 // stage-streaming kernels keep the larger grids (step2x_path in api.cu).
 //
@@ -20,7 +20,7 @@ namespace nlse {
 struct Step2xArgs {
   int n[2];
   int bc;
-  double s, h2_over_a, cL, tiny, cLF, invcLF, sG;   // as in Field
+  double s, h2_over_a, cL, tiny, cLF, invcLF, sG, mL;   // as in Field
   double dtc[4];               // dt/2, dt/2, dt, dt/6, times cLF
   const double *V, *Vs;        // V and V / cLF, or nullptr
   const double2* in;
@@ -159,6 +159,7 @@ struct Step2xTile {
     const longlong2 cc = x[e], xm = x[e - 1], xp = x[e + 1], ym = x[e - W], yp = x[e + W];
     bool bad = fbad(cc) | fbad(xm) | fbad(xp) | fbad(ym) | fbad(yp);
     long long sx = (yp.x + ym.x) + (xp.x + xm.x), sy = (yp.y + ym.y) + (xp.y + xm.y);
+    int rx, ry;
     const char2 lc = l[e], l0 = l[e - 1], l1 = l[e + 1], l2 = l[e - W], l3 = l[e + W];   // fix_correction
     if constexpr (ORDER == 4) {
       const longlong2 xm2 = x[e - 2], xp2 = x[e + 2], ym2 = x[e - 2 * W], yp2 = x[e + 2 * W];
@@ -166,16 +167,18 @@ struct Step2xTile {
       sx = 16 * sx - ((ym2.x + yp2.x) + (xm2.x + xp2.x)) - 60 * cc.x;
       sy = 16 * sy - ((ym2.y + yp2.y) + (xm2.y + xp2.y)) - 60 * cc.y;
       const char2 m0 = l[e - 2], m1 = l[e + 2], m2 = l[e - 2 * W], m3 = l[e + 2 * W];
-      sx += (16 * ((l0.x + l1.x) + (l2.x + l3.x)) - ((m0.x + m1.x) + (m2.x + m3.x)) - 60 * lc.x + 128) >> 8;
-      sy += (16 * ((l0.y + l1.y) + (l2.y + l3.y)) - ((m0.y + m1.y) + (m2.y + m3.y)) - 60 * lc.y + 128) >> 8;
+      rx = 16 * ((l0.x + l1.x) + (l2.x + l3.x)) - ((m0.x + m1.x) + (m2.x + m3.x)) - 60 * lc.x;
+      ry = 16 * ((l0.y + l1.y) + (l2.y + l3.y)) - ((m0.y + m1.y) + (m2.y + m3.y)) - 60 * lc.y;
     } else {
-      sx += -4 * cc.x + (((l0.x + l1.x) + (l2.x + l3.x) - 4 * lc.x + 128) >> 8);
-      sy += -4 * cc.y + (((l0.y + l1.y) + (l2.y + l3.y) - 4 * lc.y + 128) >> 8);
+      sx -= 4 * cc.x;
+      sy -= 4 * cc.y;
+      rx = (l0.x + l1.x) + (l2.x + l3.x) - 4 * lc.x;
+      ry = (l0.y + l1.y) + (l2.y + l3.y) - 4 * lc.y;
     }
     const double N = fma(A.sG, norm2(pc), -(with_v ? Vs[e] : 0.0));
     double2 aL;
     if (!bad) {
-      aL = {i2d_rn(sx, eadj), i2d_rn(sy, eadj)};
+      aL = {__dmul_rn(A.mL, i2d_low(sx, rx, eadj)), __dmul_rn(A.mL, i2d_low(sy, ry, eadj))};
     } else {   // an operand out of the fixed-point range: the FP64 stencil
       const Field<L64> f = field();
       TileAccX2<W> acc{d, x, e, F};
