@@ -347,7 +347,8 @@ __device__ __forceinline__ int fix_low(double v, int F) {
 // error is the measure (256^2 window, 32 steps, against 64 bits: 3.6e-16; the plain fixed-point sum 6.3e-16, with this
 // 3.6e-16; before the scale followed 1.6 times a power of two the plain sum had 1.6e-15).  Over 70 planes of 25 to 285
 // sites a side the ratio to the FP64 stencil's error is 0.92 to 1.08, 1.00 on the mean; with this rounded to whole units
-// before the sum's own rounding it was up to 1.17 (central differences), and with the unit cL * 2^-F up to 1.35.  All operands or none: the errors of a smooth field's neighbours cancel in the sum.
+// before the sum's own rounding it was up to 1.17 (central differences), and with the unit cL * 2^-F up to 1.35.  All
+// operands or none: the errors of a smooth field's neighbours cancel in the sum.
 template <class T, int D, int ORDER, class Acc>
 __device__ __forceinline__ longlong2 fix_correction(const Acc& acc, double2 pc, int F) {
   int x = (ORDER == 4 ? -30 : -2) * D * fix_low(pc.x, F), y = (ORDER == 4 ? -30 : -2) * D * fix_low(pc.y, F);

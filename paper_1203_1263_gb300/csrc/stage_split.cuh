@@ -123,9 +123,10 @@ __device__ __forceinline__ unsigned int boundary_site(const StageArgs<T>& A, int
 
 // Blocks [0, b1): the n1 deep sites; [b1, b2): the n2 shell sites; the rest: the n3 boundary sites.  Three CTAs per SM
 // for the exact sums on planes (at two, a little over two CTAs per SM take a whole wave more: 282^2 56.2 against 48.8 us
-// per step, 1000^2 243 and 191), two with the correction's operands (unbounded, 256^2 66.9 against 52.4).
+// per step, 1000^2 243 and 191), two with the correction's operands (unbounded, 256^2 66.9 against 52.4).  The others are
+// left to the compiler (0; a bound of one makes it take up to 26 registers more).
 template <class T, int D, int ORDER, bool EXACT, class I, bool FINE = false>
-__global__ void __launch_bounds__(256, EXACT && D == 2 ? (FINE ? 2 : 3) : 1)
+__global__ void __launch_bounds__(256, EXACT && D == 2 ? (FINE ? 2 : 3) : 0)
     k_stage_split(const StageArgs<T> A, unsigned b1, unsigned b2, int64_t n1, int64_t n2, int64_t n3) {
   using R = typename T::R;
   using C2 = typename V2<R>::t;
