@@ -134,10 +134,10 @@ inline bool march_ok(const int* n, int bc) {
 
 // Flat grids that are mostly MSD walls: with a thread per boundary site (walls_apart) they are slower than the tiles
 // with a thread per wall site (2SHOC, this form and that: 6x600x700 142 and 131, 700x6x700 198 and 173; 6x300x300 38
-// and 43, 700x700x6 410 and 470).
+// and 43, 700x700x6 410 and 470; central differences with V 6x500x1000 126 and 119, without 6x600x700 86 and 97).
 template <int ORDER, class T>
 inline bool march_thin(const Field<T>& f) {
-  return ORDER == 4 && f.bc == BC_MSD && (f.n[0] < 8 || f.n[1] < 8) && boundary_count(3, f.n, f.m) > 500000;
+  return f.bc == BC_MSD && (f.n[0] < 8 || f.n[1] < 8) && boundary_count(3, f.n, f.m) > (ORDER == 4 ? 500000 : 900000);
 }
 
 // Whether the steps of a grid take the columns: a few million sites, or rows that TMA cannot take (the figures above).
