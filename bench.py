@@ -69,9 +69,9 @@ LAUNCHES_PER_STEP = {"c128": 17, "c64": 16, "c64_acc64": 16}
 # ncu capture (profiles/rk4_step_256x256x512_traffic_and_launches.md), with the hash of the 3D stage
 # path's sources it was taken at: the figure is reported only while csrc_hash() still matches.
 TRAFFIC_PER_STEP = {  # dtype -> (bytes per step, csrc hash of the capture)
-    "c128": (10879.3e6, "2e6b77f10862c6a4"),
-    "c64": (5534.8e6, "2e6b77f10862c6a4"),
-    "c64_acc64": (6315.9e6, "2e6b77f10862c6a4"),
+    "c128": (10878.0e6, "239a3445c3d39942"),
+    "c64": (5536.6e6, "239a3445c3d39942"),
+    "c64_acc64": (6316.6e6, "239a3445c3d39942"),
 }
 
 # The sources the 3D stage path (deep kernels, wall slabs, scale update, step loop) is built from.
