@@ -173,7 +173,7 @@ const char *nlse_last_error(void);
  *   2 = tiled kernel with the exact-sum stencil (NLSE_C128 only; other
  *       dtypes treat it as 1): the Laplacian's stencil sums are formed exactly
  *       in 64-bit fixed point on the integer pipe and converted to FP64 once;
- *       2D grids of up to about 280 x 280 run a tile's four stages in one
+ *       2D grids of up to about 273 x 273 run a tile's four stages in one
  *       launch per step; on 1D lines of up to ~49,000 sites one thread-block cluster of up to 16
  *       CTAs keeps the line in shared memory and runs every step of an
  *       nlse_step call in one launch,

@@ -35,8 +35,8 @@ cudaError_t launch_order(const Step2xArgs& A, int ty, int ntx, int n, bool early
 
 }  // namespace
 
-// One wave of 16-row tiles (about 280 x 280): beyond, the halo's FP64 work costs more than the stage kernels'
-// launches (us per step, Dirichlet 2SHOC: 256^2 21.3 against 52.8; 450^2 55 against 48, periodic 54 against 37).
+// One wave of 16-row tiles (up to 273 x 273): beyond, the halo's FP64 work costs more than the stage kernels'
+// launches (us per step, Dirichlet 2SHOC: 256^2 24.0 against 47.5; 450^2 55 against 48, periodic 54 against 37).
 bool step2x_fits(int ny, int nx, bool periodic) {
   int ntx;
   return (int64_t)ny * nx < (int64_t(1) << 20) && tiles(ny, nx, periodic, 16, &ntx) <= kPerSm * 152;
